@@ -213,6 +213,7 @@ size_t carve(sph_ctx* c, void* base, uint32_t n, const Table& t, int passes) {
         c->val[b] = cv.take<uint32_t>(n);
     }
     c->posc = cv.take<float4>(n);
+    c->posu = cv.take<float4>(n);
     c->ace = cv.take<float4>(n);
     c->stage_pos = cv.take<double>(3 * (size_t)n);
     c->stage_vr = cv.take<float>(4 * (size_t)n);
@@ -384,6 +385,7 @@ void rebuild_after_keys(sph_ctx* c, bool with_pre) {
         ra.dpvr = c->pvr[1];
     }
     ra.posc = c->posc;
+    ra.posu = c->posu;
     ra.hist_to_zero = c->hist;
     ra.status = c->status;
     launch_reorder(c->d, ra, st);
@@ -397,6 +399,7 @@ void enqueue_interact(sph_ctx* c, bool counts, bool set_dt) {
     ia.n_units = c->uoff + c->tab.nrows;
     ia.status = c->status;
     ia.posc = c->posc;
+    ia.posu = c->posu;
     ia.velrhop = c->vr[c->cur];
     ia.key = c->key[c->skey];
     ia.id = c->id[c->cur];
@@ -1133,6 +1136,7 @@ int sph_autotune(sph_ctx* c, uint32_t reps, float* ms_per_variant, uint32_t* bes
         ia.n_units = c->uoff + c->tab.nrows;
         ia.status = c->status;
         ia.posc = c->posc;
+        ia.posu = c->posu;
         ia.velrhop = c->vr[c->cur];
         ia.key = c->key[c->skey];
         ia.id = c->id[c->cur];

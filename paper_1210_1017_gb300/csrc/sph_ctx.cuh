@@ -40,7 +40,7 @@ struct sph_ctx {
     // mid-step reorder (read by the corrector)
     double *px[2], *py[2], *pz[2];
     float4* pvr[2];
-    float4 *posc, *ace;
+    float4 *posc, *posu, *ace;   // posu: posc with x in fixed point (k_reorder)
     double* stage_pos;       // host transfer staging: 3n doubles
     float* stage_vr;         // 4n floats (velocity, then density)
     uint32_t *key[2], *val[2];

@@ -169,6 +169,7 @@ struct ReorderArgs {
     double *dpx, *dpy, *dpz;
     float4* dpvr;
     float4* posc;
+    float4* posu;                    // posc with x in fixed point along the row
     uint32_t* hist_to_zero;          // cleared for the next rebuild
     uint32_t* status;
 };
@@ -196,6 +197,7 @@ struct InteractArgs {
     const uint32_t* n_units;
     uint32_t* status;
     const float4* posc;
+    const float4* posu;   // x in fixed point (cells of 2^26, modulo 2^32), y, z, P
     const float4* velrhop;
     const uint32_t* key;
     const uint32_t* id;
@@ -211,6 +213,19 @@ struct InteractArgs {
     ReduceArgs red;
     int set_dt;
 };
+// One interaction shape.
+struct Variant {
+    int warps;              // warps of particles (the unit is warps x 32 particles)
+    int split;              // warps per group of 32 particles
+    int stage;              // staged candidates
+    // [kernel: Wendland C2, cubic spline][with counts]
+    void (*fn[2][2])(const Dev, const InteractArgs);
+    size_t smem;
+    int grid;               // persistent grid on this GPU (set by prepare_interact)
+    int max_per_sm;         // resident blocks that the TMEM columns allow (0: any)
+};
+// The shapes whose candidate test runs on the tensor cores (sph_interact_tc.cu).
+Variant tc_variant_n(int k);
 uint32_t max_units(uint32_t n, uint32_t nrows, uint64_t ncells);   // bound on units
 int variant_unit(int variant);               // particles per unit of a variant
 int variant_stage(int variant);              // staged candidates of a variant

@@ -12,36 +12,11 @@
 #include <mutex>
 
 #include "sph_internal.cuh"
+#include "sph_pair.cuh"
 
 namespace sph {
 
 namespace {
-
-constexpr uint32_t kFull = 0xffffffffu;
-
-__device__ __forceinline__ float sqrt_approx(float x) {
-    float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// Index q with base[q] <= v < base[q + 1] (base has n + 1 ascending entries).
-__device__ __forceinline__ uint32_t find_instance(const uint32_t* __restrict__ base, uint32_t n,
-                                                  uint32_t v) {
-    uint32_t lo = 0, hi = n;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (__ldg(base + mid) <= v) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
 
 // Sec. 3.1 cell label: floor((x - x0) * (1/(2h))) per axis in FP64, each
 // operation rounded as written; label = cell_base + cx + ncx (cy + ncy cz)
@@ -192,6 +167,7 @@ __global__ void __launch_bounds__(256) k_reorder(const Dev d, const ReorderArgs 
     }
     if (a.spvr) a.dpvr[dst] = a.spvr[v];
     float4 pc = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t xu = 0;
     if (c < d.ncells) {
         const Inst& I = d.inst[find_instance(d.cell_base, d.n_inst, c)];
         const uint32_t lc = c - I.cell_base;
@@ -203,14 +179,13 @@ __global__ void __launch_bounds__(256) k_reorder(const Dev d, const ReorderArgs 
         pc.y = __double2float_rn(y - (I.y0 + (double)cy * d.cs));
         pc.z = __double2float_rn(z - (I.z0 + (double)cz * d.cs));
         pc.w = p_over_rho2(d, I.B, vr.w);
+        xu = (cx << 26) + (uint32_t)__float2int_rn(pc.x * (67108864.0f / d.csf));
     }
     a.posc[dst] = pc;
+    a.posu[dst] = make_float4(__uint_as_float(xu), pc.y, pc.z, pc.w);
 }
 
 // ----------------------------------------------------------- interaction --
-
-constexpr uint32_t kIdxMask = (1u << 26) - 1;
-constexpr uint32_t kWaitLimit = 1u << 22;
 
 // Shape of one interaction variant: W warps per block (units of W*32
 // particles), STAGE staged candidates, WCAP hit-mask words per lane.  Dynamic
@@ -235,53 +210,6 @@ struct Shape {
     static_assert(fb_cap >= 16 && (size_t)W * fb_cap * 32 * sizeof(uint32_t) <= stage_bytes,
                   "fallback lists must fit in the staging area");
     static_assert(STAGE <= (1 << 16) && STAGE % 2 == 0, "staged index must fit 16 bits");
-};
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-
-// 1-D bulk copy global -> shared (TMA engine), completion counted on bar.
-// Both addresses 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-            "r"(smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for phase `parity` of bar; false if it gave up.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
-    for (uint32_t k = 0; k < kWaitLimit; ++k)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
-struct PairAcc {
-    float ax, ay, az, dr, mu;
-    float npf;       // pairs counted by the FP32 test (exact below 2^24)
-    uint32_t np;
 };
 
 // The sign bits (15 and 31) of a and of b, each spread over one byte of the
@@ -310,203 +238,6 @@ constexpr KeepTable make_keep_table() {
 }
 __constant__ KeepTable c_keep = make_keep_table();
 
-// Pair terms of Eqs. 7 and 9 for i (pi, vi) and j (pj, vj) at offset
-// (dx, dy, dz) = r_i - r_j.  MOM: evaluate the momentum terms (a warp-uniform
-// choice).  They are accumulated for every particle; the caller keeps them
-// only for fluid particles, since boundary particles never move (Sec. 2.3).
-// A pair with v_ij = 0 whose offset lies outside the support (the particle
-// itself, placed 4 cells away) contributes exactly nothing and is not
-// counted, which lets lane work be padded with it.  Masks are products with
-// 0 or 1 rather than selects, keeping the integer/logic pipe free.
-// KERN: 0 Wendland C2, 1 cubic spline (Sec. 2.2).
-template <int KERN, bool MOM, bool CHECK = false>
-__device__ __forceinline__ void pair_terms(const Dev& d, float c0, const float4& pi,
-                                           const float4& vi, float ci, float dx, float dy, float dz,
-                                           const float4& pj, const float4& vj, PairAcc& s) {
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    // CHECK: the entry came from the conservative half-precision pre-filter;
-    // the FP32 neighbour test (the same predicate as the candidate test of the
-    // global-memory path) decides and counts the pair: use = [d2 < (2h)^2],
-    // the saturated sign of 2^100 ((2h)^2 - d2), exact (power-of-two scaling)
-    const float use = CHECK ? __saturatef(fmaf(d2, -0x1p100f, d.r2max * 0x1p100f)) : 1.f;
-    if (CHECK) s.npf += use;
-    // grad_i W = F r_ij.  Wendland C2: F = -5 aD/h^2 (1 - q/2)^3.  Cubic
-    // spline: F = aD/h^2 (9/4 q - 3) for q < 1, -3/4 aD/h^2 (2 - q)^2 / q
-    // for 1 <= q < 2 (a select: the outer piece is infinite at q = 0).
-    const float q = sqrt_approx(d2) * d.inv_h;
-    float shape;
-    if (KERN == 1) {
-        const float wo = 2.0f - q;
-        const float outer = -0.75f * (wo * wo) * rcp_approx(q);
-        const float inner = fmaf(2.25f, q, -3.0f);
-        shape = q < 1.0f ? inner : outer;
-    } else {
-        const float wq = fmaf(-0.5f, q, 1.0f);
-        shape = wq * wq * wq;
-    }
-    const float F = CHECK ? d.fc * shape * use : d.fc * shape;
-    const float dvx = vi.x - vj.x, dvy = vi.y - vj.y, dvz = vi.z - vj.z;
-    const float vr = fmaf(dvx, dx, fmaf(dvy, dy, dvz * dz));
-    s.dr = fmaf(vr, F, s.dr);                                      // Eq. 7
-    if (MOM) {
-        const float nu = d.h * vr * rcp_approx(d2 + d.eta2);       // Sec. 2.2
-        const float rrj = vj.w * d.inv_rho0;
-        const float cj = c0 * rrj * rrj * rrj;
-        // Pi_ij only for approaching pairs (v_ij . r_ij < 0, the sign of nu)
-        const float visc = -d.alpha * (ci + cj) * fminf(nu, 0.f) * rcp_approx(vi.w + vj.w);
-        const float f = (pi.w + pj.w + visc) * F;                  // Eq. 9
-        s.ax = fmaf(-f, dx, s.ax);
-        s.ay = fmaf(-f, dy, s.ay);
-        s.az = fmaf(-f, dz, s.az);
-        s.mu = fmaxf(s.mu, CHECK ? fabsf(nu) * use : fabsf(nu));
-    }
-}
-
-// Sec. 3.3 reductions, by one block once every interaction block has
-// published its counters (pairs, candidates, status bits) and atomically
-// raised the per-instance maxima: the counters are summed (integer sums and
-// maxima do not depend on the order), then per instance
-//   dt = CFL min( sqrt(h / max|a|), h / (max c + max mu) )
-// (0 for instances that are done), and the maxima are cleared for the next
-// evaluation.  Loads bypass L1 (the partials may come from the same kernel).
-// Run by a block of at most 256 threads (an interaction block).
-__device__ void reduce_counters_and_dt(const Dev& d, const ReduceArgs& a, int set_dt) {
-    __shared__ unsigned long long s_u[8][3];
-    __shared__ uint32_t s_b[8];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    unsigned long long pf = 0, pb = 0, nc = 0;
-    uint32_t bad = 0;
-    for (uint32_t i = threadIdx.x; i < a.nparts; i += blockDim.x) {
-        const uint4 u = __ldcg(a.part_u + i);
-        pf += u.x;
-        nc += u.y;
-        bad |= u.z;
-        pb += u.w;
-    }
-    for (int o = 16; o; o >>= 1) {
-        pf += __shfl_xor_sync(kFull, pf, o);
-        pb += __shfl_xor_sync(kFull, pb, o);
-        nc += __shfl_xor_sync(kFull, nc, o);
-        bad |= __shfl_xor_sync(kFull, bad, o);
-    }
-    if (lane == 0) {
-        s_u[w][0] = pf;
-        s_u[w][1] = pb;
-        s_u[w][2] = nc;
-        s_b[w] = bad;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long qf = 0, qb = 0, qc = 0;
-        uint32_t bb = 0;
-        for (int k = 0; k < nw; ++k) {
-            qf += s_u[k][0];
-            qb += s_u[k][1];
-            qc += s_u[k][2];
-            bb |= s_b[k];
-        }
-        a.counters[0] += qf + qb;
-        a.counters[1] += qc;
-        a.counters[2] = qf + qb;
-        a.counters[3] = qc;
-        a.counters[4] = qf;
-        a.counters[5] = qb;
-        a.counters[6] += qf;
-        a.counters[7] += qb;
-        if (bb) atomicOr(a.status, bb);
-    }
-    for (uint32_t q = threadIdx.x; q < d.n_inst; q += blockDim.x) {
-        uint32_t* tm = d.is.terms + 3 * q;
-        const float fa = __uint_as_float(__ldcg(tm + 0));
-        const float fc = __uint_as_float(__ldcg(tm + 1));
-        const float fm = __uint_as_float(__ldcg(tm + 2));
-        const double amax = sqrt((double)fa);
-        if (set_dt) {
-            double dt = 0.0;
-            if (!d.is.done[q]) {
-                if (d.dt_fixed > 0.0) {
-                    dt = d.dt_fixed;
-                } else {
-                    const double dtf = amax > 0.0 ? sqrt(d.h_d / amax) : INFINITY;
-                    const double dtc = d.h_d / ((double)fc + (double)fm);
-                    dt = d.cfl * (dtf < dtc ? dtf : dtc);
-                }
-            }
-            d.is.dt[q] = dt;
-            d.is.last[3 * q + 0] = (float)amax;
-            d.is.last[3 * q + 1] = fc;
-            d.is.last[3 * q + 2] = fm;
-        }
-        tm[0] = 0u;
-        tm[1] = 0u;
-        tm[2] = 0u;
-    }
-}
-
-// Packed accumulators of two pair streams (the two pairs a lane evaluates
-// per step of the pair phase), one in each half of a float2.  The momentum
-// sums hold +sum f r_ij (the caller negates once at the end; negation is
-// exact, so this equals summing the negated terms).
-struct PairAcc2 {
-    float2 ax, ay, az, dr, npf;
-    float mu;
-};
-
-__device__ __forceinline__ float2 ff2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
-
-// pair_terms<KERN, true, true> for two pairs at once, with the Blackwell
-// packed FP32 operations (__ffma2_rn, __fadd2_rn, __fmul2_rn: two FP32
-// results per instruction, each rounded as the scalar operation); the
-// square roots, reciprocals, min/max and the saturated support test stay
-// scalar.  Same arithmetic per pair as pair_terms.
-template <int KERN, bool MOM>
-__device__ __forceinline__ void pair_terms2(const Dev& d, float c0, const float4& pi,
-                                            const float4& vi, float ci, float2 dx, float2 dy,
-                                            float2 dz, const float4& pa, const float4& va,
-                                            const float4& pb, const float4& vb, PairAcc2& s) {
-    const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-    const float r2s = d.r2max * 0x1p100f;
-    const float2 use = ff2(__saturatef(fmaf(d2.x, -0x1p100f, r2s)),
-                           __saturatef(fmaf(d2.y, -0x1p100f, r2s)));
-    s.npf = __fadd2_rn(s.npf, use);
-    const float2 q = __fmul2_rn(ff2(sqrt_approx(d2.x), sqrt_approx(d2.y)), dup2(d.inv_h));
-    float2 shape;
-    if (KERN == 1) {
-        const float2 wo = __ffma2_rn(q, dup2(-1.0f), dup2(2.0f));
-        const float2 outer =
-            __fmul2_rn(__fmul2_rn(dup2(-0.75f), __fmul2_rn(wo, wo)), ff2(rcp_approx(q.x), rcp_approx(q.y)));
-        const float2 inner = __ffma2_rn(dup2(2.25f), q, dup2(-3.0f));
-        shape = ff2(q.x < 1.0f ? inner.x : outer.x, q.y < 1.0f ? inner.y : outer.y);
-    } else {
-        const float2 wq = __ffma2_rn(dup2(-0.5f), q, dup2(1.0f));
-        shape = __fmul2_rn(__fmul2_rn(wq, wq), wq);
-    }
-    const float2 F = __fmul2_rn(__fmul2_rn(dup2(d.fc), shape), use);
-    const float2 m1 = dup2(-1.0f);
-    const float2 dvx = __ffma2_rn(ff2(va.x, vb.x), m1, dup2(vi.x));
-    const float2 dvy = __ffma2_rn(ff2(va.y, vb.y), m1, dup2(vi.y));
-    const float2 dvz = __ffma2_rn(ff2(va.z, vb.z), m1, dup2(vi.z));
-    const float2 vr = __ffma2_rn(dvx, dx, __ffma2_rn(dvy, dy, __fmul2_rn(dvz, dz)));
-    s.dr = __ffma2_rn(vr, F, s.dr);                                 // Eq. 7
-    if (MOM) {
-        const float2 de = __fadd2_rn(d2, dup2(d.eta2));
-        const float2 nu = __fmul2_rn(__fmul2_rn(dup2(d.h), vr), ff2(rcp_approx(de.x), rcp_approx(de.y)));
-        const float2 rrj = __fmul2_rn(ff2(va.w, vb.w), dup2(d.inv_rho0));
-        const float2 cj = __fmul2_rn(__fmul2_rn(__fmul2_rn(dup2(c0), rrj), rrj), rrj);
-        const float2 rs = __fadd2_rn(dup2(vi.w), ff2(va.w, vb.w));
-        const float2 nmin = ff2(fminf(nu.x, 0.f), fminf(nu.y, 0.f));
-        const float2 visc = __fmul2_rn(
-            __fmul2_rn(__fmul2_rn(dup2(-d.alpha), __fadd2_rn(dup2(ci), cj)), nmin),
-            ff2(rcp_approx(rs.x), rcp_approx(rs.y)));
-        const float2 f = __fmul2_rn(__fadd2_rn(__fadd2_rn(dup2(pi.w), ff2(pa.w, pb.w)), visc), F);
-        s.ax = __ffma2_rn(f, dx, s.ax);                              // Eq. 9 (sign later)
-        s.ay = __ffma2_rn(f, dy, s.ay);
-        s.az = __ffma2_rn(f, dz, s.az);
-        s.mu = fmaxf(s.mu, fmaxf(fabsf(nu.x) * use.x, fabsf(nu.y) * use.y));
-    }
-}
-
 // Sec. 3.2.  One block takes work units in turn: up to W*32 consecutive
 // sorted particles of one row of cells (same instance, cy, cz) spanning at
 // most kSpan cells with no more than two empty cells in a row, so the
@@ -530,8 +261,8 @@ __device__ __forceinline__ void pair_terms2(const Dev& d, float c0, const float4
 // keeps a similar share of its own neighbours in each part); the parts' sums
 // are added in a fixed order at the end.  More warps per block at the same
 // staging footprint.
-template <int W, int STAGE, int WCAP, int MINB, bool COUNTS, int SPLIT, int KERN, bool PK,
-          bool TU, bool DYN>
+template <int W, int STAGE, int WCAP, int MINB, bool COUNTS, int SPLIT, int KERN, bool TU,
+          bool DYN>
 __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, const InteractArgs a) {
     pdl_wait();
     constexpr int NT = W * SPLIT * 32;
@@ -677,7 +408,8 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
     }
     const float rri = vi.w * d.inv_rho0;
     const float ci = c0 * rri * rri * rri;
-    PairAcc acc = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u};
+    const float ri3 = rri * rri * rri, visc_k = -d.alpha * d.h * c0;
+    PairAcc acc = {0.f, 0.f, 0.f, 0.f, 0.f, 0u};
     uint32_t ncand = 0;
     __syncthreads();
     const bool staged = s_mode != 0;
@@ -861,38 +593,20 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
                         pp[k] = s_p[j2[k]];
                         vv[k] = s_v[j2[k]];
                     }
-                    if (PK) {
-                        const float2 m1 = dup2(-1.0f);
-                        const float2 dx2 = __ffma2_rn(ff2(pp[0].x, pp[1].x), m1, ff2(qx2[0], qx2[1]));
-                        const float2 dy2 = __ffma2_rn(ff2(pp[0].y, pp[1].y), m1, dup2(pi.y));
-                        const float2 dz2 = __ffma2_rn(ff2(pp[0].z, pp[1].z), m1, dup2(pi.z));
-                        if (anyfluid)
-                            pair_terms2<KERN, true>(d, c0, pi, vi, ci, dx2, dy2, dz2, pp[0], vv[0],
-                                                    pp[1], vv[1], acc2);
-                        else
-                            pair_terms2<KERN, false>(d, c0, pi, vi, ci, dx2, dy2, dz2, pp[0], vv[0],
-                                                     pp[1], vv[1], acc2);
-                    } else if (anyfluid) {
-#pragma unroll
-                        for (int k = 0; k < kPop; ++k)
-                            pair_terms<KERN, true, true>(d, c0, pi, vi, ci, qx2[k] - pp[k].x,
-                                                         pi.y - pp[k].y, pi.z - pp[k].z, pp[k],
-                                                         vv[k], acc);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < kPop; ++k)
-                            pair_terms<KERN, false, true>(d, c0, pi, vi, ci, qx2[k] - pp[k].x,
-                                                          pi.y - pp[k].y, pi.z - pp[k].z, pp[k],
-                                                          vv[k], acc);
-                    }
+                    const float2 m1 = dup2(-1.0f);
+                    const float2 dx2 = __ffma2_rn(ff2(pp[0].x, pp[1].x), m1, ff2(qx2[0], qx2[1]));
+                    const float2 dy2 = __ffma2_rn(ff2(pp[0].y, pp[1].y), m1, dup2(pi.y));
+                    const float2 dz2 = __ffma2_rn(ff2(pp[0].z, pp[1].z), m1, dup2(pi.z));
+                    if (anyfluid)
+                        pair_terms2<KERN, true>(d, visc_k, pi, vi, ri3, dx2, dy2, dz2, pp[0], vv[0],
+                                                pp[1], vv[1], acc2);
+                    else
+                        pair_terms2<KERN, false>(d, visc_k, pi, vi, ri3, dx2, dy2, dz2, pp[0], vv[0],
+                                                 pp[1], vv[1], acc2);
                 }
                 __syncwarp();   // every lane is done reading before the words are reused
-                acc.np += (uint32_t)acc.npf;
-                acc.npf = 0.f;
-                if (PK) {
-                    acc.np += (uint32_t)acc2.npf.x + (uint32_t)acc2.npf.y;
-                    acc2.npf = dup2(0.f);
-                }
+                acc.np += (uint32_t)acc2.npf.x + (uint32_t)acc2.npf.y;
+                acc2.npf = dup2(0.f);
                 nw = 0;
                 lane_hits = 0;
                 lane_nz = 0;
@@ -968,14 +682,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
                 }
             }
             flush();
-            if (PK) {
-                // the two streams' sums, in a fixed order (momentum negated once)
-                acc.ax -= acc2.ax.x + acc2.ax.y;
-                acc.ay -= acc2.ay.x + acc2.ay.y;
-                acc.az -= acc2.az.x + acc2.az.y;
-                acc.dr += acc2.dr.x + acc2.dr.y;
-                acc.mu = fmaxf(acc.mu, acc2.mu);
-            }
+            add_pairs2(d, acc2, acc);
         } else {
             // candidates straight from global memory (unit too large to stage)
             uint32_t* lst = reinterpret_cast<uint32_t*>(s_raw) + w * (FBCAP * 32);
@@ -991,7 +698,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
                         const float oz = (float)((int)(e >> 30) - 1);
                         const float4 pj = __ldg(a.posc + j);
                         const float4 vj = __ldg(a.velrhop + j);
-                        pair_terms<KERN, true>(d, c0, pi, vi, ci, fmaf(ox, d.csf, pi.x) - pj.x,
+                        pair_terms<KERN>(d, c0, pi, vi, ci, fmaf(ox, d.csf, pi.x) - pj.x,
                                                fmaf(oy, d.csf, pi.y) - pj.y,
                                                fmaf(oz, d.csf, pi.z) - pj.z, pj, vj, acc);
                     }
@@ -1715,55 +1422,39 @@ uint32_t max_units(uint32_t n, uint32_t nrows, uint64_t ncells) {
 
 namespace {
 
-using KernelPtr = void (*)(const Dev, const InteractArgs);
-
-struct Variant {
-    int warps;              // warps of particles (the unit is warps x 32 particles)
-    int split;              // warps per group of 32 particles
-    int stage;              // staged candidates
-    KernelPtr fn[2][2];     // [kernel: Wendland C2, cubic spline][with counts]
-    size_t smem;
-    int grid;   // persistent grid on this GPU (set by prepare_interact)
-};
-
 // (warps, staged candidates, hit-mask words per lane, resident blocks per SM
 // that the shared memory allows -- also the register budget hint)
-#define SPH_VARIANT_D(Wv, Sv, Cv, Bv, Pv, PKv, TUv, Dv)                               \
+#define SPH_VARIANT_D(Wv, Sv, Cv, Bv, Pv, TUv, Dv)                                   \
     Variant {                                                                        \
         Wv, Pv, Sv,                                                                  \
-            {{k_interact<Wv, Sv, Cv, Bv, false, Pv, 0, PKv, TUv, Dv>,                \
-              k_interact<Wv, Sv, Cv, Bv, true, Pv, 0, PKv, TUv, Dv>},                \
-             {k_interact<Wv, Sv, Cv, Bv, false, Pv, 1, PKv, TUv, Dv>,                \
-              k_interact<Wv, Sv, Cv, Bv, true, Pv, 1, PKv, TUv, Dv>}},               \
-            Shape<Wv * Pv, Sv, Cv>::smem, 0                                          \
+            {{k_interact<Wv, Sv, Cv, Bv, false, Pv, 0, TUv, Dv>,                     \
+              k_interact<Wv, Sv, Cv, Bv, true, Pv, 0, TUv, Dv>},                     \
+             {k_interact<Wv, Sv, Cv, Bv, false, Pv, 1, TUv, Dv>,                     \
+              k_interact<Wv, Sv, Cv, Bv, true, Pv, 1, TUv, Dv>}},                    \
+            Shape<Wv * Pv, Sv, Cv>::smem, 0, 0                                       \
     }
-#define SPH_VARIANT_T(Wv, Sv, Cv, Bv, Pv, PKv, TUv) \
-    SPH_VARIANT_D(Wv, Sv, Cv, Bv, Pv, PKv, TUv, false)
-#define SPH_VARIANT(Wv, Sv, Cv, Bv, Pv, PKv) SPH_VARIANT_T(Wv, Sv, Cv, Bv, Pv, PKv, false)
+#define SPH_VARIANT_T(Wv, Sv, Cv, Bv, Pv, TUv) SPH_VARIANT_D(Wv, Sv, Cv, Bv, Pv, TUv, false)
+#define SPH_VARIANT(Wv, Sv, Cv, Bv, Pv) SPH_VARIANT_T(Wv, Sv, Cv, Bv, Pv, false)
 
 Variant g_variants[kNumVariants] = {
-    SPH_VARIANT(4, 2048, 24, 2, 2, false),   // 128-particle units, two warps per 32 particles
-    SPH_VARIANT(4, 2048, 32, 2, 1, false),   // 128-particle units
-    SPH_VARIANT(3, 1280, 16, 3, 2, false),   // 96-particle units, two warps per 32, three per SM
-    SPH_VARIANT(3, 1408, 16, 3, 2, false),
-    SPH_VARIANT(2, 1280, 24, 3, 2, false),   // 64-particle units, two warps per 32 particles
-    SPH_VARIANT(4, 1792, 20, 2, 2, false),
-    SPH_VARIANT(3, 1152, 24, 4, 1, false),   // 96-particle units, four blocks per SM
-    // the same shapes with the pair terms of two pairs in packed FP32
-    SPH_VARIANT(4, 2048, 24, 2, 2, true),
-    SPH_VARIANT(3, 1408, 16, 3, 2, true),
-    SPH_VARIANT(4, 1792, 20, 2, 2, true),
-    // packed, and the candidate test's first eight pairs of a word unconditional
-    SPH_VARIANT_T(4, 2048, 24, 2, 2, true, true),
-    SPH_VARIANT_T(3, 1408, 16, 3, 2, true, true),
+    // candidate test on the tensor cores
+    tc_variant_n(0), tc_variant_n(1), tc_variant_n(2), tc_variant_n(3), tc_variant_n(4),
+    tc_variant_n(5), tc_variant_n(6),
+    // 128- and 96-particle units, two warps per 32 particles
+    SPH_VARIANT(4, 2048, 24, 2, 2),
+    SPH_VARIANT(3, 1408, 16, 3, 2),
+    SPH_VARIANT(4, 1792, 20, 2, 2),
+    // the candidate test's first eight pairs of a word unconditional
+    SPH_VARIANT_T(4, 2048, 24, 2, 2, true),
+    SPH_VARIANT_T(3, 1408, 16, 3, 2, true),
     // 32-particle units shared by four warps, four blocks per SM: shorter
     // dependent chains per unit for small systems (fewer units than SMs)
-    SPH_VARIANT_T(1, 1024, 12, 4, 4, true, true),
+    SPH_VARIANT_T(1, 1024, 12, 4, 4, true),
     // units taken from a counter, the next unit's record and cell offsets
     // fetched during the current one
-    SPH_VARIANT_D(4, 2048, 24, 2, 2, true, true, true),
-    SPH_VARIANT_D(3, 1408, 16, 3, 2, true, true, true),
-    SPH_VARIANT_D(1, 1024, 12, 4, 4, true, true, true),
+    SPH_VARIANT_D(4, 2048, 24, 2, 2, true, true),
+    SPH_VARIANT_D(3, 1408, 16, 3, 2, true, true),
+    SPH_VARIANT_D(1, 1024, 12, 4, 4, true, true),
 };
 
 }  // namespace
@@ -1841,20 +1532,34 @@ void prepare_interact() {
         const bool want = !(e && e[0] == '0');
         g_pdl = want && probe_pdl();
     });
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, smem_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     for (Variant& v : g_variants) {
         for (int k = 0; k < 2; ++k)
             for (int c = 0; c < 2; ++c)
                 cudaFuncSetAttribute(v.fn[k][c], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)v.smem);
-        // one grid for both kernels of the shape: the smaller residency
+        // one grid for both kernels of the shape: the smaller residency.  The
+        // occupancy call counts one block per SM for a kernel that allocates
+        // TMEM, so the tensor-core shapes are sized by their shared memory,
+        // registers and TMEM columns instead
         int per_sm = 0;
         for (int k = 0; k < 2; ++k) {
             int r = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, v.fn[k][0], v.warps * v.split * 32,
-                                                          v.smem);
+            if (v.max_per_sm) {
+                cudaFuncAttributes fa{};
+                cudaFuncGetAttributes(&fa, v.fn[k][0]);
+                const int by_smem = (int)((size_t)smem_sm / (v.smem + fa.sharedSizeBytes + 1024u));
+                const int regs = (fa.numRegs + 7) / 8 * 8 * v.warps * v.split * 32;
+                const int by_regs = regs > 0 ? 65536 / regs : 1;
+                r = by_smem < by_regs ? by_smem : by_regs;
+                if (r > v.max_per_sm) r = v.max_per_sm;
+            } else {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, v.fn[k][0],
+                                                              v.warps * v.split * 32, v.smem);
+            }
             per_sm = k == 0 || r < per_sm ? r : per_sm;
         }
         v.grid = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
