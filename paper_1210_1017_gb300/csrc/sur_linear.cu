@@ -5,7 +5,10 @@
 // ReLU mask of the backward pass) fused after the tcgen05.ld of the fp32
 // accumulator.  Also the weight gradient dW = X^T dY, reduced over rows in
 // TMEM per block and then across blocks in a fixed order.
+#include <cuda.h>
 #include <cuda_bf16.h>
+
+#include <mutex>
 
 #include "sur_gemm.cuh"
 #include "sur_internal.cuh"
@@ -530,12 +533,8 @@ __global__ void __launch_bounds__(256, 2) k_edge_encoder(const EdgeArgs g) {
     if (w == 0) tmem_dealloc(tmem, 256);
 }
 
-// Named barrier of one half of a 512-thread block (ids 1 and 2, 256 threads),
-// and its AND-reduction over a predicate.
-__device__ __forceinline__ void half_sync(int h) {
-    asm volatile("bar.sync %0, 256;" ::"r"(h + 1) : "memory");
-}
-
+// AND-reduction over the 256 threads of one half of a 512-thread block (named
+// barriers 1 and 2).
 __device__ __forceinline__ bool half_and(int h, bool v) {
     uint32_t r;
     asm volatile(
@@ -549,37 +548,54 @@ __device__ __forceinline__ bool half_and(int h, bool v) {
 
 // The fused edge update of a message-passing layer, per 128-edge tile:
 //   z = relu(e W1c + b1 + P[src] + Q[dst]),  e' = e + z W2 + b2
-// (MMA 1 into TMEM, z written as MMA 2's K-major operand in shared memory and
-// to Z when training, MMA 2, the residual e read back from the staged tile),
 // as two independent halves of 256 threads that share the weights: half h
 // takes the tiles 2 b + h, 2 b + h + 2 grid, ... of block b with its own
-// mbarrier, its own 256 TMEM columns (accumulators of MMA 1 and MMA 2) and
-// its own named barrier, so one half's MMAs, copies and barriers overlap the
-// other half's epilogues.  Per half: the e tile, and the P[src] rows that z
-// overwrites; the Q[dst] rows go to registers (each thread's row and 64
-// columns): the next tile's are loaded while this tile's MMA 2 and second
-// epilogue run.  The next tile's e and P[src] copies are issued at the end
-// of a tile, the row indices a tile ahead.
-constexpr size_t kEdgePPSmem = (size_t)6 * 128 * 128 * 2;   // W1c, W2, 2 x (e, P/z)
+// mbarriers, 256 TMEM columns and named barrier, so one half's MMAs, copies
+// and barriers overlap the other half's epilogues.
+//
+// HBM is the floor (e in, e' out: 512 B per edge, 768 with Z), so the loads
+// of a tile are in flight before its turn and nothing goes through L1 row by
+// row that can go as a tile: with per-thread copies of the e, e' and z rows
+// the kernel ran at the L1's rate of one 128-byte line per clock (69% of it,
+// 0.68 instructions per clock).  The e tile comes by TMA in the 128-byte
+// swizzle, is read by MMA 1 and by the second epilogue (a thread per row: no
+// bank conflicts), overwritten in place by e' and stored by TMA.  z is MMA
+// 2's A operand in TMEM (tcgen05.st), which leaves shared memory for two e
+// tiles per half; the gathered rows go to registers a tile ahead, 32 bytes
+// per load.  Accumulators and z alternate between the halves X and Y of the
+// 256 columns: MMA 1 of tile t in X, z in Y, MMA 2 back into X, and MMA 1 of
+// tile t + 1 into Y as soon as MMA 2 has read z, under tile t's second
+// epilogue.  On one GB300, with Z, 1.5M edges: 572 us with the loads issued at
+// the end of a tile, 466 with z in TMEM and the loads ahead, 300 with the
+// tiles by TMA (3.9 TB/s of e, e' and z, 57% of the copy bandwidth).
+constexpr uint32_t kETile = 128 * 128 * 2;                  // bytes of one e tile
+constexpr size_t kEdgePPSmem = (size_t)6 * kETile + 1024;   // W1c, W2, 2 x 2 e tiles; alignment
 
-__global__ void __launch_bounds__(512, 1) k_edge_pp(const EdgeArgs g) {
+__global__ void __launch_bounds__(512, 1)
+    k_edge_pp(const EdgeArgs g, const __grid_constant__ CUtensorMap map_e,
+              const __grid_constant__ CUtensorMap map_out, const bool wide) {
     constexpr int N = 128;
-    constexpr uint32_t T = 128 * 128 * 2;
-    extern __shared__ __align__(128) unsigned char s_raw[];
+    constexpr uint32_t T = kETile, BOX = T / 2;          // a box: 64 columns of 128 rows
+    extern __shared__ unsigned char s_dyn[];
     __shared__ __align__(16) float s_b1[128], s_b2[128];
-    __shared__ __align__(8) uint64_t s_bar[2];
+    // completions of MMA 1 and of MMA 2, per half (a barrier each: MMA 1 of the
+    // next tile may complete before every thread has seen MMA 2); e tile loaded,
+    // per half and buffer
+    __shared__ __align__(8) uint64_t s_bar[2][2], s_full[2][2];
     __shared__ uint32_t s_tmem;
+    unsigned char* s_raw = s_dyn + ((1024u - (sm_addr(s_dyn) & 1023u)) & 1023u);
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int h = tid >> 8, lt = tid & 255;              // half, thread within the half
     unsigned char* sw1 = s_raw;                          // W1c^T
     unsigned char* sw2 = s_raw + T;                      // W2^T
-    unsigned char* se = s_raw + (2 + h) * T;             // e tile of this half
-    unsigned char* spz = s_raw + (4 + h) * T;            // P[src] rows, then z
     if (w == 0) tmem_alloc(&s_tmem, 512);
-    if (tid == 0) {
-        mbar_init1(&s_bar[0]);
-        mbar_init1(&s_bar[1]);
-    }
+    if (tid == 0)
+        for (int k = 0; k < 2; ++k) {
+            mbar_init1(&s_bar[k][0]);
+            mbar_init1(&s_bar[k][1]);
+            mbar_init1(&s_full[k][0]);
+            mbar_init1(&s_full[k][1]);
+        }
     for (int c = tid; c < N * (N / 8); c += 512) {
         const int r = c % N, gk = c / N;
         cp_async16(sw1 + kmajor_offset(r, gk * 8, N), g.W1t + (size_t)r * N + gk * 8, true);
@@ -589,169 +605,200 @@ __global__ void __launch_bounds__(512, 1) k_edge_pp(const EdgeArgs g) {
         s_b1[tid] = g.b1[tid];
         s_b2[tid] = g.b2[tid];
     }
-    const uint32_t ntiles = (g.M + 127) / 128;
-    const uint32_t stride = 2 * gridDim.x;
-    const int wq = w & 3, part = (w >> 2) & 1;           // lane quarter, column half
-    const int r = wq * 32 + lane;                        // epilogue row of this thread
-    const uint32_t gr = (uint32_t)(lt & 127);            // gather row of this thread
-    const int gh = lt >> 7;                              // its half of the row's pieces
-    // copies of one tile's e and P[src] rows by this half
-    auto issue_tile = [&](uint32_t t, uint32_t srow) {
-#pragma unroll
-        for (int c = lt; c < 128 * (N / 8); c += 256) {
-            const int rr = c & 127, gk = c >> 7;
-            const bool ok = t * 128 + rr < g.M;
-            const __nv_bfloat16* p = ok ? g.E + (size_t)(t * 128 + rr) * N + gk * 8 : g.E;
-            cp_async16(se + kmajor_offset(rr, gk * 8, N), p, ok);
-        }
-        const bool ok = t * 128 + gr < g.M;
-        const __nv_bfloat16* p = ok ? g.P + (size_t)srow * N : g.P;
-#pragma unroll
-        for (int gk = 8 * gh; gk < 8 * gh + 8; ++gk)
-            cp_async16(spz + kmajor_offset(gr, gk * 8, N), p + gk * 8, ok);
-    };
-    // this thread's 64 columns of one Q[dst] row
-    uint4 qv[8];
-    auto load_q = [&](uint32_t t, uint32_t drow) {
-        const bool ok = t * 128 + r < g.M;
-        const uint4* q = reinterpret_cast<const uint4*>(g.Q + (size_t)(ok ? drow : 0u) * N + part * 64);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) qv[k] = ok ? __ldg(q + k) : make_uint4(0u, 0u, 0u, 0u);
-    };
-    uint32_t tile = 2 * blockIdx.x + (uint32_t)h;
-    uint32_t nsrc = 0, ndst = 0;                         // rows of the half's next tile
-    if (tile < ntiles) {
-        const uint32_t mg = tile * 128 + gr, me = tile * 128 + (uint32_t)r;
-        issue_tile(tile, mg < g.M ? g.src[mg] : 0u);
-        load_q(tile, me < g.M ? g.dst[me] : 0u);
-        const uint32_t nt = tile + stride;
-        if (nt < ntiles) {
-            if (nt * 128 + gr < g.M) nsrc = g.src[nt * 128 + gr];
-            if (nt * 128 + (uint32_t)r < g.M) ndst = g.dst[nt * 128 + r];
-        }
-    }
-    cp_async_commit();
-    cp_async_wait_all();                                 // weights of both halves, first tiles
+    cp_async_wait_all();
     fence_async_shared();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = s_tmem + (uint32_t)(h * 256);
-    const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
-    uint32_t phase = 0;
-    bool ok = true;
-    for (; tile < ntiles && ok; tile += stride) {
-        cp_async_wait_all();                             // e, P[src] of this tile
-        fence_async_shared();
-        tc_fence_before();
-        half_sync(h);
-        if (lt == 0) {
-            tc_fence_after();
+    const uint32_t ntiles = (g.M + 127) / 128;
+    const uint32_t stride = 2 * gridDim.x;
+    unsigned char* se0 = s_raw + (2 + 2 * h) * T;        // this half's two e tiles
+    const int wq = w & 3, part = (w >> 2) & 1;           // lane quarter, column half
+    const int r = wq * 32 + lane;                        // this thread's row of a tile
+    const bool mover = lt == 32;                         // moves the half's tiles
+    auto load_e = [&](uint32_t t, uint32_t b) {
+        mbar_expect(&s_full[h][b], T);
+        tma_load(se0 + b * T, &map_e, 0, (int)(t * 128), &s_full[h][b]);
+        tma_load(se0 + b * T + BOX, &map_e, 64, (int)(t * 128), &s_full[h][b]);
+    };
+    // this thread's 64 columns of a node row (wide: 32-byte aligned rows)
+    auto load_row = [&](uint4 (&v)[8], const __nv_bfloat16* rows, uint32_t row, bool ok) {
+        const uint4* q = reinterpret_cast<const uint4*>(rows + (size_t)(ok ? row : 0u) * N + part * 64);
+        if (wide) {
 #pragma unroll
-            for (int s = 0; s < N / 16; ++s) {
-                const uint64_t ad = smem_desc(sm_addr(se) + s * 256, kLBO, (N / 8) * 128);
-                const uint64_t bd = smem_desc(sm_addr(sw1) + s * 256, kLBO, (N / 8) * 128);
-                tc_mma(tmem, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
-            }
-            tc_commit(&s_bar[h]);
+            for (int k = 0; k < 8; k += 2) ldg32(q + k, v[k], v[k + 1]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = __ldg(q + k);
         }
-        const uint32_t m = tile * 128 + (uint32_t)r;
-        const bool valid = m < g.M;
-        const uint32_t next = tile + stride;
-        bool got = mbar_wait(&s_bar[h], phase);
-        ok = half_and(h, got);
-        if (!ok) break;
-        phase ^= 1u;
+    };
+    uint4 pv[8], qv[8];                                  // P[src], Q[dst] of the tile in hand
+    uint32_t tile = 2 * blockIdx.x + (uint32_t)h;
+    uint32_t nsrc = 0, ndst = 0;                         // node rows of the half's next tile
+    if (tile < ntiles) {
+        if (mover) {
+            load_e(tile, 0);
+            if (tile + stride < ntiles) load_e(tile + stride, 1);
+        }
+        const uint32_t m0 = tile * 128 + (uint32_t)r, m1 = m0 + stride * 128;
+        load_row(pv, g.P, m0 < g.M ? g.src[m0] : 0u, m0 < g.M);
+        load_row(qv, g.Q, m0 < g.M ? g.dst[m0] : 0u, m0 < g.M);
+        if (tile + stride < ntiles && m1 < g.M) {
+            nsrc = g.src[m1];
+            ndst = g.dst[m1];
+        }
+    }
+    const uint32_t tmem = s_tmem + (uint32_t)(h * 256);
+    const uint32_t quarter = (uint32_t)(wq * 32) << 16;
+    // MMA 1 of the e tile in buffer se into accumulator columns d (one thread)
+    auto mma1 = [&](const unsigned char* se, uint32_t d) {
         tc_fence_after();
-        // epilogue 1: z = relu(((acc + b1) + P[src]) + Q[dst]) over the P rows, and to Z
+#pragma unroll
+        for (int s = 0; s < N / 16; ++s) {
+            const uint64_t ad = smem_desc_sw128(sm_addr(se) + (s >> 2) * BOX + (s & 3) * 32);
+            const uint64_t bd = smem_desc(sm_addr(sw1) + s * 256, kLBO, (N / 8) * 128);
+            tc_mma(d, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
+        }
+        tc_commit(&s_bar[h][0]);
+    };
+    uint32_t phase = 0, x = 0, buf = 0, epar = 0;        // x: column offset of X (0 or 128);
+                                                         // bit b of epar: phase of s_full[h][b]
+    bool ok = true, first = true;
+    if (tile < ntiles && lt == 0 && mbar_wait(&s_full[h][0], 0)) mma1(se0, tmem);
+    for (; tile < ntiles; tile += stride) {
+        unsigned char* se = se0 + buf * T + part * BOX;  // this thread's box of the tile
+        const uint32_t m = tile * 128 + (uint32_t)r;
+        const uint32_t next = tile + stride;
+        bool got = mbar_wait(&s_bar[h][0], phase);       // MMA 1
+        tc_fence_after();
+        // epilogue 1: z = relu(((acc + b1) + P[src]) + Q[dst]) into Y, and to Z
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+            // the next tile's e, once the store of the tile before this one has
+            // read that buffer (it has by the middle of this epilogue)
+            if (k == 2 && mover && !first && next < ntiles) {
+                bulk_wait_read();
+                load_e(next, buf ^ 1u);
+            }
+            if (k == 2) __syncwarp();
             const int c0 = part * 64 + 16 * k;
             float v[16];
-            tmem_ld16(lane_base + c0, v);
+            tmem_ld16(tmem + x + quarter + c0, v);
             float t[16], u[16];
-            unpack8(*reinterpret_cast<const uint4*>(spz + kmajor_offset(r, c0, N)), t);
-            unpack8(*reinterpret_cast<const uint4*>(spz + kmajor_offset(r, c0 + 8, N)), t + 8);
+            unpack8(pv[2 * k], t);
+            unpack8(pv[2 * k + 1], t + 8);
             unpack8(qv[2 * k], u);
             unpack8(qv[2 * k + 1], u + 8);
-            const float2* b2v = reinterpret_cast<const float2*>(s_b1 + c0);
-            __nv_bfloat162 hh[8];
+            const float4* b4 = reinterpret_cast<const float4*>(s_b1 + c0);
+            uint32_t z[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]), b2v[q]);
-                a = __fadd2_rn(a, make_float2(t[2 * q], t[2 * q + 1]));
-                a = __fadd2_rn(a, make_float2(u[2 * q], u[2 * q + 1]));
-                hh[q] = __floats2bfloat162_rn(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+                const float4 bb = b4[q >> 1];
+                float2 s = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]),
+                                      q & 1 ? make_float2(bb.z, bb.w) : make_float2(bb.x, bb.y));
+                s = __fadd2_rn(s, make_float2(t[2 * q], t[2 * q + 1]));
+                s = __fadd2_rn(s, make_float2(u[2 * q], u[2 * q + 1]));
+                // rounding and the maximum with 0 commute
+                const __nv_bfloat162 zz =
+                    __hmax2(__floats2bfloat162_rn(s.x, s.y), __floats2bfloat162_rn(0.f, 0.f));
+                z[q] = *reinterpret_cast<const uint32_t*>(&zz);
             }
-            const uint4 z0 = *reinterpret_cast<uint4*>(&hh[0]);
-            const uint4 z1 = *reinterpret_cast<uint4*>(&hh[4]);
-            *reinterpret_cast<uint4*>(spz + kmajor_offset(r, c0, N)) = z0;
-            *reinterpret_cast<uint4*>(spz + kmajor_offset(r, c0 + 8, N)) = z1;
-            if (g.Z && valid) {
+            tmem_st8(tmem + (x ^ 128u) + quarter + (uint32_t)(c0 / 2), z);
+            if (g.Z && m < g.M) {
                 uint4* o = reinterpret_cast<uint4*>(g.Z + (size_t)m * N + c0);
-                o[0] = z0;
-                o[1] = z1;
+                const uint4 z0 = make_uint4(z[0], z[1], z[2], z[3]);
+                const uint4 z1 = make_uint4(z[4], z[5], z[6], z[7]);
+                if (wide) {
+                    stg32(o, z0, z1);
+                } else {
+                    o[0] = z0;
+                    o[1] = z1;
+                }
             }
         }
-        fence_async_shared();
+        tmem_st_wait();
         tc_fence_before();
-        half_sync(h);                                    // z complete
+        ok = half_and(h, got);                           // z complete
+        if (!ok) break;
         if (lt == 0) {
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < N / 16; ++s) {
-                const uint64_t ad = smem_desc(sm_addr(spz) + s * 256, kLBO, (N / 8) * 128);
                 const uint64_t bd = smem_desc(sm_addr(sw2) + s * 256, kLBO, (N / 8) * 128);
-                tc_mma(tmem + 128, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
+                tc_mma_ta(tmem + x, tmem + (x ^ 128u) + s * 8, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
             }
-            tc_commit(&s_bar[h]);
+            tc_commit(&s_bar[h][1]);
         }
-        // the next tile's Q[dst] rows into registers, the rows of the one after
-        uint32_t nsrc2 = 0, ndst2 = 0;
+        // the next tile's node rows into registers, the row numbers of the
+        // one after
         if (next < ntiles) {
-            load_q(next, ndst);
-            const uint32_t n2 = next + stride;
-            if (n2 < ntiles) {
-                if (n2 * 128 + gr < g.M) nsrc2 = __ldg(g.src + n2 * 128 + gr);
-                if (n2 * 128 + (uint32_t)r < g.M) ndst2 = __ldg(g.dst + n2 * 128 + r);
+            const bool nok = next * 128 + (uint32_t)r < g.M;
+            load_row(pv, g.P, nsrc, nok);
+            load_row(qv, g.Q, ndst, nok);
+            const uint32_t m2 = (next + stride) * 128 + (uint32_t)r;
+            if (next + stride < ntiles && m2 < g.M) {
+                nsrc = __ldg(g.src + m2);
+                ndst = __ldg(g.dst + m2);
             }
         }
-        got = mbar_wait(&s_bar[h], phase);
-        ok = half_and(h, got);
-        if (!ok) break;
-        phase ^= 1u;
+        got = mbar_wait(&s_bar[h][1], phase);            // MMA 2
         tc_fence_after();
-        // epilogue 2: e' = (acc + b2) + e
+        // z has been read: MMA 1 of the next tile over it
+        if (got && lt == 0 && next < ntiles) {
+            got = mbar_wait(&s_full[h][buf ^ 1u], (epar >> (buf ^ 1u)) & 1u);
+            if (got) mma1(se0 + (buf ^ 1u) * T, tmem + (x ^ 128u));
+        }
+        // this tile's e has long landed (MMA 1 read it): the wait makes it
+        // visible to this thread
+        got = mbar_wait(&s_full[h][buf], (epar >> buf) & 1u) && got;
+        epar ^= 1u << buf;
+        // epilogue 2: e' = (acc + b2) + e, over e
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int c0 = part * 64 + 16 * k;
             float v[16];
-            tmem_ld16(lane_base + 128 + c0, v);
-            if (!valid) continue;
+            tmem_ld16(tmem + x + quarter + c0, v);
+            uint4* e0 = reinterpret_cast<uint4*>(se + sw128_offset(r, 2 * k));
+            uint4* e1 = reinterpret_cast<uint4*>(se + sw128_offset(r, 2 * k + 1));
             float t[16];
-            unpack8(*reinterpret_cast<const uint4*>(se + kmajor_offset(r, c0, N)), t);
-            unpack8(*reinterpret_cast<const uint4*>(se + kmajor_offset(r, c0 + 8, N)), t + 8);
-            const float2* b2v = reinterpret_cast<const float2*>(s_b2 + c0);
+            unpack8(*e0, t);
+            unpack8(*e1, t + 8);
+            const float4* b4 = reinterpret_cast<const float4*>(s_b2 + c0);
             __nv_bfloat162 hh[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]), b2v[q]);
-                a = __fadd2_rn(a, make_float2(t[2 * q], t[2 * q + 1]));
-                hh[q] = __floats2bfloat162_rn(a.x, a.y);
+                const float4 bb = b4[q >> 1];
+                float2 s = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]),
+                                      q & 1 ? make_float2(bb.z, bb.w) : make_float2(bb.x, bb.y));
+                s = __fadd2_rn(s, make_float2(t[2 * q], t[2 * q + 1]));
+                hh[q] = __floats2bfloat162_rn(s.x, s.y);
             }
-            uint4* o = reinterpret_cast<uint4*>(g.Eout + (size_t)m * N + c0);
-            o[0] = *reinterpret_cast<uint4*>(&hh[0]);
-            o[1] = *reinterpret_cast<uint4*>(&hh[4]);
+            *e0 = *reinterpret_cast<uint4*>(&hh[0]);
+            *e1 = *reinterpret_cast<uint4*>(&hh[4]);
         }
+        fence_async_shared();
         tc_fence_before();
-        half_sync(h);                                    // e and z tiles free
-        if (next < ntiles) issue_tile(next, nsrc);
-        cp_async_commit();
-        nsrc = nsrc2;
-        ndst = ndst2;
+        ok = half_and(h, got);                           // X free, e' complete
+        if (!ok) break;
+        if (mover) {
+            tma_store(&map_out, se0 + buf * T, 0, (int)(tile * 128));
+            tma_store(&map_out, se0 + buf * T + BOX, 64, (int)(tile * 128));
+            bulk_commit();
+        }
+        first = false;
+        x ^= 128u;
+        buf ^= 1u;
+        phase ^= 1u;
     }
-    if (!ok && lt == 0 && g.status) atomicOr(g.status, 1u);
-    cp_async_wait_all();
+    if (!ok) {
+        if (lt == 0 && g.status) atomicOr(g.status, 1u);
+        mbar_wait(&s_bar[h][0], phase);                  // let MMAs and copies in flight
+        mbar_wait(&s_bar[h][1], phase);                  // land first
+        mbar_wait(&s_full[h][0], epar & 1u);
+        mbar_wait(&s_full[h][1], (epar >> 1) & 1u);
+    }
+    if (mover) bulk_wait();
+    tc_fence_before();
     __syncthreads();
     if (w == 0) tmem_dealloc(s_tmem, 512);
 }
@@ -829,19 +876,54 @@ bool launch_linear(int K, int N, const LinearArgs& g, cudaStream_t st) {
     return true;
 }
 
-// The layer: two halves per block, one block per SM (192 KB of shared memory,
+namespace {
+
+// Tensor map of an M x 128 bf16 matrix in boxes of 128 rows x 64 columns with
+// the 128-byte swizzle.  Rows past M load as zeros and are not stored.
+bool tile_map(CUtensorMap* map, const void* base, uint32_t M) {
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                             &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Encode>(fn);
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {128, M}, strides[1] = {256};
+    const cuuint32_t box[2] = {64, 128}, step[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+                  box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
+}
+
+}  // namespace
+
+// The layer: two halves per block, one block per SM (193 KB of shared memory,
 // the SM's 512 TMEM columns).
-void launch_edge_layer(const EdgeArgs& g, cudaStream_t st) {
-    static bool init = false;
-    if (!init) {
+bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st) {
+    static std::once_flag once;
+    std::call_once(once, [] {
         cudaFuncSetAttribute(k_edge_pp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEdgePPSmem);
-        init = true;
-    }
-    if (g.M == 0) return;
+    });
+    if (g.M == 0) return true;
+    CUtensorMap map_e, map_out;
+    if (!tile_map(&map_e, g.E, g.M) || !tile_map(&map_out, g.Eout, g.M)) return false;
+    const uintptr_t all = reinterpret_cast<uintptr_t>(g.P) | reinterpret_cast<uintptr_t>(g.Q) |
+                          reinterpret_cast<uintptr_t>(g.Z);
     const uint32_t tiles = (g.M + 127) / 128;
     uint32_t grid = (uint32_t)num_sms();
     if (grid > (tiles + 1) / 2) grid = (tiles + 1) / 2;
-    k_edge_pp<<<grid, 512, kEdgePPSmem, st>>>(g);
+    k_edge_pp<<<grid, 512, kEdgePPSmem, st>>>(g, map_e, map_out, all % 32u == 0u);
+    return true;
 }
 
 // The encoder: two 256-thread blocks per SM.

@@ -614,8 +614,8 @@ int linear(sur_ctx* c, const __nv_bfloat16* A, uint32_t lda, const Layer& l, boo
 
 // The fused edge update of one layer: z = relu(e W1c + b1 + P[src] + Q[dst])
 // (kept for the backward pass when z != null), e' = e + z W2 + b2.
-void edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* e,
-                __nv_bfloat16* z, __nv_bfloat16* e_out) {
+int edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* e,
+               __nv_bfloat16* z, __nv_bfloat16* e_out) {
     EdgeArgs g = {};
     g.E = e;
     g.W1t = l1.Wt;
@@ -629,7 +629,8 @@ void edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat1
     g.M = c->E;
     g.Z = z;
     g.Eout = e_out;
-    launch_edge_layer(g, c->st);
+    if (!launch_edge_layer(g, c->st)) return fail(c, SPH_ERR_CUDA, "edge layer: no tensor maps");
+    return SPH_OK;
 }
 
 // The two edge-encoder layers in one kernel: e0 = relu(xe W + b) W' + b'
@@ -770,7 +771,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
         const Layer* w = &Ls[4 + 6 * l];
         if ((rc = linear(c, xn_cur, 2 * L, w[0], false, n, kEpiNone, nullptr, 0, c->P, nullptr, L))) return rc;
         if ((rc = linear(c, xn_cur, 2 * L, w[1], false, n, kEpiNone, nullptr, 0, c->Q, nullptr, L))) return rc;
-        edge_layer(c, w[2], w[3], e_in, train ? z1 : nullptr, e_out);
+        if ((rc = edge_layer(c, w[2], w[3], e_in, train ? z1 : nullptr, e_out))) return rc;
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, e_out, nullptr,
                                                                            xn_cur + L, nullptr, 2 * L);
         if ((rc = linear(c, xn_cur, 0, w[4], false, n, kEpiRelu, nullptr, 0, y1, nullptr, L))) return rc;
