@@ -194,7 +194,15 @@ __device__ __forceinline__ void bulk_wait() {
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// 32 bytes of global memory in one instruction (32-byte aligned).
+// 32 bytes of global memory in one instruction (32-byte aligned); ldg32: data
+// that the kernel does not write.
+__device__ __forceinline__ void ld32(const void* p, uint4& a, uint4& b) {
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z),
+                   "=r"(b.w)
+                 : "l"(p)
+                 : "memory");
+}
 __device__ __forceinline__ void ldg32(const void* p, uint4& a, uint4& b) {
     asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z),

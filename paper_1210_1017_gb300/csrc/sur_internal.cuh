@@ -32,6 +32,7 @@ struct LinearArgs {
     float* out_f32;             // M x ldo (may be null)
     uint32_t ldo;
     uint32_t* status;           // bit 0: a bounded wait gave up
+    bool wide;                  // 32-byte accesses in the epilogue (set by launch_linear)
 };
 
 // D[128 x N] = P^T Q summed over rows [0, M): P is M x 128, Q is M x N (bf16,

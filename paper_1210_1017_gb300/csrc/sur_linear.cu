@@ -23,14 +23,14 @@ __device__ __forceinline__ constexpr uint32_t tmem_cols() {
 }
 
 // Issue the asynchronous copies of a (128 x K) bf16 tile (rows past nrows
-// zero-filled) into the canonical K-major layout; consecutive threads take
-// consecutive rows of one 16-byte column piece.
+// zero-filled) into the canonical K-major layout; two lanes take the 32 bytes
+// of a memory sector, consecutive pairs consecutive rows.
 template <int K, int THR = 128>
 __device__ __forceinline__ void issue_rows(unsigned char* dst, const __nv_bfloat16* src,
                                            uint32_t row0, uint32_t nrows, uint32_t ld) {
 #pragma unroll
     for (int c = threadIdx.x; c < 128 * (K / 8); c += THR) {
-        const int r = c & 127, gk = c >> 7;
+        const int r = (c >> 1) & 127, gk = 2 * (c >> 8) + (c & 1);
         const bool ok = row0 + r < nrows;
         const __nv_bfloat16* p = ok ? src + (size_t)(row0 + r) * ld + gk * 8 : src;
         cp_async16(dst + kmajor_offset(r, gk * 8, K), p, ok);
@@ -56,34 +56,37 @@ struct EpiOps {
     uint4 b[NP / 8];
 };
 
+// NV 16-byte pieces of a row, 32 bytes per load when `wide` (the L1 takes one
+// 128-byte line per clock and a thread's row is a line of its own, so halving
+// the loads halves that cost).
+template <int NV>
+__device__ __forceinline__ void load_pieces(uint4* v, const void* row, bool wide) {
+    const uint4* p = reinterpret_cast<const uint4*>(row);
+    if (wide) {
+#pragma unroll
+        for (int i = 0; i < NV; i += 2) ld32(p + i, v[i], v[i + 1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = p[i];
+    }
+}
+
 template <int N, int NP>
 __device__ __forceinline__ void epi_load(EpiOps<NP>& o, const LinearArgs& g, uint32_t m,
                                          uint32_t gi, uint32_t gj, uint32_t ldr, int col0) {
     switch (g.epi) {
-        case kEpiEdge1: {
-            const uint4* p = reinterpret_cast<const uint4*>(g.gp + (size_t)gi * N + col0);
-            const uint4* q = reinterpret_cast<const uint4*>(g.gq + (size_t)gj * N + col0);
-#pragma unroll
-            for (int i = 0; i < NP / 8; ++i) {
-                o.a[i] = p[i];
-                o.b[i] = q[i];
-            }
+        case kEpiEdge1:
+            load_pieces<NP / 8>(o.a, g.gp + (size_t)gi * N + col0, g.wide);
+            load_pieces<NP / 8>(o.b, g.gq + (size_t)gj * N + col0, g.wide);
             break;
-        }
         case kEpiResidual:
-        case kEpiReluMask: {
-            const uint4* p = reinterpret_cast<const uint4*>(g.res + (size_t)m * ldr + col0);
-#pragma unroll
-            for (int i = 0; i < NP / 8; ++i) o.a[i] = p[i];
+        case kEpiReluMask:
+            load_pieces<NP / 8>(o.a, g.res + (size_t)m * ldr + col0, g.wide);
             break;
-        }
         case kEpiAccum: {
-            const uint4* p = reinterpret_cast<const uint4*>(g.out_f32 + (size_t)m * g.ldo + col0);
-#pragma unroll
-            for (int i = 0; i < NP / 8; ++i) {
-                o.a[i] = p[i];
-                o.b[i] = p[NP / 8 + i];
-            }
+            const float* p = g.out_f32 + (size_t)m * g.ldo + col0;
+            load_pieces<NP / 8>(o.a, p, g.wide);
+            load_pieces<NP / 8>(o.b, p + NP / 2, g.wide);
             break;
         }
         default: break;
@@ -174,7 +177,7 @@ __global__ void __launch_bounds__(linear_threads<N>(), 1) k_linear(const LinearA
 #pragma unroll
             for (int cl = 0; cl < NP; cl += 16) {
                 const int c0 = col0 + h * NP + cl;
-                float v[16];
+                alignas(16) float v[16];
                 tmem_ld16(tmem + ((uint32_t)(wq * 32) << 16) + c0, v);
                 if (!valid) continue;
                 if (g.bias) {
@@ -228,18 +231,29 @@ __global__ void __launch_bounds__(linear_threads<N>(), 1) k_linear(const LinearA
                     default: break;
                 }
                 if (g.out_f32) {
-                    float4* o = reinterpret_cast<float4*>(g.out_f32 + (size_t)m * g.ldo + c0);
+                    const uint4* vv = reinterpret_cast<const uint4*>(v);
+                    uint4* o = reinterpret_cast<uint4*>(g.out_f32 + (size_t)m * g.ldo + c0);
+                    if (g.wide) {
+                        stg32(o, vv[0], vv[1]);
+                        stg32(o + 2, vv[2], vv[3]);
+                    } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                        for (int q = 0; q < 4; ++q) o[q] = vv[q];
+                    }
                 }
                 if (g.out_bf16) {
                     __nv_bfloat162 hh[8];
 #pragma unroll
                     for (int q = 0; q < 8; ++q) hh[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+                    const uint4 h0 = *reinterpret_cast<uint4*>(&hh[0]);
+                    const uint4 h1 = *reinterpret_cast<uint4*>(&hh[4]);
                     uint4* o = reinterpret_cast<uint4*>(g.out_bf16 + (size_t)m * g.ldo + c0);
-                    o[0] = *reinterpret_cast<uint4*>(&hh[0]);
-                    o[1] = *reinterpret_cast<uint4*>(&hh[4]);
+                    if (g.wide) {
+                        stg32(o, h0, h1);
+                    } else {
+                        o[0] = h0;
+                        o[1] = h1;
+                    }
                 }
             }
         }
@@ -379,15 +393,27 @@ __global__ void __launch_bounds__(128) k_wgrad(const WgradArgs g) {
     if (w == 0) tmem_dealloc(tmem, tmem_cols<N>());
 }
 
-__global__ void k_wgrad_reduce(const float* __restrict__ partial, int nparts, int count,
-                               float* __restrict__ out, float scale) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+// Adds the partials: 32 outputs per block (128 bytes of each partial), its
+// eight warps taking every eighth partial, their sums added in warp order.
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partial, int nparts,
+                                                      int count, float* __restrict__ out,
+                                                      float scale) {
+    __shared__ float s_sum[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int b = 0; b < nparts; ++b) s += partial[(size_t)b * count + i];
+    if (i < count) {
+#pragma unroll 8
+        for (int b = w; b < nparts; b += 8) s += partial[(size_t)b * count + i];
+    }
+    s_sum[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || i >= count) return;
+    s = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += s_sum[k][lane];
     out[i] = s * scale;
 }
-
 
 // The network's edge encoder (its two edge layers) in one kernel, per
 // 128-edge tile: tcgen05 MMA 1 (x W1, K = 16: the edge features) into TMEM
@@ -846,7 +872,7 @@ void launch_wgrad_t(const WgradArgs& g, int sms, cudaStream_t st) {
     if (grid > tiles) grid = tiles ? tiles : 1;
     k_wgrad<N><<<grid, 128, smem, st>>>(g);
     const int count = 128 * N;
-    k_wgrad_reduce<<<(count + 255) / 256, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
+    k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
 }
 
 int g_sms = 0;
@@ -863,9 +889,15 @@ int num_sms() {
     return g_sms;
 }
 
-bool launch_linear(int K, int N, const LinearArgs& g, cudaStream_t st) {
+bool launch_linear(int K, int N, const LinearArgs& args, cudaStream_t st) {
     const int sms = num_sms();
-    if (g.M == 0) return true;
+    if (args.M == 0) return true;
+    LinearArgs g = args;
+    // every row and 16-column group that the epilogue touches 32-byte aligned
+    const uintptr_t all = reinterpret_cast<uintptr_t>(g.res) | reinterpret_cast<uintptr_t>(g.gp) |
+                          reinterpret_cast<uintptr_t>(g.gq) | reinterpret_cast<uintptr_t>(g.out_bf16) |
+                          reinterpret_cast<uintptr_t>(g.out_f32);
+    g.wide = all % 32u == 0u && (g.ldr | g.ldo) % 16u == 0u;
     if (K == 16 && N == 128) launch_linear_t<16, 128>(g, sms, st);
     else if (K == 128 && N == 128) launch_linear_t<128, 128>(g, sms, st);
     else if (K == 256 && N == 128) launch_linear_t<256, 128>(g, sms, st);

@@ -39,13 +39,6 @@ struct Layer {
     __nv_bfloat16* W;        // kin x kout (backward operand)
 };
 
-__global__ void k_cast_bf16(const float* __restrict__ in, __nv_bfloat16* __restrict__ out,
-                            size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        out[i] = __float2bfloat16_rn(in[i]);
-}
-
 // W (kin x kout, fp32 row-major) -> bf16 W and bf16 W^T.
 __global__ void k_refresh(const float* __restrict__ w, int kin, int kout, __nv_bfloat16* W,
                           __nv_bfloat16* Wt) {
@@ -234,42 +227,105 @@ __global__ void k_rowsum(uint32_t n, const uint32_t* __restrict__ rowptr, const 
     }
 }
 
-// out[i] += in[i] (fp32), and a bf16 copy of the sum.
-__global__ void k_add_gather(size_t count, float* __restrict__ acc, const float* __restrict__ node,
-                             const uint32_t* __restrict__ src, uint32_t ldn,
-                             __nv_bfloat16* __restrict__ out_bf) {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const size_t e = t / L, c = t % L;
-        float v = acc[t];
-        if (node) v += node[(size_t)src[e] * ldn + c];
-        acc[t] = v;
-        out_bf[t] = __float2bfloat16_rn(v);
+// Column sums: every kernel that reads a matrix by rows for another purpose
+// also adds up its columns where they are wanted.  A block of 256 threads
+// takes rows of C columns with V columns (16 bytes) per thread, 256 V / C rows
+// at a time; a thread sums its columns over the block's rows, the block adds
+// its threads in a fixed order and writes one partial; k_colsum_final adds
+// the partials in a fixed order.  (One column per thread read 2 or 4 bytes a
+// lane: 200 us for 1.27M x 128, a quarter to a half of the copy bandwidth.)
+constexpr uint32_t kColParts = 4 * 152;   // blocks: four per SM
+
+template <int V>
+__device__ __forceinline__ void colsum_block(const float (&s)[V], int C, float* __restrict__ part) {
+    __shared__ float s_sum[256 * V];
+    const int tpr = C / V;                  // threads per row
+#pragma unroll
+    for (int v = 0; v < V; ++v) s_sum[(threadIdx.x / tpr) * C + (threadIdx.x % tpr) * V + v] = s[v];
+    __syncthreads();
+    for (int c = threadIdx.x; c < C; c += 256) {
+        float t = 0.f;
+        for (int r = 0; r < 256 / tpr; ++r) t += s_sum[r * C + c];
+        part[(size_t)blockIdx.x * C + c] = t;
     }
 }
 
-// Column sums of an (M x C) matrix into grad[0:C] (block partials in a fixed
-// order, then one block adds them).
-template <typename T>
-__global__ void k_colsum_part(uint32_t M, int C, const T* __restrict__ in, uint32_t ld,
-                              float* __restrict__ part) {
-    const int c = threadIdx.x;   // blockDim = C
-    float s = 0.f;
-#pragma unroll 8
-    for (uint32_t m = blockIdx.x; m < M; m += gridDim.x) {
-        if constexpr (sizeof(T) == 2) s += __bfloat162float(in[(size_t)m * ld + c]);
-        else s += in[(size_t)m * ld + c];
+__device__ __forceinline__ void unpack_row(const uint4& u, float (&f)[8]) {
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 t = __bfloat1622float2(h[q]);
+        f[2 * q] = t.x;
+        f[2 * q + 1] = t.y;
     }
-    part[(size_t)blockIdx.x * C + c] = s;
 }
 
-__global__ void k_colsum_final(int nparts, int C, const float* __restrict__ part,
-                               float* __restrict__ out, float scale) {
-    const int c = threadIdx.x;
-    if (c >= C) return;
+// Column sums of an (M x C) bf16 matrix, row stride ld (both multiples of 8).
+__global__ void __launch_bounds__(256) k_colsum_bf16(uint32_t M, int C,
+                                                     const __nv_bfloat16* __restrict__ in,
+                                                     uint32_t ld, float* __restrict__ part) {
+    const int tpr = C / 8;
+    const uint32_t rpb = 256 / tpr;
+    const uint32_t col = (threadIdx.x % tpr) * 8, step = gridDim.x * rpb;
+    float s[8] = {};
+#pragma unroll 4
+    for (uint32_t m = blockIdx.x * rpb + threadIdx.x / tpr; m < M; m += step) {
+        float f[8];
+        unpack_row(__ldg(reinterpret_cast<const uint4*>(in + (size_t)m * ld + col)), f);
+#pragma unroll
+        for (int v = 0; v < 8; ++v) s[v] += f[v];
+    }
+    colsum_block<8>(s, C, part);
+}
+
+// The rows of an (M x 128) fp32 matrix: acc += node[src] (with GATHER; row
+// stride ldn), a bf16 copy, and the column sums of the result.
+template <bool GATHER>
+__global__ void __launch_bounds__(256) k_rows_f32(uint32_t M, float* __restrict__ acc,
+                                                  const float* __restrict__ node,
+                                                  const uint32_t* __restrict__ src, uint32_t ldn,
+                                                  __nv_bfloat16* __restrict__ out_bf,
+                                                  float* __restrict__ part) {
+    const uint32_t col = (threadIdx.x & 31) * 4, step = gridDim.x * 8;
+    float s[4] = {};
+#pragma unroll 4
+    for (uint32_t m = blockIdx.x * 8 + threadIdx.x / 32; m < M; m += step) {
+        float4* p = reinterpret_cast<float4*>(acc + (size_t)m * L + col);
+        float4 v = *p;
+        if (GATHER) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(node + (size_t)src[m] * ldn + col));
+            v.x += q.x;
+            v.y += q.y;
+            v.z += q.z;
+            v.w += q.w;
+            *p = v;
+        }
+        const __nv_bfloat162 b0 = __floats2bfloat162_rn(v.x, v.y), b1 = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(out_bf + (size_t)m * L + col) = make_uint2(
+            *reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
+        s[0] += v.x;
+        s[1] += v.y;
+        s[2] += v.z;
+        s[3] += v.w;
+    }
+    colsum_block<4>(s, L, part);
+}
+
+// out[c] = the sum of the partials, 1024 / C slices of them in parallel.
+__global__ void __launch_bounds__(1024) k_colsum_final(int nparts, int C,
+                                                       const float* __restrict__ part,
+                                                       float* __restrict__ out) {
+    __shared__ float s_sum[1024];
+    const int c = threadIdx.x % C, g = threadIdx.x / C, ng = 1024 / C;
     float s = 0.f;
-    for (int b = 0; b < nparts; ++b) s += part[(size_t)b * C + c];
-    out[c] = s * scale;
+#pragma unroll 4
+    for (int b = g; b < nparts; b += ng) s += part[(size_t)b * C + c];
+    s_sum[threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.x >= C) return;
+    float t = 0.f;
+    for (int k = 0; k < ng; ++k) t += s_sum[k * C + c];
+    out[c] = t;
 }
 
 // Loss over fluid nodes and its gradient: out (n x 16 fp32, sorted order),
@@ -681,17 +737,29 @@ void wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
 
 namespace {
 
-void colsum(sur_ctx* c, const void* in, bool bf16, uint32_t M, int C, uint32_t ld, float* out) {
-    const uint32_t parts = M == 0 ? 1u : (M < 1024u ? M : 1024u);
-    if (bf16)
-        k_colsum_part<__nv_bfloat16><<<parts, C, 0, c->st>>>(M, C, (const __nv_bfloat16*)in, ld, c->colpart);
-    else
-        k_colsum_part<float><<<parts, C, 0, c->st>>>(M, C, (const float*)in, ld, c->colpart);
-    k_colsum_final<<<1, C, 0, c->st>>>((int)parts, C, c->colpart, out, 1.f);
+// Blocks of a column-sum pass over M rows, `rpb` rows at a time.
+uint32_t col_parts(uint32_t M, uint32_t rpb) {
+    const uint32_t b = (M + rpb - 1) / rpb;
+    return b == 0 ? 1u : (b < kColParts ? b : kColParts);
 }
 
-void cast(sur_ctx* c, const float* in, __nv_bfloat16* out, size_t n) {
-    k_cast_bf16<<<gridcap(n, 256), 256, 0, c->st>>>(in, out, n);
+// Column sums of an (M x C) bf16 matrix into out[0:C].
+void colsum(sur_ctx* c, const __nv_bfloat16* in, uint32_t M, int C, uint32_t ld, float* out) {
+    const uint32_t parts = col_parts(M, 256 / (C / 8));
+    k_colsum_bf16<<<parts, 256, 0, c->st>>>(M, C, in, ld, c->colpart);
+    k_colsum_final<<<1, 1024, 0, c->st>>>((int)parts, C, c->colpart, out);
+}
+
+// acc (M x 128 fp32) += node[src] when node != null; bf16 copy to out_bf,
+// column sums to out.
+void rows_f32(sur_ctx* c, float* acc, uint32_t M, const float* node, const uint32_t* src,
+              uint32_t ldn, __nv_bfloat16* out_bf, float* out) {
+    const uint32_t parts = col_parts(M, 8);
+    if (node)
+        k_rows_f32<true><<<parts, 256, 0, c->st>>>(M, acc, node, src, ldn, out_bf, c->colpart);
+    else
+        k_rows_f32<false><<<parts, 256, 0, c->st>>>(M, acc, nullptr, nullptr, 0, out_bf, c->colpart);
+    k_colsum_final<<<1, 1024, 0, c->st>>>((int)parts, L, c->colpart, out);
 }
 
 void refresh_all(sur_ctx* c) {
@@ -814,10 +882,10 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
     // decoder
     const Layer* dec = &Ls[4 + 6 * c->NL];
     __nv_bfloat16* h_last = c->XN[c->NL];
-    colsum(c, c->dout, true, n, KOUT, KOUT, c->g + dec[1].b_off);
+    colsum(c, c->dout, n, KOUT, KOUT, c->g + dec[1].b_off);
     wgrad(c, dec[1], c->D1, L, c->dout, KOUT, n);
     if ((rc = linear(c, c->dout, 0, dec[1], true, n, kEpiReluMask, c->D1, L, c->dD1, nullptr, L))) return rc;
-    colsum(c, c->dD1, true, n, L, L, c->g + dec[0].b_off);
+    colsum(c, c->dD1, n, L, L, c->g + dec[0].b_off);
     wgrad(c, dec[0], h_last, 2 * L, c->dD1, L, n);
     if ((rc = linear(c, c->dD1, 0, dec[0], true, n, kEpiNone, nullptr, 0, nullptr, c->dH, L))) return rc;
     cudaMemsetAsync(c->dE, 0, (size_t)E * L * sizeof(float), st);
@@ -828,22 +896,19 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         __nv_bfloat16* z1 = c->Z1[l];
         __nv_bfloat16* y1 = c->Y1[l];
         // node update h' = h + W4 relu(W3 [h, agg] + b3) + b4
-        cast(c, c->dH, c->dHb, (size_t)n * L);
-        colsum(c, c->dH, false, n, L, L, c->g + w[5].b_off);
+        rows_f32(c, c->dH, n, nullptr, nullptr, 0, c->dHb, c->g + w[5].b_off);
         wgrad(c, w[5], y1, L, c->dHb, L, n);
         if ((rc = linear(c, c->dHb, 0, w[5], true, n, kEpiReluMask, y1, L, c->dY1, nullptr, L))) return rc;
-        colsum(c, c->dY1, true, n, L, L, c->g + w[4].b_off);
+        colsum(c, c->dY1, n, L, L, c->g + w[4].b_off);
         wgrad(c, w[4], xn_cur, 2 * L, c->dY1, L, n, 0);
         wgrad(c, w[4], xn_cur + L, 2 * L, c->dY1, L, n, 1);
         if ((rc = linear(c, c->dY1, 0, w[4], true, n, kEpiNone, nullptr, 0, nullptr, c->dXN, 2 * L))) return rc;
         k_add_strided<<<nblk((size_t)n * L, 256), 256, 0, st>>>(n, c->dH, c->dXN, 2 * L);
         // aggregation and edge update e' = e + W2 relu(pre) + b2
-        k_add_gather<<<gridcap((size_t)E * L, 256), 256, 0, st>>>((size_t)E * L, c->dE, c->dXN + L,
-                                                                  c->src, 2 * L, c->dEb);
-        colsum(c, c->dE, false, E, L, L, c->g + w[3].b_off);
+        rows_f32(c, c->dE, E, c->dXN + L, c->src, 2 * L, c->dEb, c->g + w[3].b_off);
         wgrad(c, w[3], z1, L, c->dEb, L, E);
         if ((rc = linear(c, c->dEb, 0, w[3], true, E, kEpiReluMask, z1, L, c->dpre, nullptr, L))) return rc;
-        colsum(c, c->dpre, true, E, L, L, c->g + w[2].b_off);
+        colsum(c, c->dpre, E, L, L, c->g + w[2].b_off);
         wgrad(c, w[2], e_in, L, c->dpre, L, E);
         if ((rc = linear(c, c->dpre, 0, w[2], true, E, kEpiAccum, nullptr, 0, nullptr, c->dE, L))) return rc;
         // pre = W1a h_i + W1b h_j + ...: sums over the edges of i and of j
@@ -857,17 +922,15 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         if ((rc = linear(c, c->dQb, 0, w[1], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
     }
     // encoders
-    cast(c, c->dE, c->dEb, (size_t)E * L);
-    colsum(c, c->dE, false, E, L, L, c->g + Ls[3].b_off);
+    rows_f32(c, c->dE, E, nullptr, nullptr, 0, c->dEb, c->g + Ls[3].b_off);
     wgrad(c, Ls[3], c->ee1, L, c->dEb, L, E);
     if ((rc = linear(c, c->dEb, 0, Ls[3], true, E, kEpiReluMask, c->ee1, L, c->dEe1, nullptr, L))) return rc;
-    colsum(c, c->dEe1, true, E, L, L, c->g + Ls[2].b_off);
+    colsum(c, c->dEe1, E, L, L, c->g + Ls[2].b_off);
     wgrad(c, Ls[2], c->xe, KIN, c->dEe1, L, E);
-    cast(c, c->dH, c->dHb, (size_t)n * L);
-    colsum(c, c->dH, false, n, L, L, c->g + Ls[1].b_off);
+    rows_f32(c, c->dH, n, nullptr, nullptr, 0, c->dHb, c->g + Ls[1].b_off);
     wgrad(c, Ls[1], c->en1, L, c->dHb, L, n);
     if ((rc = linear(c, c->dHb, 0, Ls[1], true, n, kEpiReluMask, c->en1, L, c->dEn1, nullptr, L))) return rc;
-    colsum(c, c->dEn1, true, n, L, L, c->g + Ls[0].b_off);
+    colsum(c, c->dEn1, n, L, L, c->g + Ls[0].b_off);
     wgrad(c, Ls[0], c->xn, KIN, c->dEn1, L, n);
     if (loss_host) {
         cudaMemcpyAsync(loss_host, c->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
