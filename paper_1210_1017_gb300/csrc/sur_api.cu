@@ -96,7 +96,7 @@ int sur_edge_encoder(const void* X, const void* W1t, const void* W2t, const floa
     g.M = M;
     g.Z = static_cast<__nv_bfloat16*>(Z);
     g.Eout = static_cast<__nv_bfloat16*>(Eout);
-    launch_edge_encoder(g, static_cast<cudaStream_t>(stream));
+    if (!launch_edge_encoder(g, static_cast<cudaStream_t>(stream))) return SPH_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 

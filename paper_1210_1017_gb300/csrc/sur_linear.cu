@@ -416,32 +416,40 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
 }
 
 // The network's edge encoder (its two edge layers) in one kernel, per
-// 128-edge tile: tcgen05 MMA 1 (x W1, K = 16: the edge features) into TMEM
-// columns [0, 128); the first epilogue writes z = relu(acc + b1) as the
-// K-major A operand of MMA 2 in shared memory (and to global memory for the
-// backward pass); MMA 2 (z W2) into columns [128, 256); the second epilogue
-// writes e0 = acc + b2.  z never reaches HBM in inference.  The x tile is
-// double-buffered (the next tile's copies in flight during this one).  256
-// threads, two blocks per SM (76 KB of shared memory and 256 TMEM columns
-// each): the two warps that share a TMEM lane quarter split the columns.
+// 128-edge tile: tcgen05 MMA 1 (x W1, K = 16: the edge features) into X; the
+// first epilogue writes z = relu(acc + b1) to TMEM as MMA 2's A operand (and to
+// global memory for the backward pass); MMA 2 (z W2) back into X; the second
+// epilogue writes e0 = acc + b2 to shared memory in the 128-byte swizzle, from
+// where it is stored by TMA.  z never reaches HBM in inference.  X and Y are the
+// halves of 256 TMEM columns and change roles from tile to tile, so MMA 1 of
+// the next tile runs under this tile's second epilogue.  Bound by HBM: 32 B of
+// features in, 256 B out (512 with Z); row stores by thread held the L1 at one
+// line per clock.  256 threads, two blocks per SM (77 KB of shared memory): the
+// two warps that share a TMEM lane quarter split the columns.
 constexpr int kEncK = 16;
-constexpr size_t kEncSmem = (size_t)128 * kEncK * 2 * 3 + (size_t)128 * 128 * 2 * 2;   // W1, 2 x x; W2, z
+constexpr uint32_t kETile = 128 * 128 * 2;                  // bytes of a 128 x 128 bf16 tile
+// e0 and W2, then W1 and two x tiles; alignment
+constexpr size_t kEncSmem = (size_t)2 * kETile + (size_t)128 * kEncK * 2 * 3 + 1024;
 
-__global__ void __launch_bounds__(256, 2) k_edge_encoder(const EdgeArgs g) {
-    constexpr int K1 = kEncK, N = 128, NT = 256, CW = 64;   // CW: epilogue columns per thread
-    constexpr uint32_t T = 128 * 128 * 2;          // bytes of one 128 x 128 bf16 tile
+__global__ void __launch_bounds__(256, 2)
+    k_edge_encoder(const EdgeArgs g, const __grid_constant__ CUtensorMap map_out, const bool wide) {
+    constexpr int K1 = kEncK, N = 128, NT = 256;
+    constexpr uint32_t T = kETile, BOX = T / 2;
     constexpr uint32_t T1 = 128 * K1 * 2;          // bytes of one 128 x K1 tile
-    extern __shared__ __align__(128) unsigned char s_raw[];
-    unsigned char* sw1 = s_raw;                    // W1^T, N x K1
-    unsigned char* sw2 = sw1 + T1;                 // W2^T, N x N
-    unsigned char* sz = sw2 + T;                   // z tile
-    unsigned char* sa0 = sz + T;                   // 2 x x tile
+    extern __shared__ unsigned char s_dyn[];
+    unsigned char* so = s_dyn + ((1024u - (sm_addr(s_dyn) & 1023u)) & 1023u);   // e0 tile
+    unsigned char* sw2 = so + T;                   // W2^T, N x N
+    unsigned char* sw1 = sw2 + T;                  // W1^T, N x K1
+    unsigned char* sx0 = sw1 + T1;                 // 2 x x tile
     __shared__ __align__(16) float s_b1[128], s_b2[128];
-    __shared__ __align__(8) uint64_t s_bar;
+    __shared__ __align__(8) uint64_t s_bar[2];     // MMA 1, MMA 2
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     if (w == 0) tmem_alloc(&s_tmem, 256);
-    if (tid == 0) mbar_init1(&s_bar);
+    if (tid == 0) {
+        mbar_init1(&s_bar[0]);
+        mbar_init1(&s_bar[1]);
+    }
     const uint32_t ntiles = (g.M + 127) / 128;
     for (int c = tid; c < N * (K1 / 8); c += NT) {
         const int r = c % N, gk = c / N;
@@ -455,106 +463,128 @@ __global__ void __launch_bounds__(256, 2) k_edge_encoder(const EdgeArgs g) {
         s_b1[tid] = g.b1[tid];
         s_b2[tid] = g.b2[tid];
     }
-    if (blockIdx.x < ntiles) issue_rows<K1, NT>(sa0, g.E, blockIdx.x * 128, g.M, K1);
+    uint32_t tile = blockIdx.x;
+    if (tile < ntiles) issue_rows<K1, NT>(sx0, g.E, tile * 128, g.M, K1);
     cp_async_commit();
+    cp_async_wait_all();
+    fence_async_shared();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     const int wq = w & 3, part = w >> 2;                 // lane quarter, column half
-    const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
-    uint32_t phase = 0, buf = 0;
-    bool ok = true;
-    for (uint32_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, buf ^= 1u) {
-        unsigned char* sa = sa0 + buf * T1;
-        cp_async_wait_all();                       // x of this tile (and the weights)
-        fence_async_shared();
-        __syncthreads();
-        if (tid == 0) {
-            tc_fence_after();
-#pragma unroll
-            for (int s = 0; s < K1 / 16; ++s) {
-                const uint64_t ad = smem_desc(sm_addr(sa) + s * 256, kLBO, (K1 / 8) * 128);
-                const uint64_t bd = smem_desc(sm_addr(sw1) + s * 256, kLBO, (K1 / 8) * 128);
-                tc_mma(tmem, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
-            }
-            tc_commit(&s_bar);
-        }
-        // the next tile's x into the other buffer (its last reader, the
-        // previous tile's MMA 1, has completed)
-        const uint32_t next = tile + gridDim.x;
-        if (next < ntiles) issue_rows<K1, NT>(sa0 + (buf ^ 1u) * T1, g.E, next * 128, g.M, K1);
-        cp_async_commit();
-        const int r = wq * 32 + lane;              // this thread's row of the tile
-        const uint32_t m = tile * 128 + r;
-        const bool valid = m < g.M;
-        bool got = mbar_wait(&s_bar, phase);
-        ok = __syncthreads_and(got) != 0;
-        if (!ok) break;
-        phase ^= 1u;
+    const uint32_t quarter = (uint32_t)(wq * 32) << 16;
+    const int r = wq * 32 + lane;                        // this thread's row of a tile
+    auto mma1 = [&](const unsigned char* sx, uint32_t d) {
         tc_fence_after();
-        // epilogue 1: z = relu(acc + b1) -> shared (MMA 2) and global
-#pragma unroll 2
-        for (int c0 = part * CW; c0 < part * CW + CW; c0 += 16) {
+        tc_mma(d, smem_desc(sm_addr(sx), kLBO, (K1 / 8) * 128),
+               smem_desc(sm_addr(sw1), kLBO, (K1 / 8) * 128), idesc_bf16(N), 0u);
+        tc_commit(&s_bar[0]);
+    };
+    uint32_t phase = 0, x = 0, buf = 0;                  // x: column offset of X (0 or 128)
+    bool ok = true;
+    if (tile < ntiles && tid == 0) mma1(sx0, tmem);
+    for (; tile < ntiles; tile += gridDim.x) {
+        const uint32_t m = tile * 128 + (uint32_t)r;
+        const uint32_t next = tile + gridDim.x;
+        // the next tile's x into the other buffer (its last reader, MMA 1 of
+        // the tile before, has completed)
+        if (next < ntiles) issue_rows<K1, NT>(sx0 + (buf ^ 1u) * T1, g.E, next * 128, g.M, K1);
+        cp_async_commit();
+        bool got = mbar_wait(&s_bar[0], phase);          // MMA 1
+        tc_fence_after();
+        // epilogue 1: z = relu(acc + b1) into Y, and to Z
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c0 = part * 64 + 16 * k;
             float v[16];
-            tmem_ld16(lane_base + c0, v);
-            const float2* b2v = reinterpret_cast<const float2*>(s_b1 + c0);
-            __nv_bfloat162 hh[8];
+            tmem_ld16(tmem + x + quarter + c0, v);
+            const float4* b4 = reinterpret_cast<const float4*>(s_b1 + c0);
+            uint32_t z[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]), b2v[q]);
-                hh[q] = __floats2bfloat162_rn(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+                const float4 bb = b4[q >> 1];
+                const float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]),
+                                            q & 1 ? make_float2(bb.z, bb.w) : make_float2(bb.x, bb.y));
+                // rounding and the maximum with 0 commute
+                const __nv_bfloat162 zz =
+                    __hmax2(__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(0.f, 0.f));
+                z[q] = *reinterpret_cast<const uint32_t*>(&zz);
             }
-            const uint4 z0 = *reinterpret_cast<uint4*>(&hh[0]);
-            const uint4 z1 = *reinterpret_cast<uint4*>(&hh[4]);
-            *reinterpret_cast<uint4*>(sz + kmajor_offset(r, c0, N)) = z0;
-            *reinterpret_cast<uint4*>(sz + kmajor_offset(r, c0 + 8, N)) = z1;
-            if (g.Z && valid) {
+            tmem_st8(tmem + (x ^ 128u) + quarter + (uint32_t)(c0 / 2), z);
+            if (g.Z && m < g.M) {
                 uint4* o = reinterpret_cast<uint4*>(g.Z + (size_t)m * N + c0);
-                o[0] = z0;
-                o[1] = z1;
+                const uint4 z0 = make_uint4(z[0], z[1], z[2], z[3]);
+                const uint4 z1 = make_uint4(z[4], z[5], z[6], z[7]);
+                if (wide) {
+                    stg32(o, z0, z1);
+                } else {
+                    o[0] = z0;
+                    o[1] = z1;
+                }
             }
         }
+        tmem_st_wait();
+        cp_async_wait_all();                             // the next tile's x
+        if (tid == 32) bulk_wait_read();                 // the e0 tile has been read
         fence_async_shared();
         tc_fence_before();
-        __syncthreads();                           // z complete
+        ok = __syncthreads_and(got) != 0;                // z and the next x complete
+        if (!ok) break;
         if (tid == 0) {
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < N / 16; ++s) {
-                const uint64_t ad = smem_desc(sm_addr(sz) + s * 256, kLBO, (N / 8) * 128);
                 const uint64_t bd = smem_desc(sm_addr(sw2) + s * 256, kLBO, (N / 8) * 128);
-                tc_mma(tmem + 128, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
+                tc_mma_ta(tmem + x, tmem + (x ^ 128u) + s * 8, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
             }
-            tc_commit(&s_bar);
+            tc_commit(&s_bar[1]);
         }
-        got = mbar_wait(&s_bar, phase);
-        ok = __syncthreads_and(got) != 0;
-        if (!ok) break;
-        phase ^= 1u;
+        got = mbar_wait(&s_bar[1], phase);               // MMA 2
         tc_fence_after();
+        // z has been read: MMA 1 of the next tile over it
+        if (got && tid == 0 && next < ntiles) mma1(sx0 + (buf ^ 1u) * T1, tmem + (x ^ 128u));
         // epilogue 2: e0 = acc + b2
-#pragma unroll 2
-        for (int c0 = part * CW; c0 < part * CW + CW; c0 += 16) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c0 = part * 64 + 16 * k;
             float v[16];
-            tmem_ld16(lane_base + 128 + c0, v);
-            if (!valid) continue;
-            const float2* b2v = reinterpret_cast<const float2*>(s_b2 + c0);
+            tmem_ld16(tmem + x + quarter + c0, v);
+            const float4* b4 = reinterpret_cast<const float4*>(s_b2 + c0);
             __nv_bfloat162 hh[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]), b2v[q]);
+                const float4 bb = b4[q >> 1];
+                const float2 a = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]),
+                                            q & 1 ? make_float2(bb.z, bb.w) : make_float2(bb.x, bb.y));
                 hh[q] = __floats2bfloat162_rn(a.x, a.y);
             }
-            uint4* o = reinterpret_cast<uint4*>(g.Eout + (size_t)m * N + c0);
-            o[0] = *reinterpret_cast<uint4*>(&hh[0]);
-            o[1] = *reinterpret_cast<uint4*>(&hh[4]);
+            *reinterpret_cast<uint4*>(so + part * BOX + sw128_offset(r, 2 * k)) =
+                *reinterpret_cast<uint4*>(&hh[0]);
+            *reinterpret_cast<uint4*>(so + part * BOX + sw128_offset(r, 2 * k + 1)) =
+                *reinterpret_cast<uint4*>(&hh[4]);
         }
+        fence_async_shared();
         tc_fence_before();
-        __syncthreads();
+        ok = __syncthreads_and(got) != 0;                // X free, e0 complete
+        if (!ok) break;
+        if (tid == 32) {
+            tma_store(&map_out, so, 0, (int)(tile * 128));
+            tma_store(&map_out, so + BOX, 64, (int)(tile * 128));
+            bulk_commit();
+        }
+        x ^= 128u;
+        buf ^= 1u;
+        phase ^= 1u;
     }
-    if (!ok && tid == 0 && g.status) atomicOr(g.status, 1u);
+    if (!ok) {
+        if (tid == 0 && g.status) atomicOr(g.status, 1u);
+        mbar_wait(&s_bar[0], phase);                     // let an MMA in flight land first
+        mbar_wait(&s_bar[1], phase);
+    }
+    if (tid == 32) bulk_wait();
     cp_async_wait_all();
+    tc_fence_before();
     __syncthreads();
     if (w == 0) tmem_dealloc(tmem, 256);
 }
@@ -594,7 +624,6 @@ __device__ __forceinline__ bool half_and(int h, bool v) {
 // epilogue.  On one GB300, with Z, 1.5M edges: 572 us with the loads issued at
 // the end of a tile, 466 with z in TMEM and the loads ahead, 300 with the
 // tiles by TMA (3.9 TB/s of e, e' and z, 57% of the copy bandwidth).
-constexpr uint32_t kETile = 128 * 128 * 2;                  // bytes of one e tile
 constexpr size_t kEdgePPSmem = (size_t)6 * kETile + 1024;   // W1c, W2, 2 x 2 e tiles; alignment
 
 __global__ void __launch_bounds__(512, 1)
@@ -959,17 +988,19 @@ bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st) {
 }
 
 // The encoder: two 256-thread blocks per SM.
-void launch_edge_encoder(const EdgeArgs& g, cudaStream_t st) {
-    static bool init = false;
-    if (!init) {
+bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st) {
+    static std::once_flag once;
+    std::call_once(once, [] {
         cudaFuncSetAttribute(k_edge_encoder, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncSmem);
-        init = true;
-    }
-    if (g.M == 0) return;
+    });
+    if (g.M == 0) return true;
+    CUtensorMap map_out;
+    if (!tile_map(&map_out, g.Eout, g.M)) return false;
     const uint32_t tiles = (g.M + 127) / 128;
     uint32_t grid = (uint32_t)(num_sms() * 2);
     if (grid > tiles) grid = tiles;
-    k_edge_encoder<<<grid, 256, kEncSmem, st>>>(g);
+    k_edge_encoder<<<grid, 256, kEncSmem, st>>>(g, map_out, reinterpret_cast<uintptr_t>(g.Z) % 32u == 0u);
+    return true;
 }
 
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st) {

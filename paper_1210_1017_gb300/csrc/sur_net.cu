@@ -691,7 +691,7 @@ int edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16
 
 // The two edge-encoder layers in one kernel: e0 = relu(xe W + b) W' + b'
 // (the hidden activation kept for the backward pass when z != null).
-void edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z, __nv_bfloat16* e0) {
+int edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z, __nv_bfloat16* e0) {
     EdgeArgs g = {};
     g.E = c->xe;
     g.W1t = l1.Wt;
@@ -701,7 +701,8 @@ void edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z
     g.M = c->E;
     g.Z = z;
     g.Eout = e0;
-    launch_edge_encoder(g, c->st);
+    if (!launch_edge_encoder(g, c->st)) return fail(c, SPH_ERR_CUDA, "edge encoder: no tensor maps");
+    return SPH_OK;
 }
 
 // grad of W (kin x kout) += X^T dY over M rows (X: M x kin with stride ldx,
@@ -827,7 +828,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
     // encoders
     if ((rc = linear(c, c->xn, 0, Ls[0], false, n, kEpiRelu, nullptr, 0, c->en1, nullptr, L))) return rc;
     if ((rc = linear(c, c->en1, 0, Ls[1], false, n, kEpiNone, nullptr, 0, c->XN[0], nullptr, 2 * L))) return rc;
-    edge_encoder(c, Ls[2], Ls[3], train ? c->ee1 : nullptr, c->Ebuf[0]);
+    if ((rc = edge_encoder(c, Ls[2], Ls[3], train ? c->ee1 : nullptr, c->Ebuf[0]))) return rc;
     // message passing
     for (int l = 0; l < c->NL; ++l) {
         __nv_bfloat16* xn_cur = c->XN[train ? l : l % 2];
