@@ -381,7 +381,7 @@ int sph_read_array(sph_ctx *ctx, int which, void *host, uint64_t bytes);
  * capacity < m returns SPH_ERR_CAPACITY with counts filled and nothing
  * copied.  The state itself is not reordered (the cell order stays).
  * Needs built cells and a single simulation (SPH_ERR_STATE otherwise).
- * Sync; a radix-sort look-back that gave up shows in sph_check. */
+ * Sync. */
 #define SPH_SUBDOMAIN_EDGE     0
 #define SPH_SUBDOMAIN_MIGRATE  1
 int sph_subdomain_select(sph_ctx *ctx, int mode, double xlo, double xhi,
@@ -416,11 +416,11 @@ int sph_check(sph_ctx *ctx);
 int sph_clear_status(sph_ctx *ctx);
 
 /* Self-test of the failure path; the paper has no counterpart.  Bounded
- * device waits must be testable without hanging a GPU: this runs the radix
- * sort's decoupled look-back (the same device code as the sort) against a
- * predecessor tile whose status nothing ever publishes, with a limit of
+ * device waits must be testable without hanging a GPU: this runs the
+ * decoupled look-back of the cell sort's scan (the same device code) against
+ * a predecessor tile whose word nothing ever publishes, with a limit of
  * `polls` polls (1 to 2^20).  The wait gives up and sets SPH_STATUS_TIMEOUT
- * in the context's status word, as a stalled sort would, so sph_check
+ * in the context's status word, as a stalled scan would, so sph_check
  * returns SPH_ERR_TIMEOUT.  The particle state and cells are untouched (the
  * look-back runs on status words reserved for this test).  Sync. */
 int sph_selftest_timeout(sph_ctx *ctx, uint32_t polls);
@@ -476,8 +476,8 @@ const char *sph_last_error(const sph_ctx *ctx);
 void sph_destroy(sph_ctx *ctx);
 
 /* Sec. 3.1 / Sec. 4.3: stable LSD radix sort of (key, value) pairs by the
- * low key_bits bits of the key (8 bits per pass, onesweep with decoupled
- * look-back).  Equal keys keep their input order, so sorting labels whose
+ * low key_bits bits of the key (8 bits per pass; its kernels do not wait on
+ * one another).  Equal keys keep their input order, so sorting labels whose
  * values are ids in ascending order reproduces the (label, id) order of the
  * paper's example.  d_vals_in may be NULL: values are then the input
  * indices 0..n-1.  All arrays are device arrays of n uint32; outputs must
@@ -490,16 +490,16 @@ int sph_radix_sort_pairs(const uint32_t *d_keys_in, const uint32_t *d_vals_in,
                          uint64_t scratch_bytes, void *stream);
 
 /* Outcome of the last sph_radix_sort_pairs call of n pairs on d_scratch:
- * waits for stream, then SPH_OK, or SPH_ERR_TIMEOUT if a decoupled look-back
- * wait gave up (its bounded spin ran out; the order is then not valid).
+ * waits for stream, then SPH_OK, or SPH_ERR_TIMEOUT if a bounded device wait
+ * on d_scratch gave up (the sort itself has none: the self-test below).
  * Each sort clears the flag before it starts.  Arguments as for the sort
  * (n >= 1).  Sync. */
 int sph_radix_sort_status(const void *d_scratch, uint64_t scratch_bytes,
                           uint32_t n, void *stream);
 
 /* Self-test of that failure path; the paper has no counterpart.  Runs the
- * sort's look-back on d_scratch (laid out for n pairs) against a
- * predecessor tile whose status nothing publishes, with a limit of `polls`
+ * library's look-back on d_scratch (laid out for n pairs) against a
+ * predecessor tile whose word nothing publishes, with a limit of `polls`
  * polls (1 to 2^20), so the wait gives up and the next
  * sph_radix_sort_status reports SPH_ERR_TIMEOUT.  Sync. */
 int sph_radix_sort_selftest_timeout(void *d_scratch, uint64_t scratch_bytes,
@@ -511,7 +511,7 @@ int sph_radix_sort_selftest_timeout(void *d_scratch, uint64_t scratch_bytes,
  * device memory belongs to another allocator's pool, or a latency-critical
  * loop that must not call cudaMalloc/cudaFree (they can synchronise the
  * device).  The scratch lives in a fixed array inside libsph.so, about
- * 9.4 MB per device: it is reserved on every device whose context loads the
+ * 8.7 MB per device: it is reserved on every device whose context loads the
  * library's module, whether or not this entry point is ever called, and
  * held until the process exits; nothing is allocated per call.  Limits and
  * behaviour:
@@ -523,8 +523,8 @@ int sph_radix_sort_selftest_timeout(void *d_scratch, uint64_t scratch_bytes,
  *     any stream capture.  The address is kept for the life of the process:
  *     after cudaDeviceReset (or any teardown of the device's primary
  *     context) it is stale, so do not use this entry point after one
- *   - a look-back wait that gave up is reported by
- *     sph_radix_sort_static_status, not by the return value
+ *   - sph_radix_sort_static_status reports a wait that gave up, as
+ *     sph_radix_sort_status does
  *   - all calls on one device share the array and it keeps the last call's
  *     contents (each call clears what must start at zero); calls that overlap
  *     on the GPU race, so serialise them (e.g. one stream)
@@ -536,8 +536,8 @@ int sph_radix_sort_pairs_static(const uint32_t *d_keys_in,
                                 uint32_t n, uint32_t key_bits, void *stream);
 
 /* Outcome of the last sph_radix_sort_pairs_static call on the current
- * device: waits for stream, then SPH_OK or SPH_ERR_TIMEOUT (a look-back
- * wait gave up; the order is then not valid).  Reads the fixed array; the
+ * device: waits for stream, then SPH_OK or SPH_ERR_TIMEOUT (a bounded wait on
+ * the array gave up: the self-test below).  Reads the fixed array; the
  * same first-call and overlap rules apply.  Sync. */
 int sph_radix_sort_static_status(void *stream);
 

@@ -224,7 +224,6 @@ size_t carve(sph_ctx* c, void* base, uint32_t n, const Table& t, int passes) {
     c->cscan_words = cv.take<unsigned long long>(scan_bsum_count(t.ncells + 1));
     c->cscan_ctl = cv.take<uint32_t>(2);
     c->hist = cv.take<uint32_t>(4 * 256);
-    const uint32_t tiles = os_tiles(n);
     (void)passes;
     // status words the failure-path self-test runs its look-back against
     c->os_bytes = 4 * sizeof(uint32_t) + 256 * sizeof(uint32_t);
@@ -234,10 +233,10 @@ size_t carve(sph_ctx* c, void* base, uint32_t n, const Table& t, int passes) {
         c->sub_key[b] = cv.take<uint32_t>(n);
         c->sub_val[b] = cv.take<uint32_t>(n);
     }
-    c->sub_hist = cv.take<uint32_t>(5 * 256);
-    c->sub_os_bytes = 5 * sizeof(uint32_t) + (size_t)5 * tiles * 256 * sizeof(uint32_t);
-    c->sub_os = cv.take<uint32_t>(c->sub_os_bytes / sizeof(uint32_t));
-    c->sub_cnt = cv.take<uint32_t>(4);
+    c->sub_os = cv.take<uint32_t>(radix_sort_words(n));
+    c->sub_cnt = cv.take<uint32_t>(8);
+    c->sub_bits = cv.take<uint32_t>(2 * (((size_t)n + 31) / 32));
+    c->sub_bsum = cv.take<uint32_t>(sub_bit_blocks(n));
     c->csum = cv.take<uint32_t>(t.ncells + t.nrows + 1);
     c->ucnt = cv.take<uint32_t>(t.nrows + 1);
     c->uoff = cv.take<uint32_t>(t.nrows + 2);
@@ -1059,7 +1058,7 @@ int sph_check(sph_ctx* c) {
     rc = cuda_check(c, cudaStreamSynchronize(c->st), "check sync");
     if (rc) return rc;
     if (status & SPH_STATUS_TIMEOUT)
-        return fail(c, SPH_ERR_TIMEOUT, "a bounded device wait gave up (radix-sort look-back or staging copy)");
+        return fail(c, SPH_ERR_TIMEOUT, "a bounded device wait gave up (scan look-back or staging copy)");
     if (status & SPH_STATUS_NONFINITE) return fail(c, SPH_ERR_NONFINITE, "non-finite interaction result");
     if (status & SPH_STATUS_CAPACITY) return fail(c, SPH_ERR_CAPACITY, "a cell exceeded the id tie-break capacity");
     if (status & SPH_STATUS_BOUNDS)
@@ -1375,8 +1374,7 @@ uint64_t sph_radix_sort_scratch_bytes(uint32_t n) {
     Carver cv(nullptr);
     cv.take<uint32_t>(n);       // temporary keys
     cv.take<uint32_t>(n);       // temporary values
-    cv.take<uint32_t>(4 * 256); // digit histograms
-    cv.take<uint32_t>(4 + (size_t)4 * os_tiles(n) * 256);   // tile counters + status
+    cv.take<uint32_t>(radix_sort_words(n));   // tile counts, digit totals
     cv.take<uint32_t>(1);       // error word
     return (cv.used + kAlign - 1) / kAlign * kAlign;
 }
@@ -1393,26 +1391,10 @@ int sph_radix_sort_pairs(const uint32_t* kin, const uint32_t* vin, uint32_t* kou
     Carver cv(scratch);
     uint32_t* tk = cv.take<uint32_t>(n);
     uint32_t* tv = cv.take<uint32_t>(n);
-    uint32_t* hist = cv.take<uint32_t>(4 * 256);
-    const uint32_t tiles = os_tiles(n);
-    uint32_t* tilectr = cv.take<uint32_t>(4 + (size_t)4 * tiles * 256);
+    uint32_t* words = cv.take<uint32_t>(radix_sort_words(n));
     uint32_t* err = cv.take<uint32_t>(1);
-    const int passes = ((int)key_bits + 7) / 8;
-    cudaMemsetAsync(hist, 0, 4 * 256 * sizeof(uint32_t), st);
-    cudaMemsetAsync(tilectr, 0, (4 + (size_t)passes * tiles * 256) * sizeof(uint32_t), st);
     cudaMemsetAsync(err, 0, sizeof(uint32_t), st);
-    launch_digit_hist(kin, n, passes, (int)key_bits, hist, st);
-    // ping-pong so that the last pass lands in the outputs
-    const uint32_t* ck = kin;
-    const uint32_t* cv_ = vin;
-    for (int p = 0; p < passes; ++p) {
-        const bool to_out = ((passes - 1 - p) % 2) == 0;
-        uint32_t* ok = to_out ? kout : tk;
-        uint32_t* ov = to_out ? vout : tv;
-        launch_onesweep_pass(ck, cv_, ok, ov, n, p, (int)key_bits, hist, tilectr + 4, tilectr, err, st);
-        ck = ok;
-        cv_ = ov;
-    }
+    launch_radix_sort(kin, vin, kout, vout, tk, tv, n, (int)key_bits, words, st);
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 
@@ -1421,8 +1403,7 @@ static uint32_t* sort_err_word(void* scratch, uint32_t n) {
     Carver cv(scratch);
     cv.take<uint32_t>(n);
     cv.take<uint32_t>(n);
-    cv.take<uint32_t>(4 * 256);
-    cv.take<uint32_t>(4 + (size_t)4 * os_tiles(n) * 256);
+    cv.take<uint32_t>(radix_sort_words(n));
     return cv.take<uint32_t>(1);
 }
 
@@ -1455,13 +1436,11 @@ int sph_radix_sort_selftest_timeout(void* d_scratch, uint64_t scratch_bytes, uin
     Carver cv(d_scratch);
     cv.take<uint32_t>(n);
     cv.take<uint32_t>(n);
-    cv.take<uint32_t>(4 * 256);
-    uint32_t* tilectr = cv.take<uint32_t>(4 + (size_t)4 * os_tiles(n) * 256);
+    uint32_t* words = cv.take<uint32_t>(radix_sort_words(n));
     uint32_t* err = cv.take<uint32_t>(1);
     cudaMemsetAsync(err, 0, sizeof(uint32_t), st);
-    // tile 1 of the first pass waits on tile 0's status words, zeroed here
-    // and published by nobody
-    launch_lookback_selftest(tilectr + 4, polls, err, st);
+    // a look-back of tile 1 on tile 0's word, zeroed here and published by nobody
+    launch_lookback_selftest(words, polls, err, st);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return SPH_ERR_CUDA;
     return SPH_OK;

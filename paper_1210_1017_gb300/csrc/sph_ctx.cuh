@@ -57,13 +57,12 @@ struct sph_ctx {
     uint4* part_u;
     uint32_t *done, *status;
     uint32_t* id_flag;       // set by the upload when some id >= n
-    // sub-domain selection (Sec. 4.3): ping-pong (key, value) arrays of the
-    // selected particles for the radix sorts, their digit histograms (4
-    // passes by id + 1 by label), tile counters and look-back status, and
-    // the label counters
+    // sub-domain selection (Sec. 4.3): counters; bit maps of the selected ids
+    // per label and their block sums (dense ids; sub_val[0] then maps ids to
+    // state indexes); ping-pong (key, value) arrays of the selected particles
+    // and the words of their radix sorts (other ids)
     uint32_t *sub_key[2], *sub_val[2];
-    uint32_t *sub_hist, *sub_os, *sub_cnt;
-    size_t sub_os_bytes = 0;
+    uint32_t *sub_os, *sub_cnt, *sub_bits, *sub_bsum;
     double *diag_out, *diag_part;
     unsigned long long* front;   // per-member front images (sph_front)
     unsigned long long* counters;

@@ -142,17 +142,24 @@ constexpr int kOsThreads = 256;
 constexpr int kOsItems = 16;
 constexpr int kOsTile = kOsThreads * kOsItems;
 inline uint32_t os_tiles(uint32_t n) { return (n + kOsTile - 1) / kOsTile; }
-void launch_digit_hist(const uint32_t* keys, uint32_t n, int passes, int bits_total,
-                       uint32_t* hist, cudaStream_t st);
-// Failure-path self-test: the radix sort's look-back waits on 256 status
-// words that nothing sets (zeroed here) and gives up after `limit` polls,
-// setting kStatusTimeout in *err.
-void launch_lookback_selftest(uint32_t* zeroed256, uint32_t limit, uint32_t* err,
-                              cudaStream_t st);
-void launch_onesweep_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
-                          uint32_t* vout, uint32_t n, int pass, int bits_total,
-                          const uint32_t* hist, uint32_t* status, uint32_t* tilectr,
-                          uint32_t* err, cudaStream_t st);
+// Failure-path self-test: a scan's look-back waits on a word that nothing sets
+// (zeroed here, 16 bytes) and gives up after `limit` polls, setting
+// kStatusTimeout in *err.
+void launch_lookback_selftest(uint32_t* zeroed, uint32_t limit, uint32_t* err, cudaStream_t st);
+// Stable sort of n pairs by the low key_bits bits of the key (vin null: the
+// values are the input indexes).  tk, tv: n temporaries (used by more than
+// one digit place); words: radix_sort_words(n) words without initial contents.
+// Its kernels do not wait on one another.
+size_t radix_sort_words(uint32_t n);
+void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
+                       uint32_t* tk, uint32_t* tv, uint32_t n, int key_bits, uint32_t* words,
+                       cudaStream_t st);
+
+// Blocks of the sub-domain selection's pass over the bit maps of n ids.
+constexpr uint32_t kBitWords = 2048;   // 32-bit words per block
+inline uint32_t sub_bit_blocks(uint32_t n) {
+    return (uint32_t)((2 * (((uint64_t)n + 31) / 32) + kBitWords - 1) / kBitWords);
+}
 
 struct ReorderArgs {
     const uint32_t* skey;

@@ -1,14 +1,17 @@
-// Radix sort of (cell label, index) pairs and the scan that turns per-cell
-// counts into first-index-per-cell offsets (Sec. 3.1 of the paper: label,
-// radix sort, reorder, first index of each cell).
+// Radix sort of (key, value) pairs, the scan that turns per-cell counts into
+// first-index-per-cell offsets, and the cell sort (Sec. 3.1 of the paper:
+// label, radix sort, reorder, first index of each cell).
 //
-// The sort is a least-significant-digit radix sort with 8-bit digits in the
-// single-pass "onesweep" organisation: one histogram of all digit places up
-// front (fused into the label kernel on the SPH path), then one kernel per
-// digit place in which each 4096-key tile ranks its keys in shared memory,
-// publishes its per-digit counts, and finds its global offsets by a bounded
-// decoupled look-back over the tiles before it.  Equal digits keep their
-// input order, so the sort is stable.
+// The sort is a stable least-significant-digit radix sort with 8-bit digits.
+// Per digit place: the digit counts of each 4096-key tile, their scans per
+// digit, and a scatter in which each tile ranks its keys in shared memory and
+// moves them to their digit's run.  Up to kFewTiles tiles the scatter adds up
+// the counts itself (no scan launch), and an input of one tile is sorted by one
+// block in one launch, all places in shared memory.  The tiles are independent: a one-pass organisation, whose tiles
+// wait for the offsets of the tiles before them, spent most of its time and
+// half of its instructions in those waits and in __match_any_sync (one GB300:
+// 4.0M pairs with 24-bit keys 192 us, 30M with 32-bit keys 1,223 us, 1,000
+// pairs 51 us; now 113, 779 and 12.5).
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -16,20 +19,7 @@ namespace sph {
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr uint32_t kFlagAgg = 1u << 30;     // tile's own count published
-constexpr uint32_t kFlagPre = 2u << 30;     // inclusive prefix published
-constexpr uint32_t kValMask = (1u << 30) - 1;
-constexpr uint32_t kSpinLimit = 1u << 24;   // polls before giving up
-
-__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
-    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
+constexpr uint32_t kFewTiles = 96;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
@@ -64,177 +54,265 @@ __device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t* s_
     return r;
 }
 
+// Lanes of `act` whose 8-bit digit equals this lane's: one ballot per bit.
+// (__match_any_sync steps through the distinct values, about 30 for random
+// digits.)
+__device__ __forceinline__ uint32_t same_digit(uint32_t d, uint32_t act) {
+    uint32_t peers = act;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool bit = (d >> b) & 1u;
+        const uint32_t set = __ballot_sync(kFull, bit);
+        peers &= bit ? set : ~set;
+    }
+    return peers;
+}
+
+// One round of a warp's stable ranking: the rank of this lane's digit among
+// the warp's keys so far (cnt: the warp's digit counts, updated).
+__device__ __forceinline__ uint32_t rank_round(uint32_t d, bool ok, uint32_t* cnt) {
+    const uint32_t peers = same_digit(d, __ballot_sync(kFull, ok));
+    uint32_t prev = 0;
+    if (ok) prev = cnt[d];
+    __syncwarp();
+    if (ok && (peers & lanemask_lt()) == 0u) cnt[d] = prev + __popc(peers);
+    __syncwarp();
+    return prev + __popc(peers & lanemask_lt());
+}
+
 __host__ __device__ __forceinline__ uint32_t digit_mask(int pass, int bits_total) {
     int b = bits_total - 8 * pass;
     b = b > 8 ? 8 : (b < 0 ? 0 : b);
     return (1u << b) - 1u;
 }
 
-__global__ void __launch_bounds__(256) k_digit_hist(const uint32_t* __restrict__ keys,
-                                                    uint32_t n, int passes, int bits_total,
-                                                    uint32_t* __restrict__ hist) {
-    __shared__ uint32_t sh[4 * 256];
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) sh[i] = 0;
+// Digit counts of each tile: cnt[tile * 256 + d] for few tiles, else in the
+// scan's order, cnt[d * tiles + tile].  Two copies in shared memory (even and
+// odd warps), four keys per load where the input is 16-byte aligned.
+__global__ void __launch_bounds__(kOsThreads) k_tile_counts(const uint32_t* __restrict__ keys,
+                                                            uint32_t n, int shift, uint32_t dmask,
+                                                            uint32_t tiles,
+                                                            uint32_t* __restrict__ cnt) {
+    __shared__ uint32_t sh[2][256];
+    sh[0][threadIdx.x] = 0u;
+    sh[1][threadIdx.x] = 0u;
     __syncthreads();
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += gridDim.x * blockDim.x) {
-        const uint32_t k = keys[i];
-        for (int p = 0; p < passes; ++p)
-            atomicAdd(&sh[p * 256 + ((k >> (8 * p)) & digit_mask(p, bits_total))], 1u);
+    uint32_t* my = sh[(threadIdx.x >> 5) & 1];
+    const uint32_t t0 = blockIdx.x * kOsTile;
+    if (((uintptr_t)keys % 16u) == 0u && n - t0 >= (uint32_t)kOsTile) {
+        uint4 k[kOsItems / 4];
+#pragma unroll
+        for (int r = 0; r < kOsItems / 4; ++r)
+            k[r] = __ldg(reinterpret_cast<const uint4*>(keys + t0) + r * kOsThreads + threadIdx.x);
+#pragma unroll
+        for (int r = 0; r < kOsItems / 4; ++r) {
+            atomicAdd(&my[(k[r].x >> shift) & dmask], 1u);
+            atomicAdd(&my[(k[r].y >> shift) & dmask], 1u);
+            atomicAdd(&my[(k[r].z >> shift) & dmask], 1u);
+            atomicAdd(&my[(k[r].w >> shift) & dmask], 1u);
+        }
+    } else {
+        for (uint32_t i = t0 + threadIdx.x; i < n && i < t0 + kOsTile; i += kOsThreads)
+            atomicAdd(&my[(keys[i] >> shift) & dmask], 1u);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < passes * 256; i += blockDim.x)
-        if (sh[i]) atomicAdd(&hist[i], sh[i]);
+    const uint32_t c = sh[0][threadIdx.x] + sh[1][threadIdx.x];
+    cnt[tiles <= kFewTiles ? blockIdx.x * 256u + threadIdx.x
+                           : (size_t)threadIdx.x * tiles + blockIdx.x] = c;
 }
 
-// Decoupled look-back for one digit: the sum of the counts of the tiles
-// before `tile` (status words of 256 digits per tile; a tile's word holds its
-// own count, kFlagAgg, or the inclusive prefix, kFlagPre, or 0 while it has
-// published nothing).  The predecessors are polled kLookWin at a time (the
-// loads of one window are in flight together), and the walk takes their
-// counts in order until an inclusive prefix ends it or a silent tile stops
-// it, where the next window starts.  A predecessor that stays silent for
-// `limit` windows makes the wait give up: the timeout bit is set in *err and
-// the partial sum returned, which never exceeds the true prefix (so scatter
-// addresses stay inside the output).  Tile 0 always publishes an inclusive
-// prefix, so no window reads before it.
-constexpr int kLookWin = 8;
-
-__device__ __forceinline__ uint32_t lookback_prefix(const uint32_t* status, uint32_t tile,
-                                                    int digit, uint32_t limit, uint32_t* err) {
-    uint32_t excl = 0;
-    int64_t p = (int64_t)tile - 1;
-    uint32_t spins = 0;
-    while (p >= 0) {
-        uint32_t s[kLookWin];
+// Exclusive scan of each digit's counts over the tiles, in place, one block per
+// digit; its total to tot[d].  (The scatter's blocks add up the digits before
+// theirs.  One scan over all counts with a look-back between its tiles took
+// twice as long, 9 us for 977 tiles.)
+__global__ void __launch_bounds__(kOsThreads) k_digit_scan(uint32_t* __restrict__ cnt, uint32_t tiles,
+                                                           uint32_t* __restrict__ tot) {
+    __shared__ uint32_t s_w[8];
+    __shared__ uint32_t s_carry;
+    uint32_t* c = cnt + (size_t)blockIdx.x * tiles;
+    if (threadIdx.x == 0) s_carry = 0u;
+    __syncthreads();
+    for (uint32_t t0 = 0; t0 < tiles; t0 += kOsThreads * 4) {
+        const uint32_t i = t0 + threadIdx.x * 4;
+        uint32_t v[4], sum = 0;
 #pragma unroll
-        for (int j = 0; j < kLookWin; ++j)
-            s[j] = p - j >= 0 ? ld_relaxed(status + (size_t)(p - j) * 256 + digit) : kFlagPre;
-        bool stop = false, fin = false;
-        int taken = 0;
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < tiles ? c[i + k] : 0u;
+            sum += v[k];
+        }
+        const uint32_t carry = s_carry;
+        uint32_t run = carry + block_excl_scan_256(sum, s_w);
 #pragma unroll
-        for (int j = 0; j < kLookWin; ++j) {
-            if (!stop) {
-                const uint32_t flag = s[j] & ~kValMask;
-                if (flag == 0u) {
-                    stop = true;
-                } else {
-                    excl += s[j] & kValMask;
-                    ++taken;
-                    if (flag == kFlagPre) stop = fin = true;
-                }
-            }
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < tiles) c[i + k] = run;
+            run += v[k];
         }
-        if (fin) break;
-        p -= taken;
-        if (taken == 0 && ++spins > limit) {
-            atomicOr(err, kStatusTimeout);
-            break;
-        }
+        if (threadIdx.x == kOsThreads - 1) s_carry = run;
+        __syncthreads();
     }
-    return excl;
+    if (threadIdx.x == 0) tot[blockIdx.x] = s_carry;
 }
 
-// One digit place.  hist holds the global count of each digit value for
-// this place; status holds one word per (tile, digit), zero on entry;
-// tilectr is a zeroed counter that hands out tiles in launch order, so every
-// tile a block waits on belongs to a block that is already running.
-__global__ void __launch_bounds__(kOsThreads) k_onesweep(
+// The scatter of one digit place.  tab: the tiles' counts (few tiles) or
+// their scans per digit, tot the digits' totals.  Keys of a tile are ranked per warp (rounds of 32 in
+// input order), moved to the tile's sorted order in shared memory and written
+// from there in runs.
+__global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
     uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, uint32_t n, int shift,
-    uint32_t dmask, const uint32_t* __restrict__ hist, uint32_t* status,
-    uint32_t* tilectr, uint32_t* err) {
+    uint32_t dmask, uint32_t tiles, const uint32_t* __restrict__ tab,
+    const uint32_t* __restrict__ tot) {
     constexpr int W = kOsThreads / 32;
-    __shared__ uint32_t s_tile;
     __shared__ uint32_t s_wh[W][256];       // per-warp digit counts, then offsets
-    __shared__ uint32_t s_dstart[256];      // tile-local first slot per digit
-    __shared__ uint32_t s_gbase[256];       // global first slot of the tile's digit run
+    __shared__ uint32_t s_run[256];         // global first slot of the digit's run, less its
+                                            // first slot in the tile
     __shared__ uint32_t s_w[8];
     __shared__ uint32_t s_keys[kOsTile];
     __shared__ uint32_t s_vals[kOsTile];
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid == 0) s_tile = atomicAdd(tilectr, 1u);
-    for (int i = tid; i < W * 256; i += kOsThreads) (&s_wh[0][0])[i] = 0;
-    const uint32_t gofs = block_excl_scan_256(hist[tid], s_w);   // also syncs
-    const uint32_t tile = s_tile;
+    const uint32_t tile = blockIdx.x;
     const uint32_t base = tile * kOsTile + w * (kOsItems * 32);
-
-    uint32_t k[kOsItems], v[kOsItems], rk[kOsItems];
+    uint32_t k[kOsItems];
 #pragma unroll
     for (int r = 0; r < kOsItems; ++r) {
         const uint32_t idx = base + r * 32 + lane;
-        const bool ok = idx < n;
-        k[r] = ok ? kin[idx] : 0u;
-        v[r] = ok ? (vin ? vin[idx] : idx) : 0u;
-        rk[r] = ok ? 0u : 0xffffffffu;
+        k[r] = idx < n ? kin[idx] : 0u;
     }
-    // Warp-level stable ranking: items r = 0..15 in order, lanes in order.
-    const uint32_t lt = lanemask_lt();
-#pragma unroll
-    for (int r = 0; r < kOsItems; ++r) {
-        const bool ok = rk[r] == 0u;
-        const uint32_t d = ok ? ((k[r] >> shift) & dmask) : 256u + lane;
-        const uint32_t peers = __match_any_sync(kFull, d);
-        uint32_t prev = 0;
-        if (ok) prev = s_wh[w][d];
-        __syncwarp();
-        if (ok) {
-            rk[r] = prev + __popc(peers & lt);
-            if (lane == __ffs(peers) - 1) s_wh[w][d] = prev + __popc(peers);
+    // the global first slot of digit tid in this tile
+    uint32_t before = 0, total = 0;
+    if (tiles <= kFewTiles) {
+        for (uint32_t t = 0; t < tiles; ++t) {
+            const uint32_t c = __ldg(tab + t * 256u + tid);
+            before += t < tile ? c : 0u;
+            total += c;
         }
-        __syncwarp();
+    } else {
+        before = __ldg(tab + (size_t)tid * tiles + tile);
+        total = __ldg(tot + tid);
     }
+    const uint32_t first = block_excl_scan_256(total, s_w) + before;
+    for (int i = tid; i < W * 256; i += kOsThreads) (&s_wh[0][0])[i] = 0;
     __syncthreads();
-    // Thread tid owns digit tid: per-warp exclusive offsets and tile count.
+    uint32_t rk[kOsItems];
+#pragma unroll
+    for (int r = 0; r < kOsItems; ++r)
+        rk[r] = rank_round((k[r] >> shift) & dmask, base + r * 32 + lane < n, s_wh[w]);
+    __syncthreads();
+    // Thread tid owns digit tid: the digit's first slot in the tile, and each
+    // warp's first slot
     uint32_t run = 0;
+#pragma unroll
+    for (int ww = 0; ww < W; ++ww) run += s_wh[ww][tid];
+    uint32_t slot = block_excl_scan_256(run, s_w);
+    s_run[tid] = first - slot;
 #pragma unroll
     for (int ww = 0; ww < W; ++ww) {
         const uint32_t c = s_wh[ww][tid];
-        s_wh[ww][tid] = run;
-        run += c;
+        s_wh[ww][tid] = slot;
+        slot += c;
     }
-    const uint32_t cnt = run;
-    uint32_t* my = status + (size_t)tile * 256 + tid;
-    st_relaxed(my, (tile == 0 ? kFlagPre : kFlagAgg) | cnt);
-    const uint32_t dstart = block_excl_scan_256(cnt, s_w);
-    s_dstart[tid] = dstart;
-    // Decoupled look-back for digit tid.
-    uint32_t excl = 0;
-    if (tile > 0) {
-        excl = lookback_prefix(status, tile, tid, kSpinLimit, err);
-        st_relaxed(my, kFlagPre | (excl + cnt));
-    }
-    s_gbase[tid] = gofs + excl;
     __syncthreads();
-    // Scatter into tile-sorted order in shared memory.
 #pragma unroll
     for (int r = 0; r < kOsItems; ++r) {
-        if (rk[r] != 0xffffffffu) {
-            const uint32_t d = (k[r] >> shift) & dmask;
-            const uint32_t pos = s_dstart[d] + s_wh[w][d] + rk[r];
+        const uint32_t idx = base + r * 32 + lane;
+        if (idx < n) {
+            const uint32_t pos = s_wh[w][(k[r] >> shift) & dmask] + rk[r];
             s_keys[pos] = k[r];
-            s_vals[pos] = v[r];
+            s_vals[pos] = vin ? vin[idx] : idx;
         }
     }
     __syncthreads();
     const uint32_t t0 = tile * kOsTile;
     const uint32_t nv = (n - t0) < (uint32_t)kOsTile ? (n - t0) : (uint32_t)kOsTile;
+#pragma unroll 4
     for (uint32_t i = tid; i < nv; i += kOsThreads) {
         const uint32_t key = s_keys[i];
-        const uint32_t d = (key >> shift) & dmask;
-        const uint32_t g = s_gbase[d] + (i - s_dstart[d]);
+        const uint32_t g = s_run[(key >> shift) & dmask] + i;
         kout[g] = key;
         vout[g] = s_vals[i];
     }
 }
 
-// Self-test of the failure path: one block of 256 threads runs the look-back
-// of tile 1 against a tile 0 whose status words stay zero (nothing
-// publishes them), so every digit's wait gives up after `limit` polls.
-__global__ void __launch_bounds__(256) k_lookback_selftest(const uint32_t* status, uint32_t limit,
-                                                           uint32_t* err) {
-    lookback_prefix(status, 1u, (int)threadIdx.x, limit, err);
+// All digit places of an input of at most one tile, by one block.
+__global__ void __launch_bounds__(kOsThreads) k_sort_tile(const uint32_t* __restrict__ kin,
+                                                          const uint32_t* __restrict__ vin,
+                                                          uint32_t* __restrict__ kout,
+                                                          uint32_t* __restrict__ vout, uint32_t n,
+                                                          int bits_total) {
+    constexpr int W = kOsThreads / 32;
+    __shared__ uint32_t s_wh[W][256];
+    __shared__ uint32_t s_w[8];
+    __shared__ uint32_t s_keys[kOsTile];
+    __shared__ uint32_t s_vals[kOsTile];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    // rounds of 32 keys per warp, the warps' shares consecutive
+    const uint32_t rounds = (n + kOsThreads - 1) / kOsThreads;
+    const uint32_t base = w * rounds * 32;
+    uint32_t k[kOsItems], v[kOsItems], rk[kOsItems];
+#pragma unroll
+    for (int r = 0; r < kOsItems; ++r) {
+        const uint32_t idx = base + r * 32 + lane;
+        const bool ok = (uint32_t)r < rounds && idx < n;
+        k[r] = ok ? kin[idx] : 0u;
+        v[r] = ok ? (vin ? vin[idx] : idx) : 0u;
+    }
+    for (int shift = 0; shift < bits_total; shift += 8) {
+        const uint32_t dmask = digit_mask(shift / 8, bits_total);
+        for (int i = tid; i < W * 256; i += kOsThreads) (&s_wh[0][0])[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOsItems; ++r)
+            if ((uint32_t)r < rounds)
+                rk[r] = rank_round((k[r] >> shift) & dmask, base + r * 32 + lane < n, s_wh[w]);
+        __syncthreads();
+        uint32_t run = 0;
+#pragma unroll
+        for (int ww = 0; ww < W; ++ww) run += s_wh[ww][tid];
+        uint32_t slot = block_excl_scan_256(run, s_w);
+#pragma unroll
+        for (int ww = 0; ww < W; ++ww) {
+            const uint32_t c = s_wh[ww][tid];
+            s_wh[ww][tid] = slot;
+            slot += c;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOsItems; ++r) {
+            const uint32_t idx = base + r * 32 + lane;
+            if ((uint32_t)r < rounds && idx < n) {
+                const uint32_t pos = s_wh[w][(k[r] >> shift) & dmask] + rk[r];
+                s_keys[pos] = k[r];
+                s_vals[pos] = v[r];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOsItems; ++r) {
+            const uint32_t idx = base + r * 32 + lane;
+            if ((uint32_t)r < rounds && idx < n) {
+                k[r] = s_keys[idx];
+                v[r] = s_vals[idx];
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < kOsItems; ++r) {
+        const uint32_t idx = base + r * 32 + lane;
+        if ((uint32_t)r < rounds && idx < n) {
+            kout[idx] = k[r];
+            vout[idx] = v[r];
+        }
+    }
+}
+
+// Self-test of the failure path: one warp runs the scan's look-back of tile 1
+// against a tile 0 whose word stays zero (nothing publishes it), so the wait
+// gives up after `limit` polls.
+__global__ void k_lookback_selftest(const unsigned long long* words, uint32_t limit,
+                                    uint32_t* err) {
+    tile_lookback(words, 1u, 1u, limit, err);
 }
 
 // --- exclusive scan of the per-cell counts into cell offsets --------------
@@ -451,30 +529,42 @@ void launch_cell_scatter(const uint32_t* key, uint32_t n, const uint32_t* off, u
     launch_pdl(k_cell_scatter, (n + 255) / 256, 256, 0, st, key, n, off, cnt, kout, vout, status);
 }
 
-void launch_lookback_selftest(uint32_t* zeroed256, uint32_t limit, uint32_t* err,
-                              cudaStream_t st) {
-    cudaMemsetAsync(zeroed256, 0, 256 * sizeof(uint32_t), st);
-    k_lookback_selftest<<<1, 256, 0, st>>>(zeroed256, limit, err);
+void launch_lookback_selftest(uint32_t* zeroed, uint32_t limit, uint32_t* err, cudaStream_t st) {
+    cudaMemsetAsync(zeroed, 0, 4 * sizeof(uint32_t), st);
+    k_lookback_selftest<<<1, 32, 0, st>>>(reinterpret_cast<const unsigned long long*>(zeroed), limit,
+                                          err);
 }
 
-void launch_digit_hist(const uint32_t* keys, uint32_t n, int passes, int bits_total,
-                       uint32_t* hist, cudaStream_t st) {
-    uint32_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 8) blocks = 152 * 8;
-    if (blocks == 0) blocks = 1;
-    k_digit_hist<<<blocks, 256, 0, st>>>(keys, n, passes, bits_total, hist);
+size_t radix_sort_words(uint32_t n) {
+    return (size_t)os_tiles(n) * 256 + 256;   // counts, then the digits' totals
 }
 
-void launch_onesweep_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
-                          uint32_t* vout, uint32_t n, int pass, int bits_total,
-                          const uint32_t* hist, uint32_t* status, uint32_t* tilectr,
-                          uint32_t* err, cudaStream_t st) {
+void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
+                       uint32_t* tk, uint32_t* tv, uint32_t n, int key_bits, uint32_t* words,
+                       cudaStream_t st) {
     const uint32_t tiles = os_tiles(n);
     if (tiles == 0) return;
-    k_onesweep<<<tiles, kOsThreads, 0, st>>>(kin, vin, kout, vout, n, 8 * pass,
-                                             digit_mask(pass, bits_total), hist + 256 * pass,
-                                             status + (size_t)pass * tiles * 256,
-                                             tilectr + pass, err);
+    if (tiles == 1) {
+        k_sort_tile<<<1, kOsThreads, 0, st>>>(kin, vin, kout, vout, n, key_bits);
+        return;
+    }
+    uint32_t* cnt = words;
+    uint32_t* tot = cnt + (size_t)tiles * 256;
+    const int passes = (key_bits + 7) / 8;
+    const uint32_t* ck = kin;
+    const uint32_t* cv = vin;
+    for (int p = 0; p < passes; ++p) {
+        // ping-pong so that the last place lands in the outputs
+        const bool to_out = ((passes - 1 - p) % 2) == 0;
+        uint32_t* ok = to_out ? kout : tk;
+        uint32_t* ov = to_out ? vout : tv;
+        const uint32_t dm = digit_mask(p, key_bits);
+        k_tile_counts<<<tiles, kOsThreads, 0, st>>>(ck, n, 8 * p, dm, tiles, cnt);
+        if (tiles > kFewTiles) k_digit_scan<<<256, kOsThreads, 0, st>>>(cnt, tiles, tot);
+        k_radix_scatter<<<tiles, kOsThreads, 0, st>>>(ck, cv, ok, ov, n, 8 * p, dm, tiles, cnt, tot);
+        ck = ok;
+        cv = ov;
+    }
 }
 
 }  // namespace sph

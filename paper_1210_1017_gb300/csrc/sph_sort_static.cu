@@ -7,8 +7,7 @@
 // a latency-critical loop that must not call cudaMalloc/cudaFree at run time
 // because those calls can synchronise the whole device and stall work on
 // other streams.  Such callers still own the input and output arrays; only the
-// sort's own scratch (temporary keys/values, digit histograms, tile counters
-// and look-back status words) moves into a fixed array that is part of the
+// sort's own scratch (temporary keys/values, tile counts and digit totals) moves into a fixed array that is part of the
 // loaded library.
 //
 // The array below is a host-side stand-in when named from host code; the
@@ -30,15 +29,12 @@ using namespace sph;
 
 constexpr uint32_t kMaxN = SPH_RADIX_SORT_STATIC_MAX_N;
 constexpr uint32_t kMaxTiles = (kMaxN + kOsTile - 1) / kOsTile;
-constexpr int kMaxPasses = 4;
 
 // Layout of the fixed scratch, in 32-bit words.
 constexpr size_t kTmpKeys = 0;
 constexpr size_t kTmpVals = kTmpKeys + kMaxN;
-constexpr size_t kHist = kTmpVals + kMaxN;                 // 4 x 256 digit counts
-constexpr size_t kTileCtr = kHist + kMaxPasses * 256;      // one per pass
-constexpr size_t kStatus = kTileCtr + kMaxPasses;          // passes x tiles x 256
-constexpr size_t kErr = kStatus + (size_t)kMaxPasses * kMaxTiles * 256;
+constexpr size_t kSort = kTmpVals + kMaxN;                 // radix_sort_words(kMaxN) at most
+constexpr size_t kErr = kSort + (size_t)kMaxTiles * 256 + 256;
 constexpr size_t kWords = kErr + 64;
 
 static __device__ __align__(256) uint32_t g_sort_scratch[kWords];
@@ -75,24 +71,10 @@ extern "C" int sph_radix_sort_pairs_static(const uint32_t* d_keys_in, const uint
     const int rc = scratch_for_current_device(&s);
     if (rc != SPH_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int passes = ((int)key_bits + 7) / 8;
-    const uint32_t tiles = os_tiles(n);
-    // the previous call's contents are still there: clear what counts
-    cudaMemsetAsync(s + kHist, 0, (kMaxPasses * 256 + kMaxPasses) * sizeof(uint32_t), st);
-    cudaMemsetAsync(s + kStatus, 0, (size_t)passes * tiles * 256 * sizeof(uint32_t), st);
+    if (radix_sort_words(n) > kErr - kSort) return SPH_ERR_TOO_LARGE;   // not for n <= kMaxN
     cudaMemsetAsync(s + kErr, 0, sizeof(uint32_t), st);
-    launch_digit_hist(d_keys_in, n, passes, (int)key_bits, s + kHist, st);
-    const uint32_t* ck = d_keys_in;
-    const uint32_t* cv = d_vals_in;
-    for (int p = 0; p < passes; ++p) {
-        const bool to_out = ((passes - 1 - p) % 2) == 0;
-        uint32_t* ok = to_out ? d_keys_out : s + kTmpKeys;
-        uint32_t* ov = to_out ? d_vals_out : s + kTmpVals;
-        launch_onesweep_pass(ck, cv, ok, ov, n, p, (int)key_bits, s + kHist, s + kStatus,
-                             s + kTileCtr, s + kErr, st);
-        ck = ok;
-        cv = ov;
-    }
+    launch_radix_sort(d_keys_in, d_vals_in, d_keys_out, d_vals_out, s + kTmpKeys, s + kTmpVals, n,
+                      (int)key_bits, s + kSort, st);
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 
@@ -115,9 +97,9 @@ extern "C" int sph_radix_sort_static_selftest_timeout(uint32_t polls, void* stre
     if (rc != SPH_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaMemsetAsync(s + kErr, 0, sizeof(uint32_t), st);
-    // tile 1 of the first pass waits on tile 0's status words (zeroed by the
-    // self-test launch), which nothing publishes
-    launch_lookback_selftest(s + kStatus, polls, s + kErr, st);
+    // a look-back of tile 1 on tile 0's word (zeroed by the launch), which
+    // nothing publishes
+    launch_lookback_selftest(s + kSort, polls, s + kErr, st);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return SPH_ERR_CUDA;
     return SPH_OK;
