@@ -901,10 +901,8 @@ __global__ void __launch_bounds__(128) k_row_csum(const Dev d, const uint32_t* _
 // row, mode 1 writes them at the row's offset (uint2: first particle, end).
 constexpr int kUnitChunk = 16;
 
-// The walk of row r: its units (mode 1 writes them from units[out]).  With
-// SCS the row's staged-candidate sums are read from `csum` itself (the
-// caller's shared-memory copy, indexes 0..ncx) instead of the global array.
-template <int MODE, bool SCS = false>
+// The walk of row r: its units (mode 1 writes them from units[out]).
+template <int MODE>
 __device__ __forceinline__ uint32_t unit_walk(const Dev& d, const uint32_t* __restrict__ off,
                                               const uint32_t* __restrict__ csum, uint32_t r,
                                               uint32_t out,
@@ -913,7 +911,7 @@ __device__ __forceinline__ uint32_t unit_walk(const Dev& d, const uint32_t* __re
     const int ncx = I.ncx;
     const uint32_t lr = r - I.row_base;
     const uint32_t* o = off + I.cell_base + (size_t)lr * (uint32_t)ncx;
-    const uint32_t* cs = SCS ? csum : csum + I.cell_base + (size_t)lr * (uint32_t)ncx + r;
+    const uint32_t* cs = csum + I.cell_base + (size_t)lr * (uint32_t)ncx + r;
     uint32_t n = 0;
     uint32_t start = 0xffffffffu;
     uint32_t base = 0;   // cs[first - 1] of the open unit (clamped at 0)
@@ -932,7 +930,7 @@ __device__ __forceinline__ uint32_t unit_walk(const Dev& d, const uint32_t* __re
         for (int k = 0; k < kUnitChunk + 3; ++k) {
             const int xi = x0 - 1 + k;
             const int xc = xi < 0 ? 0 : (xi < ncx ? xi : ncx);
-            cc[k] = SCS ? cs[xc] : __ldg(cs + xc);
+            cc[k] = __ldg(cs + xc);
         }
 #pragma unroll
         for (int k = 0; k < kUnitChunk; ++k) {
@@ -984,15 +982,18 @@ __global__ void __launch_bounds__(128) k_units(const Dev d, const uint32_t* __re
 
 // The unit list of a grid of few rows in one launch (d.nrows <= kFusedRows,
 // rows of at most kFusedNcx cells): one warp per row, rows taken in launch
-// order from a ticket.  The warp sums the row's 9 neighbour-row offsets into
-// shared memory (k_row_csum's sums), lane 0 counts the row's units, a
-// decoupled look-back over the rows before it (tile_lookback, one word per
-// row holding its unit count) gives the row's first unit, and lane 0 writes
-// the units.  The warp of the last row writes the total and rearms the
-// ticket and the epoch: its look-back ended on a prefix, so every row has
-// taken its ticket and read the epoch by then.  A look-back that gave up
-// leaves a partial prefix, never above the true one, so every write stays
-// inside the unit array.
+// order from a ticket.  The warp copies the row's cell offsets and sums its 9
+// neighbour-row offsets (k_row_csum's sums) into shared memory, cuts the row
+// into units (row_units), a decoupled look-back over the rows before it
+// (tile_lookback, one word per row holding its unit count) gives the row's
+// first unit, and the lanes write the units.  The warp of the last row writes
+// the total and rearms the ticket and the epoch: its look-back ended on a
+// prefix, so every row has taken its ticket and read the epoch by then.  A
+// look-back that gave up leaves a partial prefix, never above the true one, so
+// every write stays inside the unit array.
+// On the step's critical path (it runs beside the scatter and the reorder but
+// took longer than both: 13-15 us at 17k particles and 73 us at 1.39M against 11
+// and 60, with one lane walking the row's cells twice).
 constexpr uint32_t kFusedRows = 8192;
 constexpr int kFusedNcx = 1023;
 constexpr int kFusedWarps = 4;
@@ -1006,11 +1007,76 @@ __global__ void k_row_lookback_selftest(const unsigned long long* zeroed, uint32
     tile_lookback(zeroed, 1u, 1u, limit, err);
 }
 
+// unit_walk's units of one row by a warp: from the unit's first cell on, lane k
+// looks at cell lo + k (a unit spans at most kSpan = 32 cells), so the next cut
+// is the first lane with a reason for one.  o, cs: the row's cell offsets and
+// staged-candidate sums, indexes 0..ncx (shared memory).  Units from number
+// `first` on are written to list (at most cap of them); returns their number
+// in all.
+static_assert(kSpan == 32, "one lane per cell of a unit");
+__device__ __forceinline__ uint32_t row_units(const Dev& d, const uint32_t* o, const uint32_t* cs,
+                                              int ncx, uint32_t first, uint32_t cap, uint2* list) {
+    const int lane = threadIdx.x & 31;
+    // first cell >= x that holds particles (ncx: none)
+    auto next_cell = [&](int x) {
+        for (; x < ncx; x += 32) {
+            const int c = x + lane;
+            const uint32_t m = __ballot_sync(kFull, c < ncx && o[c] != o[c + 1]);
+            if (m) return x + __ffs(m) - 1;
+        }
+        return ncx;
+    };
+    uint32_t n = 0;
+    auto emit = [&](uint32_t a, uint32_t b) {
+        if (lane == 0 && n >= first && n - first < cap) list[n - first] = make_uint2(a, b);
+        ++n;
+    };
+    int lo = next_cell(0);
+    uint32_t start = o[lo];
+    while (lo < ncx) {
+        const uint32_t base = cs[lo > 0 ? lo - 1 : 0];
+        const int c = lo + lane;
+        const uint32_t a = c < ncx ? o[c] : o[ncx], b = c < ncx ? o[c + 1] : a;
+        const uint32_t held = __ballot_sync(kFull, a != b);          // lane 0 always
+        const uint32_t below = held & ((1u << lane) - 1u);
+        const bool cand = a != b && lane > 0;
+        // a cut before this cell: more than two empty cells, or too many
+        // candidates with it; a cut inside it: the unit is full
+        const uint32_t before = __ballot_sync(
+            kFull, cand && (lane - (31 - __clz(below)) > 3 ||
+                            cs[c + 2 < ncx ? c + 2 : ncx] - base > (uint32_t)d.stage));
+        const uint32_t inside = __ballot_sync(kFull, a != b && b - start > (uint32_t)d.unit);
+        const int fb = before ? __ffs(before) - 1 : 32, fi = inside ? __ffs(inside) - 1 : 32;
+        if (fb <= fi && fb < 32) {
+            const uint32_t end = __shfl_sync(kFull, a, fb);
+            emit(start, end);
+            start = end;
+            lo += fb;
+        } else if (fi < 32) {
+            emit(start, start + d.unit);
+            start += d.unit;
+            lo += fi;
+        } else {
+            // nothing in the window: the row ends, or the span limit cuts
+            const int nx = next_cell(lo + kSpan);
+            const uint32_t end = o[nx];
+            emit(start, end);
+            start = end;
+            lo = nx;
+        }
+    }
+    return n;
+}
+
+constexpr uint32_t kRowList = 128;   // units of a row kept in shared memory
+
 __global__ void __launch_bounds__(kFusedWarps * 32) k_units_fused(const Dev d,
                                                                    const uint32_t* __restrict__ off,
                                                                    const UnitsFusedArgs a) {
     pdl_wait();
     __shared__ uint32_t s_cs[kFusedWarps][kFusedNcx + 1];
+    __shared__ uint32_t s_o[kFusedWarps][kFusedNcx + 1];
+    __shared__ uint2 s_list[kFusedWarps][kRowList];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (blockIdx.x * kFusedWarps + w >= d.nrows) return;   // exactly nrows tickets
     uint32_t r = 0, ep = 0;
@@ -1025,21 +1091,24 @@ __global__ void __launch_bounds__(kFusedWarps * 32) k_units_fused(const Dev d,
     const uint32_t lr = r - I.row_base;
     const int cy = (int)(lr % (uint32_t)I.ncy), cz = (int)(lr / (uint32_t)I.ncy);
     uint32_t* cs = s_cs[w];
+    uint32_t* o = s_o[w];
     for (int x = lane; x <= ncx; x += 32) {
         uint32_t t = 0;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int yy = cy + k % 3 - 1, zz = cz + k / 3 - 1;
-            if (yy >= 0 && yy < I.ncy && zz >= 0 && zz < I.ncz)
-                t += __ldg(off + I.cell_base +
-                           ((size_t)zz * (uint32_t)I.ncy + (uint32_t)yy) * (uint32_t)ncx + x);
+            if (yy >= 0 && yy < I.ncy && zz >= 0 && zz < I.ncz) {
+                const uint32_t v = __ldg(off + I.cell_base +
+                                         ((size_t)zz * (uint32_t)I.ncy + (uint32_t)yy) * (uint32_t)ncx + x);
+                t += v;
+                if (k == 4) o[x] = v;
+            }
         }
         cs[x] = t;
     }
     __syncwarp();
-    uint32_t n = 0;
-    if (lane == 0) n = unit_walk<0, true>(d, off, cs, r, 0u, nullptr);
-    n = __shfl_sync(kFull, n, 0);
+    const uint32_t n = row_units(d, o, cs, ncx, 0u, kRowList, s_list[w]);
+    __syncwarp();
     const unsigned long long tag = (unsigned long long)ep << 34;
     uint32_t excl = 0;
     if (r > 0) {
@@ -1048,12 +1117,21 @@ __global__ void __launch_bounds__(kFusedWarps * 32) k_units_fused(const Dev d,
     }
     if (lane == 0) {
         st_relaxed64(a.words + r, tag | (2ull << 32) | (excl + n));
-        unit_walk<1, true>(d, off, cs, r, excl, a.units);
         if (r == d.nrows - 1) {
             *a.total = excl + n;
             a.ctl[0] = 0u;
             a.ctl[1] = ep + 1u;
         }
+    }
+    for (uint32_t k0 = 0; k0 < n; k0 += kRowList) {
+        if (k0 > 0) {   // a row of more units: cut it again from unit k0
+            __syncwarp();
+            row_units(d, o, cs, ncx, k0, kRowList, s_list[w]);
+            __syncwarp();
+        }
+        const uint32_t m = n - k0 < kRowList ? n - k0 : kRowList;
+        for (uint32_t k = lane; k < m; k += 32)
+            if (in_bounds(excl + k0 + k < d.units_cap, d.status)) a.units[excl + k0 + k] = s_list[w][k];
     }
 }
 
