@@ -57,7 +57,8 @@ __global__ void k_unpack(uint32_t n, const double* __restrict__ pos, const float
     vr[i] = make_float4(vel[3 * (size_t)i], vel[3 * (size_t)i + 1], vel[3 * (size_t)i + 2], rho[i]);
 }
 
-// k_unpack for a pipelined upload: the ids come from the staging slot too.
+// k_unpack with the ids from an array of their own (a pipelined upload's
+// staging slot, or the caller's).
 __global__ void k_unpack_ids(uint32_t n, const double* __restrict__ pos,
                              const float* __restrict__ vel, const float* __restrict__ rho,
                              const uint32_t* __restrict__ ids, double* x, double* y, double* z,
@@ -663,22 +664,38 @@ int sph_upload(sph_ctx* c, const double* pos, const float* vel, const float* rho
     if (!c || !pos || !vel || !rho || !ids) return fail(c, SPH_ERR_INVALID_ARG, "NULL argument");
     const size_t n = c->n;
     cudaStream_t st = c->st;
-    double* dpos = c->stage_pos;
-    float* dvel = c->stage_vr;
-    float* drho = c->stage_vr + 3 * n;
-    // cudaMemcpyDefault: host or device source (unified addressing)
-    int rc = cuda_check(c, cudaMemcpyAsync(dpos, pos, 3 * n * sizeof(double), cudaMemcpyDefault, st), "upload pos");
-    if (rc) return rc;
-    cudaMemcpyAsync(dvel, vel, 3 * n * sizeof(float), cudaMemcpyDefault, st);
-    cudaMemcpyAsync(drho, rho, n * sizeof(float), cudaMemcpyDefault, st);
-    cudaMemcpyAsync(c->id[c->cur], ids, n * sizeof(uint32_t), cudaMemcpyDefault, st);
+    // arrays of this device are unpacked in place; others are staged
+    // (cudaMemcpyDefault: any source, unified addressing)
+    const double* spos = pos;
+    const float *svel = vel, *srho = rho;
+    int rc = SPH_OK;
+    if (!on_this_device(pos)) {
+        spos = c->stage_pos;
+        rc = cuda_check(c, cudaMemcpyAsync(c->stage_pos, pos, 3 * n * sizeof(double), cudaMemcpyDefault, st), "upload pos");
+        if (rc) return rc;
+    }
+    if (!on_this_device(vel)) {
+        svel = c->stage_vr;
+        cudaMemcpyAsync(c->stage_vr, vel, 3 * n * sizeof(float), cudaMemcpyDefault, st);
+    }
+    if (!on_this_device(rho)) {
+        srho = c->stage_vr + 3 * n;
+        cudaMemcpyAsync(c->stage_vr + 3 * n, rho, n * sizeof(float), cudaMemcpyDefault, st);
+    }
+    const bool ids_here = on_this_device(ids);
+    if (!ids_here)
+        cudaMemcpyAsync(c->id[c->cur], ids, n * sizeof(uint32_t), cudaMemcpyDefault, st);
     cudaMemsetAsync(c->id_flag, 0, sizeof(uint32_t), st);
     // Verlet: the first step after an upload has no earlier state (Euler)
     cudaMemsetAsync(c->i_vphase, 0, c->n_inst * sizeof(uint32_t), st);
     drop_pending_counts(c, st);
-    k_unpack<<<(uint32_t)((n + 255) / 256), 256, 0, st>>>(c->n, dpos, dvel, drho, c->x[c->cur],
-                                                         c->y[c->cur], c->z[c->cur], c->vr[c->cur],
-                                                         c->id[c->cur], c->id_flag);
+    const uint32_t nb = (uint32_t)((n + 255) / 256);
+    if (ids_here)
+        k_unpack_ids<<<nb, 256, 0, st>>>(c->n, spos, svel, srho, ids, c->x[c->cur], c->y[c->cur],
+                                         c->z[c->cur], c->vr[c->cur], c->id[c->cur], c->id_flag);
+    else
+        k_unpack<<<nb, 256, 0, st>>>(c->n, spos, svel, srho, c->x[c->cur], c->y[c->cur],
+                                     c->z[c->cur], c->vr[c->cur], c->id[c->cur], c->id_flag);
     rc = post_launch(c, "upload");
     if (rc) return rc;
     uint32_t flag = 1;
@@ -879,18 +896,23 @@ int sph_download(sph_ctx* c, double* pos, float* vel, float* rho, uint32_t* ids)
     if (!c->have_state) return fail(c, SPH_ERR_STATE, "no state uploaded");
     const size_t n = c->n;
     cudaStream_t st = c->st;
-    double* dpos = c->stage_pos;
-    float* dv = c->stage_vr;
-    float* dr = dv + 3 * n;
+    // arrays of this device are written in place, others from the staging
+    // (cudaMemcpyDefault: any destination, unified addressing)
+    const bool hp = on_this_device(pos), hv = on_this_device(vel), hr = on_this_device(rho),
+               hi = on_this_device(ids);
+    double* dpos = hp ? pos : c->stage_pos;
+    float* dv = hv ? vel : c->stage_vr;
+    float* dr = hr ? rho : c->stage_vr + 3 * n;
     k_pack<<<(uint32_t)((n + 255) / 256), 256, 0, st>>>(c->n, c->x[c->cur], c->y[c->cur],
-                                                       c->z[c->cur], c->vr[c->cur], dpos, dv, dr);
+                                                       c->z[c->cur], c->vr[c->cur], dpos, dv, dr,
+                                                       c->id[c->cur], hi ? ids : nullptr);
     int rc = post_launch(c, "download pack");
     if (rc) return rc;
-    // cudaMemcpyDefault: host or device destination (unified addressing)
-    if (pos) cudaMemcpyAsync(pos, dpos, 3 * n * sizeof(double), cudaMemcpyDefault, st);
-    if (vel) cudaMemcpyAsync(vel, dv, 3 * n * sizeof(float), cudaMemcpyDefault, st);
-    if (rho) cudaMemcpyAsync(rho, dr, n * sizeof(float), cudaMemcpyDefault, st);
-    if (ids) cudaMemcpyAsync(ids, c->id[c->cur], n * sizeof(uint32_t), cudaMemcpyDefault, st);
+    if (pos && !hp) cudaMemcpyAsync(pos, dpos, 3 * n * sizeof(double), cudaMemcpyDefault, st);
+    if (vel && !hv) cudaMemcpyAsync(vel, dv, 3 * n * sizeof(float), cudaMemcpyDefault, st);
+    if (rho && !hr) cudaMemcpyAsync(rho, dr, n * sizeof(float), cudaMemcpyDefault, st);
+    if (ids && !hi)
+        cudaMemcpyAsync(ids, c->id[c->cur], n * sizeof(uint32_t), cudaMemcpyDefault, st);
     return cuda_check(c, cudaStreamSynchronize(st), "download");
 }
 
@@ -905,16 +927,17 @@ int sph_download_by_id(sph_ctx* c, double* pos, float* vel, float* rho) {
     if (!c->ids_dense) return fail(c, SPH_ERR_STATE, "ids are not all below n");
     const size_t n = c->n;
     cudaStream_t st = c->st;
-    double* dpos = c->stage_pos;
-    float* dv = c->stage_vr;
-    float* dr = dv + 3 * n;
+    const bool hp = on_this_device(pos), hv = on_this_device(vel), hr = on_this_device(rho);
+    double* dpos = hp ? pos : c->stage_pos;
+    float* dv = hv ? vel : c->stage_vr;
+    float* dr = hr ? rho : c->stage_vr + 3 * n;
     k_pack_by_id<<<(uint32_t)((n + 255) / 256), 256, 0, st>>>(
         c->n, c->x[c->cur], c->y[c->cur], c->z[c->cur], c->vr[c->cur], c->id[c->cur], dpos, dv, dr);
     int rc = post_launch(c, "download_by_id pack");
     if (rc) return rc;
-    if (pos) cudaMemcpyAsync(pos, dpos, 3 * n * sizeof(double), cudaMemcpyDefault, st);
-    if (vel) cudaMemcpyAsync(vel, dv, 3 * n * sizeof(float), cudaMemcpyDefault, st);
-    if (rho) cudaMemcpyAsync(rho, dr, n * sizeof(float), cudaMemcpyDefault, st);
+    if (pos && !hp) cudaMemcpyAsync(pos, dpos, 3 * n * sizeof(double), cudaMemcpyDefault, st);
+    if (vel && !hv) cudaMemcpyAsync(vel, dv, 3 * n * sizeof(float), cudaMemcpyDefault, st);
+    if (rho && !hr) cudaMemcpyAsync(rho, dr, n * sizeof(float), cudaMemcpyDefault, st);
     return cuda_check(c, cudaStreamSynchronize(st), "download_by_id");
 }
 

@@ -131,6 +131,18 @@ inline void drop_pending_counts(sph_ctx* c, cudaStream_t st) {
     c->keys_ready = false;
 }
 
+// Whether p is memory of the current device, which a kernel may read or write
+// in place of a staging copy (host, managed and peer memory are staged).
+inline bool on_this_device(const void* p) {
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (!p || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 // Record a one-line error message on the context and return the code.
 inline int fail(sph_ctx* c, int code, const std::string& msg) {
     if (c) c->err = msg;

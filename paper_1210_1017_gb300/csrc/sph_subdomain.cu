@@ -300,17 +300,8 @@ extern "C" int sph_subdomain_select(sph_ctx* c, int mode, double xlo, double xhi
     }
     // gather straight into destinations on this device, else into the
     // transfer staging (ids into the free key buffer)
-    int dev = -1;
-    cudaGetDevice(&dev);
-    auto on_device = [&](const void* p) {
-        cudaPointerAttributes at{};
-        if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        return at.type == cudaMemoryTypeDevice && at.device == dev;
-    };
-    const bool dp = on_device(pos), dv = on_device(vel), dr = on_device(rho), di = on_device(ids);
+    const bool dp = on_this_device(pos), dv = on_this_device(vel), dr = on_this_device(rho),
+               di = on_this_device(ids);
     double* spos = dp ? pos : c->stage_pos;
     float* svel = dv ? vel : c->stage_vr;
     float* srho = dr ? rho : c->stage_vr + 3 * (size_t)n;
