@@ -6,7 +6,7 @@
 // What bounds the interaction is the number of instructions a warp issues per
 // candidate and per hit (2.0 warp instructions per clock with 16 warps per SM;
 // DRAM and the FP32 pipes are far from their limits).  So the distances of a
-// unit's 128 particles to its staged candidates are one tcgen05.mma per 128
+// unit's 128 particles to its staged candidates are one tcgen05.mma per 256
 // candidates (a product of K = 16, exact to about 2e-3 of (2h)^2), whose
 // accumulator rows a warp reads back with lane = particle: one funnel shift
 // per candidate makes a hit mask, against about three instructions on the
@@ -14,14 +14,15 @@
 // as with one word per cell.  The non-empty words go to per-lane lists in
 // shared memory and the pair phase pops them with the next word always
 // loaded (ten instructions per hit).  Blocks have no barrier inside the
-// candidate loop: the last warp done with a piece issues the MMA two pieces
-// ahead.  Both sides on one GB300, ms per launch (the counter-scheduled 4 x 2
-// shape of sph_kernels.cu / this kernel): 35.4M particles 24.0 / 20.4, 1.39M
-// with obstacles 0.956 / 0.778, 256 dam breaks (5.5M) 3.85 / 3.37, 64k with
-// the cubic spline 0.094 / 0.078; executed warp instructions at 1.39M 642M /
-// 468M.  Of the 0.78 ms at 1.39M the pair phase takes 0.23, the accumulator
-// reads and masks 0.18, the operand rows and the piece loop 0.18, the units'
-// set-up 0.20 (latency of the staging copies).
+// candidate loop: the last warp done with a piece issues the next one's MMA.
+// (Two accumulators of 128 candidates, the MMA two pieces ahead, hid the MMA's
+// latency but cost a hundred instructions per warp and piece: 20.4 against
+// 18.8 ms at 35.4M particles.)  Both sides on one GB300, ms per launch (the
+// counter-scheduled 4 x 2 shape of sph_kernels.cu / this kernel): 35.4M
+// particles 24.0 / 18.8, 1.39M with obstacles 0.956 / 0.717, 256 dam breaks
+// (5.5M) 3.85 / 3.13, 64k with the cubic spline 0.094 / 0.073, 17k 0.0229 /
+// 0.0200.  Next to the pair phase (0.23 ms of it at 1.39M) the largest share is
+// the units' set-up, 0.20: the latency of the staging copies.
 #include <cuda_fp16.h>
 #include <math.h>
 
@@ -180,15 +181,15 @@ __device__ __forceinline__ uint32_t pop_hit(HitCursor& h, uint32_t end) {
 
 // Shape of a variant: W warps of particles (units of 32 W), SPLIT warps per
 // group of 32 particles, STAGE staged candidates, WCAP hit words per lane,
-// PIECE candidates per MMA (two accumulators of PIECE TMEM columns).
+// PIECE candidates per MMA (an accumulator of PIECE TMEM columns).
 template <int W, int SPLIT, int STAGE, int WCAP, int PIECE>
 struct TcShape {
-    // staged posu and velrhop (one slot more: the pad), A, two B, lists, the
+    // staged posu and velrhop (one slot more: the pad), A, B, lists, the
     // sums of the parts 1 ..
     static constexpr size_t stage_bytes = (size_t)(STAGE + 1) * sizeof(float4);
     static constexpr size_t a_off = (2 * stage_bytes + 127) / 128 * 128;
     static constexpr size_t b_off = a_off + 128 * 32;
-    static constexpr size_t l_off = b_off + 2 * (size_t)PIECE * 32;
+    static constexpr size_t l_off = b_off + (size_t)PIECE * 32;
     static constexpr size_t c_off = l_off + (size_t)W * SPLIT * (WCAP + 1) * 256;
     static constexpr size_t smem = c_off + (size_t)(SPLIT - 1) * W * 7 * 32 * 4;
     static constexpr int fb_cap = 2 * stage_bytes / ((size_t)W * SPLIT * 32 * 4) < 64
@@ -196,8 +197,7 @@ struct TcShape {
                                       : 64;
     static_assert(fb_cap >= 16, "fallback lists must fit in the staging area");
     static_assert((size_t)(STAGE + 1) * 16 <= 65536, "list entries hold byte offsets in 16 bits");
-    static_assert(PIECE % (8 * SPLIT) == 0 && PIECE % 32 == 0 && PIECE / 32 <= W * SPLIT,
-                  "a piece's columns and its builder warps");
+    static_assert(PIECE % (8 * SPLIT) == 0 && PIECE % 32 == 0, "a piece's columns and rows");
 };
 
 // mbar_wait_bounded with the thread suspended for up to 1 us per try (fewer
@@ -267,18 +267,16 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
     constexpr int NW = W * SPLIT, NT = NW * 32;
     constexpr int FBCAP = SH::fb_cap;
     constexpr uint32_t kPad = (uint32_t)STAGE * 16u;       // list entry of the pad slot
-    constexpr int COLS = 2 * PIECE;                        // TMEM columns
-    constexpr uint32_t kPartCols = PIECE / SPLIT;          // of one part of a piece
-    constexpr int kBuilders = PIECE / 32;                  // warps that write one piece's rows
-    static_assert(NW >= 4 && (COLS == 64 || COLS == 128 || COLS == 256 || COLS == 512),
-                  "TMEM lane quarters and columns");
+        constexpr uint32_t kPartCols = PIECE / SPLIT;          // of one part of a piece
+    constexpr int kBuilders = PIECE / 32;                  // groups of 32 rows of a piece
+    static_assert(NW >= 4 && (PIECE == 128 || PIECE == 256), "TMEM lane quarters and columns");
     extern __shared__ __align__(128) unsigned char s_raw[];
     float4* s_p = reinterpret_cast<float4*>(s_raw);
     float4* s_v = s_p + STAGE + 1;
     unsigned char* s_a = s_raw + SH::a_off;
     unsigned char* s_b = s_raw + SH::b_off;
-    __shared__ __align__(8) uint64_t s_bar, s_mbar[2];
-    __shared__ uint32_t s_arr[2];                // warps done with a piece, per buffer
+    __shared__ __align__(8) uint64_t s_bar, s_mbar;   // staging copies, MMA
+    __shared__ uint32_t s_arr;                   // warps done with a piece
     __shared__ uint32_t s_tmem;
     __shared__ uint32_t s_rs[9], s_base[10];
     __shared__ uint32_t s_offb[2][9][kSpan + 3];
@@ -293,12 +291,11 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int part = w / W;
-    if (w == 0) sur::tmem_alloc(&s_tmem, COLS);
+    if (w == 0) sur::tmem_alloc(&s_tmem, PIECE);
     if (tid == 0) {
         mbar_init(&s_bar, 1);
-        mbar_init(&s_mbar[0], 1);
-        mbar_init(&s_mbar[1], 1);
-        s_arr[0] = s_arr[1] = 0u;
+        mbar_init(&s_mbar, 1);
+        s_arr = 0u;
     }
     pdl_wait();
     sur::tc_fence_before();
@@ -313,12 +310,11 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
     const float fx_len = d.csf * fx_cell;                  // fixed-point x to length
     const uint32_t nunits = *a.n_units;
     // the constant second halves of operand B's rows
-    for (int t = tid; t < 2 * PIECE; t += NT)
-        *reinterpret_cast<uint4*>(s_b + (t / PIECE) * (PIECE * 32) +
-                                  sur::kmajor_offset((uint32_t)(t % PIECE), 8, 16)) =
+    for (int t = tid; t < PIECE; t += NT)
+        *reinterpret_cast<uint4*>(s_b + sur::kmajor_offset((uint32_t)t, 8, 16)) =
             make_uint4(0x3c00u, 0u, 0u, 0u);
     sur::fence_async_shared();
-    uint32_t phase = 0, mphase = 0;   // mphase: bit b, the phase of s_mbar[b]
+    uint32_t phase = 0, mphase = 0;
     if (lane < 4) s_ru[w][lane] = 0u;
     if (tid < 9)
         s_shift[tid] = make_float2((float)(tid % 3 - 1) * d.csf, (float)(tid / 3 - 1) * d.csf);
@@ -479,10 +475,9 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
         ok = mbar_wait_bounded(&s_bar, phase);
         phase ^= 1u;
         // The staged candidates go through the tensor cores in pieces of
-        // PIECE; piece k uses operand buffer and accumulator k & 1.
-        // Candidate t of a piece is row (t mod SPLIT) kPartCols + t / SPLIT of
-        // operand B, so a part's accumulator columns are contiguous and the
-        // parts take alternate candidates.
+        // PIECE.  Candidate t of a piece is row (t mod SPLIT) kPartCols + t /
+        // SPLIT of operand B, so a part's accumulator columns are contiguous
+        // and the parts take alternate candidates.
         const uint32_t nst = s_base[9];
         const uint32_t npc = (nst + PIECE - 1) / PIECE;
         // 32 rows of piece k: shift the candidates' y, z into the frame of
@@ -491,8 +486,8 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
         auto build = [&](uint32_t k, uint32_t g) {
             const uint32_t t = g * 32u + (uint32_t)lane;
             const uint32_t j = k * PIECE + t;
-            unsigned char* row = s_b + (k & 1u) * (PIECE * 32) +
-                                 sur::kmajor_offset((t % SPLIT) * kPartCols + t / SPLIT, 0, 16);
+            unsigned char* row =
+                s_b + sur::kmajor_offset((t % SPLIT) * kPartCols + t / SPLIT, 0, 16);
             if (j < nst) {
                 int r = 0;
 #pragma unroll
@@ -510,32 +505,23 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
             }
             sur::fence_async_shared();
         };
-        auto issue = [&](uint32_t k) {                   // by one thread
-            const uint32_t b = k & 1u;
+        auto issue = [&]() {                             // by one thread
             sur::tc_fence_after();
-            sur::tc_mma(tmem + b * PIECE, sur::smem_desc(smem_u32(s_a), sur::kLBO, 256),
-                        sur::smem_desc(smem_u32(s_b + b * (PIECE * 32)), sur::kLBO, 256),
-                        idesc_half(PIECE), 0u);
-            sur::tc_commit(&s_mbar[b]);
+            sur::tc_mma(tmem, sur::smem_desc(smem_u32(s_a), sur::kLBO, 256),
+                        sur::smem_desc(smem_u32(s_b), sur::kLBO, 256), idesc_half(PIECE), 0u);
+            sur::tc_commit(&s_mbar);
         };
         PairAcc2 acc2 = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f), 0.f};
         const bool anyfluid = __any_sync(kFull, fluid);
         uint32_t lp = list0, hits = 0;                  // next word of this lane's list, its hits
-#pragma unroll
-        for (uint32_t k = 0; k < 2; ++k) {
-            const uint32_t g = (uint32_t)(w + NW - (int)k * kBuilders % NW) % NW;
-            if (k < npc && g < kBuilders) build(k, g);
-        }
+        for (int g = w; g < kBuilders; g += NW) build(0, g);
         sur::fence_async_shared();
         if (__syncthreads_and(ok) == 0) {
             if (tid == 0) atomicOr(a.status, kStatusTimeout);
             mbar_wait_bounded(&s_bar, phase ^ 1u);   // let copies in flight land first
             break;
         }
-        if (tid == 0) {
-            issue(0);
-            if (npc > 1) issue(1);
-        }
+        if (tid == 0) issue();
         if (tid == 0 && nui < nunits) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(s_nx + 2)),
@@ -578,24 +564,22 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                 next_window();
             }
             while (k < npc) {
-                const uint32_t b = k & 1u;
-                const bool more = k + 2 < npc;
+                const bool more = k + 1 < npc;
                 if (!in_piece) {
-                    ok = __all_sync(kFull, mbar_sleep_bounded(&s_mbar[b], (mphase >> b) & 1u));
+                    ok = __all_sync(kFull, mbar_sleep_bounded(&s_mbar, mphase));
                     if (!ok) break;
-                    mphase ^= 1u << b;
+                    mphase ^= 1u;
                     sur::tc_fence_after();
-                    // piece k + 2's rows into the buffer that piece k's MMA has read
+                    // the next piece's rows, now that the MMA has read this one's
                     if (more) {
-                        const uint32_t g = (uint32_t)(w + NW - (int)(k % NW) * kBuilders % NW) % NW;
-                        if (g < kBuilders) build(k + 2, g);
+                        for (int g = w; g < kBuilders; g += NW) build(k + 1, g);
                         __syncwarp();
                     }
                     c = 0;
                     in_piece = true;
                 }
                 const uint32_t p0 = k * PIECE, p1 = p0 + PIECE;
-                const uint32_t tcol = lane_base + b * PIECE + part * kPartCols;
+                const uint32_t tcol = lane_base + part * kPartCols;
                 const uint32_t e0 = (p0 + part) * 16u;
                 while (wa < p1) {
                     // columns [ca, cb) of this part: candidates p0 + SPLIT c + part.
@@ -637,15 +621,15 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                     break;
                 }
                 if (more) {
-                    // the last warp done with the piece issues the MMA of k + 2
+                    // the last warp done with the piece issues the next one's MMA
                     sur::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) {
                         __threadfence_block();
-                        if (atomicAdd(&s_arr[b], 1u) == (uint32_t)NW - 1u) {
+                        if (atomicAdd(&s_arr, 1u) == (uint32_t)NW - 1u) {
                             __threadfence_block();
-                            s_arr[b] = 0u;
-                            issue(k + 2);
+                            s_arr = 0u;
+                            issue();
                         }
                     }
                     __syncwarp();
@@ -710,8 +694,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
         if (!ok) {
             if (tid == 0) atomicOr(a.status, kStatusTimeout);
             // let an MMA in flight land first
-            mbar_wait_bounded(&s_mbar[0], mphase & 1u);
-            mbar_wait_bounded(&s_mbar[1], (mphase >> 1) & 1u);
+            mbar_wait_bounded(&s_mbar, mphase);
             break;
         }
         add_pairs2(d, acc2, acc);
@@ -853,7 +836,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
 
     sur::tc_fence_before();
     __syncthreads();
-    if (w == 0) sur::tmem_dealloc(tmem, COLS);
+    if (w == 0) sur::tmem_dealloc(tmem, PIECE);
     if (tid == 0) {
         uint4 u = make_uint4(0u, 0u, 0u, 0u);
         for (int k = 0; k < NW; ++k) {
@@ -891,27 +874,28 @@ Variant tc_variant() {
     v.fn[1][0] = k_interact_tc<W, SPLIT, STAGE, WCAP, PIECE, MINB, false, 1>;
     v.fn[1][1] = k_interact_tc<W, SPLIT, STAGE, WCAP, PIECE, MINB, true, 1>;
     v.smem = TcShape<W, SPLIT, STAGE, WCAP, PIECE>::smem;
-    v.max_per_sm = 512 / (2 * PIECE);
+    v.max_per_sm = 512 / PIECE;
     return v;
 }
 
 }  // namespace
 
 // Large systems run best in 128-particle units on two blocks per SM, small
-// ones in 64-particle units on four (sph_autotune times them all; ms per
-// launch on one GB300: 35.4M particles 20.4 against 28.0, 1.39M 0.778 / 0.999,
-// 17k 0.0237 / 0.0220).  Between the first three, shared memory moves from
-// staged candidates to hit words: 1,664 / 18 take 20.4 / 0.778 ms, 1,536 / 20
-// 20.8 / 0.777, 1,408 / 22 21.9 / 0.803, 1,856 / 15 20.6 / 0.783.
+// ones and ensembles of small ones in 64-particle units on four (sph_autotune
+// times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.8 /
+// 24.0, 1.39M 0.717 / 0.862, 60k 0.073 / 0.076, 256 dam breaks 3.20 / 3.13, 17k
+// 0.0223 / 0.0200).  Between the first and the third, fourth and seventh,
+// shared memory moves from staged candidates to hit words (larger h/dp has more
+// hits per particle): 1,664 / 18 take 18.9 / 0.724 ms.
 Variant tc_variant_n(int k) {
     switch (k) {
-        case 0: return tc_variant<4, 2, 1664, 18, 128, 2>();
-        case 1: return tc_variant<2, 2, 832, 18, 64, 4>();
-        case 2: return tc_variant<4, 2, 1536, 20, 128, 2>();
-        case 3: return tc_variant<4, 2, 1280, 24, 128, 2>();
-        case 4: return tc_variant<2, 2, 1024, 15, 64, 4>();
-        case 5: return tc_variant<1, 4, 768, 14, 64, 4>();
-        default: return tc_variant<4, 2, 1856, 15, 128, 2>();
+        case 0: return tc_variant<4, 2, 1760, 16, 256, 2>();
+        case 1: return tc_variant<2, 2, 896, 16, 128, 4>();
+        case 2: return tc_variant<4, 2, 1664, 18, 256, 2>();
+        case 3: return tc_variant<4, 2, 1536, 20, 256, 2>();
+        case 4: return tc_variant<2, 2, 832, 18, 128, 4>();
+        case 5: return tc_variant<1, 4, 768, 14, 128, 4>();
+        default: return tc_variant<4, 2, 1408, 22, 256, 2>();
     }
 }
 
