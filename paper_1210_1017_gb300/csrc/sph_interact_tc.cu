@@ -19,9 +19,9 @@
 // latency but cost a hundred instructions per warp and piece: 20.4 against
 // 18.8 ms at 35.4M particles.)  Both sides on one GB300, ms per launch (the
 // counter-scheduled 4 x 2 shape of sph_kernels.cu / this kernel): 35.4M
-// particles 24.0 / 18.8, 1.39M with obstacles 0.956 / 0.717, 256 dam breaks
-// (5.5M) 3.85 / 3.13, 64k with the cubic spline 0.094 / 0.073, 17k 0.0229 /
-// 0.0200.  Next to the pair phase (0.23 ms of it at 1.39M) the largest share is
+// particles 24.0 / 18.8, 1.39M with obstacles 0.956 / 0.713, 256 dam breaks
+// (5.5M) 3.85 / 3.12, 64k with the cubic spline 0.094 / 0.073, 17k 0.0229 /
+// 0.0196.  Next to the pair phase (0.23 ms of it at 1.39M) the largest share is
 // the units' set-up, 0.20: the latency of the staging copies.
 #include <cuda_fp16.h>
 #include <math.h>
@@ -200,6 +200,15 @@ struct TcShape {
     static_assert(PIECE % (8 * SPLIT) == 0 && PIECE % 32 == 0, "a piece's columns and rows");
 };
 
+// Largest of a warp's values; a NaN counts only if all of them are NaN.  (Five
+// shuffles and maxima before, three times per warp and unit: 17k particles
+// 0.0200 -> 0.0196 ms, 1.39M 0.717 -> 0.713.)
+__device__ __forceinline__ float warp_max(float v) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+
 // mbar_wait_bounded with the thread suspended for up to 1 us per try (fewer
 // polls: they take issue slots from the warps that compute).
 __device__ __forceinline__ bool mbar_sleep_bounded(uint64_t* bar, uint32_t parity) {
@@ -267,7 +276,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
     constexpr int NW = W * SPLIT, NT = NW * 32;
     constexpr int FBCAP = SH::fb_cap;
     constexpr uint32_t kPad = (uint32_t)STAGE * 16u;       // list entry of the pad slot
-        constexpr uint32_t kPartCols = PIECE / SPLIT;          // of one part of a piece
+    constexpr uint32_t kPartCols = PIECE / SPLIT;          // of one part of a piece
     constexpr int kBuilders = PIECE / 32;                  // groups of 32 rows of a piece
     static_assert(NW >= 4 && (PIECE == 128 || PIECE == 256), "TMEM lane quarters and columns");
     extern __shared__ __align__(128) unsigned char s_raw[];
@@ -804,11 +813,9 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
         if (!(am == am)) am = 0.f;
         float cm = valid ? ci : 0.f;
         float mm = (valid && fluid) ? acc.mu : 0.f;
-        for (int o = 16; o; o >>= 1) {
-            am = fmaxf(am, __shfl_xor_sync(kFull, am, o));
-            cm = fmaxf(cm, __shfl_xor_sync(kFull, cm, o));
-            mm = fmaxf(mm, __shfl_xor_sync(kFull, mm, o));
-        }
+        am = warp_max(am);
+        cm = warp_max(cm);
+        mm = warp_max(mm);
         if (lane == 0 && act) {
             atomicMax(d.is.terms + 3 * q + 0, __float_as_uint(am));
             atomicMax(d.is.terms + 3 * q + 1, __float_as_uint(cm));
@@ -883,10 +890,10 @@ Variant tc_variant() {
 // Large systems run best in 128-particle units on two blocks per SM, small
 // ones and ensembles of small ones in 64-particle units on four (sph_autotune
 // times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.8 /
-// 24.0, 1.39M 0.717 / 0.862, 60k 0.073 / 0.076, 256 dam breaks 3.20 / 3.13, 17k
-// 0.0223 / 0.0200).  Between the first and the third, fourth and seventh,
+// 24.0, 1.39M 0.713 / 0.858, 60k 0.073 / 0.076, 256 dam breaks 3.18 / 3.12, 17k
+// 0.0212 / 0.0196).  Between the first and the third, fourth and seventh,
 // shared memory moves from staged candidates to hit words (larger h/dp has more
-// hits per particle): 1,664 / 18 take 18.9 / 0.724 ms.
+// hits per particle): 1,664 / 18 take 18.8 / 0.719 ms.
 Variant tc_variant_n(int k) {
     switch (k) {
         case 0: return tc_variant<4, 2, 1760, 16, 256, 2>();
