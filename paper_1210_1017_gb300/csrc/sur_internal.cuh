@@ -69,6 +69,27 @@ struct EdgeArgs {
     uint32_t* status;
 };
 
+// Backward pass of that update over the M edges, sorted by src, given the
+// gradient dE of e' (fp32, updated in place):
+//   v = dE + node[src]; dpre = v W2^T where z > 0, else 0; dE = v + dpre W1c^T
+// W1, W2 (kin x kout, row-major).  part_v, part_p: column sums of v and dpre,
+// one row of 128 per half-block (nparts of them, 2 x num_sms() at most).
+struct EdgeBwdArgs {
+    float* dE;
+    const float* node;          // row stride ldn (a multiple of 4)
+    uint32_t ldn;
+    const uint32_t* src;
+    const __nv_bfloat16* Z;
+    const __nv_bfloat16* W1;
+    const __nv_bfloat16* W2;
+    uint32_t M;
+    __nv_bfloat16* dEb;         // v as bf16
+    __nv_bfloat16* dpre;
+    float* part_v;
+    float* part_p;
+    uint32_t* status;
+};
+
 int num_sms();
 bool launch_linear(int K, int N, const LinearArgs& g, cudaStream_t st);
 // False when the driver has no tensor maps for the tiles (nothing launched).
@@ -76,6 +97,7 @@ bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st);
 // The edge encoder in one kernel: E (M x 16) -> Eout = relu(E W1 + b1) W2 + b2
 // (z = relu(E W1 + b1) to Z when Z != null); P, Q, src, dst unused.
 bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st);
+bool launch_edge_backward(const EdgeBwdArgs& g, uint32_t* nparts, cudaStream_t st);
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st);
 
 }  // namespace sur

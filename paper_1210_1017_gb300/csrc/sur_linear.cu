@@ -861,6 +861,292 @@ __global__ void __launch_bounds__(512, 1)
 template <int K, int N>
 size_t linear_smem() { return (size_t)2 * 128 * K * 2 + (size_t)N * K * 2; }
 
+// Sums of 16 columns over the 32 rows (lanes) of a warp: lane l gets column
+// l mod 16, added in a fixed tree (16 shuffles).
+__device__ __forceinline__ float warp_colsum16(const float (&v)[16], int lane) {
+    float a[8], b[4], c[2], d;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float keep = lane & 8 ? v[i + 8] : v[i], give = lane & 8 ? v[i] : v[i + 8];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float keep = lane & 4 ? a[i + 4] : a[i], give = lane & 4 ? a[i] : a[i + 4];
+        b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float keep = lane & 2 ? b[i + 2] : b[i], give = lane & 2 ? b[i] : b[i + 2];
+        c[i] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+    }
+    d = (lane & 1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, lane & 1 ? c[0] : c[1], 1);
+    return d + __shfl_xor_sync(0xffffffffu, d, 16);
+}
+
+// The backward pass of the fused edge update, per 128-edge tile:
+//   v = dE + node[src],  dpre = v W2^T where z > 0 and 0 elsewhere,
+//   dE = v + dpre W1c^T
+// with bf16 copies of v and dpre for the weight gradients and the column sums
+// of v (FP32) and dpre for the bias gradients.  Two independent halves of 256
+// threads per block, as in k_edge_pp, a thread per row and 64 columns.
+//
+// Bound by HBM: dE in and out, z in, both copies out, 1,792 B per edge; as five
+// kernels (gather, two layers, column sums) the same work moved 3,600 B.  The
+// bf16 tiles go by TMA in the 128-byte swizzle (dpre over z in place), the dE
+// rows by 32-byte accesses a tile ahead, through registers; v waits in TMEM
+// for the second product and is added to it in FP32.  Edges are sorted by src,
+// so the lanes of a gathering warp share one or two node rows.  The column
+// sums of v come from the rows in registers by shuffles, those of dpre from
+// the tile in shared memory, each tile summed for itself first.
+// On one GB300, 976k edges: 770 us as five kernels, 401 as one (4.4 TB/s of
+// those bytes, 64% of the copy bandwidth).
+constexpr size_t kEdgeBwdSmem = (size_t)6 * kETile + 1024;   // W2, W1c, 2 x (v, z) tiles; alignment
+
+__global__ void __launch_bounds__(512, 1)
+    k_edge_bwd(const EdgeBwdArgs g, const __grid_constant__ CUtensorMap map_z,
+               const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_p,
+               const bool wide) {
+    constexpr int N = 128;
+    constexpr uint32_t T = kETile, BOX = T / 2;          // a box: 64 columns of 128 rows
+    extern __shared__ unsigned char s_dyn[];
+    // completions of MMA 1 and MMA 2, z tile loaded, per half
+    __shared__ __align__(8) uint64_t s_bar[2][2], s_full[2];
+    __shared__ uint32_t s_tmem;
+    __shared__ float s_ce[2][4][N], s_cp[2][4][N];       // column sums of the half's row groups
+    unsigned char* s_raw = s_dyn + ((1024u - (sm_addr(s_dyn) & 1023u)) & 1023u);
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int h = tid >> 8, lt = tid & 255;              // half, thread within the half
+    unsigned char* sw2 = s_raw;                          // W2
+    unsigned char* sw1 = s_raw + T;                      // W1c
+    unsigned char* sv = s_raw + (2 + 2 * h) * T;         // v as bf16
+    unsigned char* sz = sv + T;                          // z, then dpre
+    if (w == 0) tmem_alloc(&s_tmem, 512);
+    if (tid == 0)
+        for (int k = 0; k < 2; ++k) {
+            mbar_init1(&s_bar[k][0]);
+            mbar_init1(&s_bar[k][1]);
+            mbar_init1(&s_full[k]);
+        }
+    for (int c = tid; c < N * (N / 8); c += 512) {
+        const int r = c % N, gk = c / N;
+        cp_async16(sw2 + kmajor_offset(r, gk * 8, N), g.W2 + (size_t)r * N + gk * 8, true);
+        cp_async16(sw1 + kmajor_offset(r, gk * 8, N), g.W1 + (size_t)r * N + gk * 8, true);
+    }
+    cp_async_wait_all();
+    fence_async_shared();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t ntiles = (g.M + 127) / 128;
+    const uint32_t stride = 2 * gridDim.x;
+    const int wq = w & 3, part = (w >> 2) & 1;           // lane quarter, column half
+    const int r = wq * 32 + lane;                        // this thread's row of a tile
+    const bool mover = lt == 32;                         // moves the half's tiles
+    const uint32_t quarter = (uint32_t)(wq * 32) << 16;
+    const uint32_t tv = s_tmem + (uint32_t)(h * 256) + quarter;       // v
+    const uint32_t tx = s_tmem + (uint32_t)(h * 256) + 128u;          // the products
+    auto load_z = [&](uint32_t t) {
+        mbar_expect(&s_full[h], T);
+        tma_load(sz, &map_z, 0, (int)(t * 128), &s_full[h]);
+        tma_load(sz + BOX, &map_z, 64, (int)(t * 128), &s_full[h]);
+    };
+    uint4 dv[16];                                        // dE of the tile in hand: 64 columns
+    auto load_de = [&](uint32_t m) {
+        const uint4* p = reinterpret_cast<const uint4*>(g.dE + (size_t)(m < g.M ? m : 0u) * N + part * 64);
+        if (m >= g.M) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) dv[k] = make_uint4(0u, 0u, 0u, 0u);
+        } else if (wide) {
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) ld32(p + k, dv[k], dv[k + 1]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) dv[k] = p[k];
+        }
+    };
+    // D = A B^T of the tile `a` (128-byte swizzle) and weights `b` (one thread)
+    auto mma = [&](const unsigned char* a, const unsigned char* b, uint64_t* bar) {
+        tc_fence_after();
+#pragma unroll
+        for (int s = 0; s < N / 16; ++s) {
+            const uint64_t ad = smem_desc_sw128(sm_addr(a) + (s >> 2) * BOX + (s & 3) * 32);
+            const uint64_t bd = smem_desc(sm_addr(b) + s * 256, kLBO, (N / 8) * 128);
+            tc_mma(tx, ad, bd, idesc_bf16(N), s > 0 ? 1u : 0u);
+        }
+        tc_commit(bar);
+    };
+    float ce[4] = {0.f, 0.f, 0.f, 0.f};                  // columns part 64 + 16 k + lane mod 16 of v
+    float cp[2] = {0.f, 0.f};                            // columns 2 (lt mod 64) and + 1 of dpre
+    uint32_t tile = 2 * blockIdx.x + (uint32_t)h;
+    uint32_t row = 0;                                    // node row of this thread's edge
+    if (tile < ntiles) {
+        if (mover) load_z(tile);
+        const uint32_t m = tile * 128 + (uint32_t)r;
+        load_de(m);
+        if (m < g.M) row = __ldg(g.src + m);
+    }
+    uint32_t phase = 0;
+    bool ok = true;
+    for (; tile < ntiles; tile += stride) {
+        const uint32_t m = tile * 128 + (uint32_t)r;
+        const uint32_t next = tile + stride;
+        // v = dE + node[src]: to TMEM, as bf16 to the tile, into the column sums
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint4 q[4] = {};
+            if (m < g.M) {
+                const uint4* p = reinterpret_cast<const uint4*>(g.node + (size_t)row * g.ldn + part * 64 + 16 * k);
+                if (wide) {
+                    ldg32(p, q[0], q[1]);
+                    ldg32(p + 2, q[2], q[3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) q[i] = __ldg(p + i);
+                }
+            }
+            float v[16];
+            uint32_t u[16];
+            __nv_bfloat162 hh[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint4 e = dv[4 * k + i];
+                v[4 * i] = __uint_as_float(e.x) + __uint_as_float(q[i].x);
+                v[4 * i + 1] = __uint_as_float(e.y) + __uint_as_float(q[i].y);
+                v[4 * i + 2] = __uint_as_float(e.z) + __uint_as_float(q[i].z);
+                v[4 * i + 3] = __uint_as_float(e.w) + __uint_as_float(q[i].w);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) u[i] = __float_as_uint(v[i]);
+            tmem_st8(tv + (uint32_t)(part * 64 + 16 * k), u);
+            tmem_st8(tv + (uint32_t)(part * 64 + 16 * k + 8), u + 8);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) hh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            *reinterpret_cast<uint4*>(sv + part * BOX + sw128_offset(r, 2 * k)) =
+                *reinterpret_cast<uint4*>(&hh[0]);
+            *reinterpret_cast<uint4*>(sv + part * BOX + sw128_offset(r, 2 * k + 1)) =
+                *reinterpret_cast<uint4*>(&hh[4]);
+            ce[k] += warp_colsum16(v, lane);
+        }
+        tmem_st_wait();
+        fence_async_shared();
+        tc_fence_before();
+        ok = half_and(h, ok);                            // v complete, the products' columns free
+        if (!ok) break;
+        if (lt == 0) mma(sv, sw2, &s_bar[h][0]);
+        if (mover) {
+            tma_store(&map_v, sv, 0, (int)(tile * 128));
+            tma_store(&map_v, sv + BOX, 64, (int)(tile * 128));
+            bulk_commit();
+        }
+        // the next tile's rows
+        if (next < ntiles) {
+            const uint32_t m1 = next * 128 + (uint32_t)r;
+            load_de(m1);
+            row = m1 < g.M ? __ldg(g.src + m1) : 0u;
+        }
+        bool got = mbar_wait(&s_bar[h][0], phase);
+        got = mbar_wait(&s_full[h], phase) && got;
+        tc_fence_after();
+        // dpre over z
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c0 = part * 64 + 16 * k;
+            float v[16], t[16];
+            tmem_ld16(tx + quarter + c0, v);
+            uint4* z0 = reinterpret_cast<uint4*>(sz + part * BOX + sw128_offset(r, 2 * k));
+            uint4* z1 = reinterpret_cast<uint4*>(sz + part * BOX + sw128_offset(r, 2 * k + 1));
+            unpack8(*z0, t);
+            unpack8(*z1, t + 8);
+            __nv_bfloat162 hh[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                hh[i] = __floats2bfloat162_rn(t[2 * i] > 0.f ? v[2 * i] : 0.f,
+                                              t[2 * i + 1] > 0.f ? v[2 * i + 1] : 0.f);
+            *z0 = *reinterpret_cast<uint4*>(&hh[0]);
+            *z1 = *reinterpret_cast<uint4*>(&hh[4]);
+        }
+        fence_async_shared();
+        tc_fence_before();
+        ok = half_and(h, got);                           // dpre complete
+        if (!ok) break;
+        if (lt == 0) mma(sz, sw1, &s_bar[h][1]);
+        if (mover) {
+            tma_store(&map_p, sz, 0, (int)(tile * 128));
+            tma_store(&map_p, sz + BOX, 64, (int)(tile * 128));
+            bulk_commit();
+        }
+        {   // column sums of dpre: two columns and 32 rows per thread
+            const uint32_t pr = (uint32_t)lt & 63u, r0 = (uint32_t)(lt >> 6) * 32u;
+            const unsigned char* col = sz + (pr >> 5) * BOX + (pr & 3u) * 4u;
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+            for (uint32_t i = 0; i < 32; ++i) {
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(
+                    col + sw128_offset(r0 + i, (pr & 31u) >> 2)));
+                s0 += f.x;
+                s1 += f.y;
+            }
+            cp[0] += s0;
+            cp[1] += s1;
+        }
+        got = mbar_wait(&s_bar[h][1], phase);
+        tc_fence_after();
+        if (mover) bulk_wait_read();                     // both copies have been read
+        ok = half_and(h, got);                           // the tiles are free
+        if (!ok) break;
+        if (mover && next < ntiles) load_z(next);
+        // dE = v + dpre W1c^T
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c0 = part * 64 + 16 * k;
+            float v[16], x[16];
+            tmem_ld16(tv + c0, v);
+            tmem_ld16(tx + quarter + c0, x);
+            if (m < g.M) {
+                uint4 o[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    o[i] = make_uint4(__float_as_uint(x[4 * i] + v[4 * i]),
+                                      __float_as_uint(x[4 * i + 1] + v[4 * i + 1]),
+                                      __float_as_uint(x[4 * i + 2] + v[4 * i + 2]),
+                                      __float_as_uint(x[4 * i + 3] + v[4 * i + 3]));
+                uint4* p = reinterpret_cast<uint4*>(g.dE + (size_t)m * N + c0);
+                if (wide) {
+                    stg32(p, o[0], o[1]);
+                    stg32(p + 2, o[2], o[3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p[i] = o[i];
+                }
+            }
+        }
+        phase ^= 1u;
+    }
+    if (!ok) {
+        if (lt == 0 && g.status) atomicOr(g.status, 1u);
+        mbar_wait(&s_bar[h][0], phase);                  // let MMAs and copies in flight
+        mbar_wait(&s_bar[h][1], phase);                  // land first
+        mbar_wait(&s_full[h], phase);
+    }
+    if (mover) bulk_wait();
+    if (lane < 16) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s_ce[h][wq][part * 64 + 16 * k + lane] = ce[k];
+    }
+    s_cp[h][lt >> 6][2 * (lt & 63)] = cp[0];
+    s_cp[h][lt >> 6][2 * (lt & 63) + 1] = cp[1];
+    tc_fence_before();
+    __syncthreads();
+    if (w == 0) tmem_dealloc(s_tmem, 512);
+    {
+        const int c = lt & 127;
+        const float(*s)[N] = lt < 128 ? s_ce[h] : s_cp[h];
+        float* out = lt < 128 ? g.part_v : g.part_p;
+        out[(size_t)(2 * blockIdx.x + h) * N + c] = ((s[0][c] + s[1][c]) + s[2][c]) + s[3][c];
+    }
+}
+
 template <int K, int N>
 void launch_linear_t(const LinearArgs& g, int sms, cudaStream_t st) {
     static bool init = false;
@@ -984,6 +1270,25 @@ bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st) {
     uint32_t grid = (uint32_t)num_sms();
     if (grid > (tiles + 1) / 2) grid = (tiles + 1) / 2;
     k_edge_pp<<<grid, 512, kEdgePPSmem, st>>>(g, map_e, map_out, all % 32u == 0u);
+    return true;
+}
+
+bool launch_edge_backward(const EdgeBwdArgs& g, uint32_t* nparts, cudaStream_t st) {
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_edge_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEdgeBwdSmem);
+    });
+    *nparts = 0;
+    if (g.M == 0) return true;
+    CUtensorMap map_z, map_v, map_p;
+    if (!tile_map(&map_z, g.Z, g.M) || !tile_map(&map_v, g.dEb, g.M) || !tile_map(&map_p, g.dpre, g.M))
+        return false;
+    const uintptr_t all = reinterpret_cast<uintptr_t>(g.dE) | reinterpret_cast<uintptr_t>(g.node);
+    const uint32_t tiles = (g.M + 127) / 128;
+    uint32_t grid = (uint32_t)num_sms();
+    if (grid > (tiles + 1) / 2) grid = (tiles + 1) / 2;
+    *nparts = 2 * grid;
+    k_edge_bwd<<<grid, 512, kEdgeBwdSmem, st>>>(g, map_z, map_v, map_p, all % 32u == 0u && g.ldn % 8u == 0u);
     return true;
 }
 

@@ -278,28 +278,15 @@ __global__ void __launch_bounds__(256) k_colsum_bf16(uint32_t M, int C,
     colsum_block<8>(s, C, part);
 }
 
-// The rows of an (M x 128) fp32 matrix: acc += node[src] (with GATHER; row
-// stride ldn), a bf16 copy, and the column sums of the result.
-template <bool GATHER>
-__global__ void __launch_bounds__(256) k_rows_f32(uint32_t M, float* __restrict__ acc,
-                                                  const float* __restrict__ node,
-                                                  const uint32_t* __restrict__ src, uint32_t ldn,
+// The rows of an (M x 128) fp32 matrix: a bf16 copy and the column sums.
+__global__ void __launch_bounds__(256) k_rows_f32(uint32_t M, const float* __restrict__ acc,
                                                   __nv_bfloat16* __restrict__ out_bf,
                                                   float* __restrict__ part) {
     const uint32_t col = (threadIdx.x & 31) * 4, step = gridDim.x * 8;
     float s[4] = {};
 #pragma unroll 4
     for (uint32_t m = blockIdx.x * 8 + threadIdx.x / 32; m < M; m += step) {
-        float4* p = reinterpret_cast<float4*>(acc + (size_t)m * L + col);
-        float4 v = *p;
-        if (GATHER) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(node + (size_t)src[m] * ldn + col));
-            v.x += q.x;
-            v.y += q.y;
-            v.z += q.z;
-            v.w += q.w;
-            *p = v;
-        }
+        const float4 v = __ldg(reinterpret_cast<const float4*>(acc + (size_t)m * L + col));
         const __nv_bfloat162 b0 = __floats2bfloat162_rn(v.x, v.y), b1 = __floats2bfloat162_rn(v.z, v.w);
         *reinterpret_cast<uint2*>(out_bf + (size_t)m * L + col) = make_uint2(
             *reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
@@ -311,21 +298,25 @@ __global__ void __launch_bounds__(256) k_rows_f32(uint32_t M, float* __restrict_
     colsum_block<4>(s, L, part);
 }
 
-// out[c] = the sum of the partials, 1024 / C slices of them in parallel.
+// out[c] = the sum of the partials: a block takes up to 32 columns, 1024 / 32
+// slices of the partials in parallel.  (One block for all columns had 76 loads
+// in a row per thread at 608 partials: 14 us.)
 __global__ void __launch_bounds__(1024) k_colsum_final(int nparts, int C,
                                                        const float* __restrict__ part,
                                                        float* __restrict__ out) {
     __shared__ float s_sum[1024];
-    const int c = threadIdx.x % C, g = threadIdx.x / C, ng = 1024 / C;
+    const int nc = C < 32 ? C : 32;
+    const int c = threadIdx.x % nc, g = threadIdx.x / nc, ng = 1024 / nc;
+    const int col = blockIdx.x * nc + c;
     float s = 0.f;
-#pragma unroll 4
-    for (int b = g; b < nparts; b += ng) s += part[(size_t)b * C + c];
+#pragma unroll 8
+    for (int b = g; b < nparts; b += ng) s += part[(size_t)b * C + col];
     s_sum[threadIdx.x] = s;
     __syncthreads();
-    if (threadIdx.x >= C) return;
+    if (threadIdx.x >= nc) return;
     float t = 0.f;
-    for (int k = 0; k < ng; ++k) t += s_sum[k * C + c];
-    out[c] = t;
+    for (int k = 0; k < ng; ++k) t += s_sum[k * nc + c];
+    out[col] = t;
 }
 
 // Loss over fluid nodes and its gradient: out (n x 16 fp32, sorted order),
@@ -744,23 +735,47 @@ uint32_t col_parts(uint32_t M, uint32_t rpb) {
     return b == 0 ? 1u : (b < kColParts ? b : kColParts);
 }
 
+// out[0:C] = the sums of `parts` partials of C columns (C = 16 or 128).
+void colsum_final(sur_ctx* c, uint32_t parts, int C, const float* part, float* out) {
+    k_colsum_final<<<C < 32 ? 1 : C / 32, 1024, 0, c->st>>>((int)parts, C, part, out);
+}
+
 // Column sums of an (M x C) bf16 matrix into out[0:C].
 void colsum(sur_ctx* c, const __nv_bfloat16* in, uint32_t M, int C, uint32_t ld, float* out) {
     const uint32_t parts = col_parts(M, 256 / (C / 8));
     k_colsum_bf16<<<parts, 256, 0, c->st>>>(M, C, in, ld, c->colpart);
-    k_colsum_final<<<1, 1024, 0, c->st>>>((int)parts, C, c->colpart, out);
+    colsum_final(c, parts, C, c->colpart, out);
 }
 
-// acc (M x 128 fp32) += node[src] when node != null; bf16 copy to out_bf,
-// column sums to out.
-void rows_f32(sur_ctx* c, float* acc, uint32_t M, const float* node, const uint32_t* src,
-              uint32_t ldn, __nv_bfloat16* out_bf, float* out) {
+// bf16 copy of acc (M x 128 fp32) to out_bf, column sums to out.
+void rows_f32(sur_ctx* c, const float* acc, uint32_t M, __nv_bfloat16* out_bf, float* out) {
     const uint32_t parts = col_parts(M, 8);
-    if (node)
-        k_rows_f32<true><<<parts, 256, 0, c->st>>>(M, acc, node, src, ldn, out_bf, c->colpart);
-    else
-        k_rows_f32<false><<<parts, 256, 0, c->st>>>(M, acc, nullptr, nullptr, 0, out_bf, c->colpart);
-    k_colsum_final<<<1, 1024, 0, c->st>>>((int)parts, L, c->colpart, out);
+    k_rows_f32<<<parts, 256, 0, c->st>>>(M, acc, out_bf, c->colpart);
+    colsum_final(c, parts, L, c->colpart, out);
+}
+
+// The backward pass of edge_layer (dE, dEb, dpre and both bias gradients).
+int edge_backward(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* z) {
+    EdgeBwdArgs g = {};
+    g.dE = c->dE;
+    g.node = c->dXN + L;
+    g.ldn = 2 * L;
+    g.src = c->src;
+    g.Z = z;
+    g.W1 = l1.W;
+    g.W2 = l2.W;
+    g.M = c->E;
+    g.dEb = c->dEb;
+    g.dpre = c->dpre;
+    g.part_v = c->colpart;
+    g.part_p = c->colpart + (size_t)1024 * L;
+    uint32_t parts = 0;
+    if (!launch_edge_backward(g, &parts, c->st)) return fail(c, SPH_ERR_CUDA, "edge layer: no tensor maps");
+    if (parts) {
+        colsum_final(c, parts, L, g.part_v, c->g + l2.b_off);
+        colsum_final(c, parts, L, g.part_p, c->g + l1.b_off);
+    }
+    return SPH_OK;
 }
 
 void refresh_all(sur_ctx* c) {
@@ -897,7 +912,7 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         __nv_bfloat16* z1 = c->Z1[l];
         __nv_bfloat16* y1 = c->Y1[l];
         // node update h' = h + W4 relu(W3 [h, agg] + b3) + b4
-        rows_f32(c, c->dH, n, nullptr, nullptr, 0, c->dHb, c->g + w[5].b_off);
+        rows_f32(c, c->dH, n, c->dHb, c->g + w[5].b_off);
         wgrad(c, w[5], y1, L, c->dHb, L, n);
         if ((rc = linear(c, c->dHb, 0, w[5], true, n, kEpiReluMask, y1, L, c->dY1, nullptr, L))) return rc;
         colsum(c, c->dY1, n, L, L, c->g + w[4].b_off);
@@ -906,12 +921,9 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         if ((rc = linear(c, c->dY1, 0, w[4], true, n, kEpiNone, nullptr, 0, nullptr, c->dXN, 2 * L))) return rc;
         k_add_strided<<<nblk((size_t)n * L, 256), 256, 0, st>>>(n, c->dH, c->dXN, 2 * L);
         // aggregation and edge update e' = e + W2 relu(pre) + b2
-        rows_f32(c, c->dE, E, c->dXN + L, c->src, 2 * L, c->dEb, c->g + w[3].b_off);
+        if ((rc = edge_backward(c, w[2], w[3], z1))) return rc;
         wgrad(c, w[3], z1, L, c->dEb, L, E);
-        if ((rc = linear(c, c->dEb, 0, w[3], true, E, kEpiReluMask, z1, L, c->dpre, nullptr, L))) return rc;
-        colsum(c, c->dpre, E, L, L, c->g + w[2].b_off);
         wgrad(c, w[2], e_in, L, c->dpre, L, E);
-        if ((rc = linear(c, c->dpre, 0, w[2], true, E, kEpiAccum, nullptr, 0, nullptr, c->dE, L))) return rc;
         // pre = W1a h_i + W1b h_j + ...: sums over the edges of i and of j
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, c->dpre, nullptr,
                                                                            c->dPb, nullptr, L);
@@ -923,12 +935,12 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         if ((rc = linear(c, c->dQb, 0, w[1], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
     }
     // encoders
-    rows_f32(c, c->dE, E, nullptr, nullptr, 0, c->dEb, c->g + Ls[3].b_off);
+    rows_f32(c, c->dE, E, c->dEb, c->g + Ls[3].b_off);
     wgrad(c, Ls[3], c->ee1, L, c->dEb, L, E);
     if ((rc = linear(c, c->dEb, 0, Ls[3], true, E, kEpiReluMask, c->ee1, L, c->dEe1, nullptr, L))) return rc;
     colsum(c, c->dEe1, E, L, L, c->g + Ls[2].b_off);
     wgrad(c, Ls[2], c->xe, KIN, c->dEe1, L, E);
-    rows_f32(c, c->dH, n, nullptr, nullptr, 0, c->dHb, c->g + Ls[1].b_off);
+    rows_f32(c, c->dH, n, c->dHb, c->g + Ls[1].b_off);
     wgrad(c, Ls[1], c->en1, L, c->dHb, L, n);
     if ((rc = linear(c, c->dHb, 0, Ls[1], true, n, kEpiReluMask, c->en1, L, c->dEn1, nullptr, L))) return rc;
     colsum(c, c->dEn1, n, L, L, c->g + Ls[0].b_off);
