@@ -46,6 +46,16 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
            (1ull << 46) | (2ull << 61);
 }
 
+// A tile whose rows run along K, in boxes of 64 columns (128-byte swizzled rows,
+// 8-row groups 1,024 bytes apart) `box` bytes apart, as an MN-major operand: one
+// MMA step of K = 16 advances the start address by two groups.  kIdescMN marks
+// both operands as such in the instruction descriptor.
+__device__ __forceinline__ uint64_t smem_desc_mn128(uint32_t saddr, uint32_t box) {
+    return (uint64_t)((saddr >> 4) & 0x3fffu) | ((uint64_t)(box >> 4) << 16) |
+           ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+constexpr uint32_t kIdescMN = (1u << 15) | (1u << 16);
+
 // Byte offset of the 16-byte piece c (0..7) of row r in such a tile.
 __device__ __forceinline__ uint32_t sw128_offset(uint32_t r, uint32_t c) {
     return r * 128u + ((c ^ (r & 7u)) << 4);

@@ -313,7 +313,7 @@ __device__ __forceinline__ void store_t(unsigned char* dst, const TRegs<C>& r) {
     }
 }
 
-// Weight gradient dW[C x N] = X^T dY over rows [0, M): X is M x C, dY is
+// Weight gradient dW[C x N] = X^T dY over rows [0, M) for N = 16: X is M x C, dY is
 // M x N (bf16, row-major).  Block b accumulates the row tiles b, b + grid,
 // ... in TMEM (C = 128 rows of the MMA, one MMA chain per tile), then writes
 // its partial; k_wgrad_reduce adds the partials in block order.  The loads
@@ -391,6 +391,111 @@ __global__ void __launch_bounds__(128) k_wgrad(const WgradArgs g) {
     tc_fence_before();
     __syncthreads();
     if (w == 0) tmem_dealloc(tmem, tmem_cols<N>());
+}
+
+// The same for N = 128, the rows by TMA: a tile of 128 rows of X and of dY lands
+// in shared memory as it lies in memory (feature-contiguous, 128-byte swizzle)
+// and is the MMA's operand in that form (both "MN-major": the transposes are the
+// descriptors'), so no register ever holds a row.  Three stages of 64 KB keep
+// 192 KB in flight per SM: one thread loads, one issues the MMAs.  The tiles of
+// a block take turns with four accumulators (the 512 TMEM columns), added in
+// FP32 at the end, so no accumulation chain is longer than with the three
+// blocks per SM of the register version, and the partials are a third as many.
+// Bound by HBM (512 B per row).  On one GB300 with the sum of the partials, us at
+// 976k / 250k / 17k rows: 192 / 76 / 22.5 with rows transposed in registers, 98 /
+// 39 / 16.4 now (5.1 TB/s, 75% of the copy bandwidth); errors against 64 bits
+// 1.5e-8 / 1.4e-8 / 2.1e-8 of the sum of absolute terms before, 1.1e-8 / 5.6e-9 /
+// 9.4e-9 now.
+constexpr int kWgStages = 3, kWgAcc = 4;
+constexpr uint32_t kWgMinTiles = 2;   // tiles per block where there are enough (fewer partials)
+constexpr size_t kWgSmem = (size_t)kWgStages * 2 * 32768 + 1024;
+
+__global__ void __launch_bounds__(128, 1)
+    k_wgrad_tma(const WgradArgs g, const __grid_constant__ CUtensorMap map_x,
+                const __grid_constant__ CUtensorMap map_y) {
+    constexpr int N = 128;
+    constexpr uint32_t T = 128 * 128 * 2, BOX = T / 2;
+    extern __shared__ unsigned char s_dyn[];
+    __shared__ __align__(8) uint64_t s_full[kWgStages], s_empty[kWgStages], s_done;
+    __shared__ uint32_t s_tmem;
+    unsigned char* s_raw = s_dyn + ((1024u - (sm_addr(s_dyn) & 1023u)) & 1023u);
+    const int tid = threadIdx.x, w = tid >> 5;
+    if (w == 0) tmem_alloc(&s_tmem, 512);
+    if (tid == 0) {
+        for (int s = 0; s < kWgStages; ++s) {
+            mbar_init1(&s_full[s]);
+            mbar_init1(&s_empty[s]);
+        }
+        mbar_init1(&s_done);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    const uint32_t ntiles = (g.M + 127) / 128;
+    const uint32_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    bool ok = true;
+    if (tid == 0) {                                      // loads
+        for (uint32_t i = 0; i < mine && ok; ++i) {
+            const uint32_t s = i % kWgStages, use = i / kWgStages;
+            if (use > 0) ok = mbar_wait(&s_empty[s], (use - 1) & 1u);
+            if (!ok) break;
+            unsigned char* x = s_raw + s * 2 * T;
+            const int row = (int)((blockIdx.x + i * gridDim.x) * 128);
+            mbar_expect(&s_full[s], 2 * T);
+            tma_load(x, &map_x, 0, row, &s_full[s]);
+            tma_load(x + BOX, &map_x, 64, row, &s_full[s]);
+            tma_load(x + T, &map_y, 0, row, &s_full[s]);
+            tma_load(x + T + BOX, &map_y, 64, row, &s_full[s]);
+        }
+    } else if (tid == 32) {                              // MMAs
+        for (uint32_t i = 0; i < mine && ok; ++i) {
+            const uint32_t s = i % kWgStages, use = i / kWgStages;
+            ok = mbar_wait(&s_full[s], use & 1u);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t x = sm_addr(s_raw + s * 2 * T);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)                  // 16 rows of the tile each
+                tc_mma(tmem + (i % kWgAcc) * N, smem_desc_mn128(x + k * 2048, BOX),
+                       smem_desc_mn128(x + T + k * 2048, BOX), idesc_bf16(N) | kIdescMN,
+                       (i >= (uint32_t)kWgAcc || k > 0) ? 1u : 0u);
+            tc_commit(&s_empty[s]);
+        }
+        tc_commit(&s_done);
+    }
+    __syncwarp();
+    const bool all = __syncthreads_and(ok) != 0;
+    const bool got = mbar_wait(&s_done, 0);              // every MMA issued has completed
+    if (!(all && got)) {
+        if (tid == 0) {
+            if (g.status) atomicOr(g.status, 1u);
+            for (int s = 0; s < kWgStages; ++s) {        // let copies in flight land first
+                const uint32_t uses = (mine + kWgStages - 1 - s) / kWgStages;
+                if (uses) mbar_wait(&s_full[s], (uses - 1) & 1u);
+            }
+        }
+    }
+    tc_fence_after();
+    const uint32_t used = all && got ? (mine < (uint32_t)kWgAcc ? mine : (uint32_t)kWgAcc) : 0u;
+    uint4* o = reinterpret_cast<uint4*>(g.partial + ((size_t)blockIdx.x * 128 + tid) * N);
+    const uint32_t quarter = (uint32_t)(w * 32) << 16;   // feature row tid of dW
+#pragma unroll 1
+    for (int c0 = 0; c0 < N; c0 += 16) {
+        float v[16] = {};
+        for (uint32_t a = 0; a < used; ++a) {
+            float t[16];
+            tmem_ld16(tmem + quarter + a * N + c0, t);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) v[q] += t[q];
+        }
+        const uint4* vv = reinterpret_cast<const uint4*>(v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[c0 / 4 + q] = vv[q];
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (w == 0) tmem_dealloc(tmem, 512);
 }
 
 // Adds the partials: 32 outputs per block (128 bytes of each partial), its
@@ -1174,6 +1279,33 @@ void launch_linear_t(const LinearArgs& g, int sms, cudaStream_t st) {
     k_linear<K, N><<<grid, linear_threads<N>(), smem, st>>>(g);
 }
 
+// Tensor map of an M x 128 bf16 matrix (row stride ld) in boxes of 128 rows x 64 columns with
+// the 128-byte swizzle.  Rows past M load as zeros and are not stored.
+bool tile_map(CUtensorMap* map, const void* base, uint32_t M, uint32_t ld = 128) {
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                             &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Encode>(fn);
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {128, M}, strides[1] = {(cuuint64_t)ld * 2};
+    const cuuint32_t box[2] = {64, 128}, step[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+                  box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
+}
+
 template <int N>
 void launch_wgrad_t(const WgradArgs& g, int sms, cudaStream_t st) {
     static bool init = false;
@@ -1188,6 +1320,26 @@ void launch_wgrad_t(const WgradArgs& g, int sms, cudaStream_t st) {
     k_wgrad<N><<<grid, 128, smem, st>>>(g);
     const int count = 128 * N;
     k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
+}
+
+bool launch_wgrad_tma(const WgradArgs& g, int sms, cudaStream_t st) {
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_wgrad_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+    });
+    constexpr int count = 128 * 128;
+    if (g.M == 0) return cudaMemsetAsync(g.dW, 0, count * sizeof(float), st) == cudaSuccess;
+    CUtensorMap map_x, map_y;
+    if (!tile_map(&map_x, g.X, g.M, g.ldp ? g.ldp : 128u) ||
+        !tile_map(&map_y, g.dY, g.M, g.ldq ? g.ldq : 128u))
+        return false;
+    const uint32_t tiles = (g.M + 127) / 128;
+    uint32_t grid = (tiles + kWgMinTiles - 1) / kWgMinTiles;
+    if (grid > (uint32_t)sms) grid = (uint32_t)sms;
+    if (grid > g.nparts) grid = g.nparts;
+    k_wgrad_tma<<<grid, 128, kWgSmem, st>>>(g, map_x, map_y);
+    k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
+    return true;
 }
 
 int g_sms = 0;
@@ -1222,37 +1374,6 @@ bool launch_linear(int K, int N, const LinearArgs& args, cudaStream_t st) {
     else return false;
     return true;
 }
-
-namespace {
-
-// Tensor map of an M x 128 bf16 matrix in boxes of 128 rows x 64 columns with
-// the 128-byte swizzle.  Rows past M load as zeros and are not stored.
-bool tile_map(CUtensorMap* map, const void* base, uint32_t M) {
-    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static const Encode encode = [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                             &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            fn = nullptr;
-        }
-        return reinterpret_cast<Encode>(fn);
-    }();
-    if (!encode) return false;
-    const cuuint64_t dims[2] = {128, M}, strides[1] = {256};
-    const cuuint32_t box[2] = {64, 128}, step[2] = {1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
-                  box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
-}
-
-}  // namespace
 
 // The layer: two halves per block, one block per SM (193 KB of shared memory,
 // the SM's 512 TMEM columns).
@@ -1309,8 +1430,8 @@ bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st) {
 }
 
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st) {
-    if (N == 128) launch_wgrad_t<128>(g, num_sms(), st);
-    else if (N == 16) launch_wgrad_t<16>(g, num_sms(), st);
+    if (N == 128) return launch_wgrad_tma(g, num_sms(), st);
+    if (N == 16) launch_wgrad_t<16>(g, num_sms(), st);
     else return false;
     return true;
 }

@@ -698,7 +698,7 @@ int edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z,
 
 // grad of W (kin x kout) += X^T dY over M rows (X: M x kin with stride ldx,
 // dY: M x kout with stride ldy); kin = 16 layers are computed as (dY^T X)^T.
-void wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
+int wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
            const __nv_bfloat16* dY, uint32_t ldy, uint32_t M, int kin_half = -1) {
     WgradArgs g = {};
     g.M = M;
@@ -715,14 +715,15 @@ void wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
         g.dW = c->wg_tmp;
         launch_wgrad(KIN, g, c->st);
         k_transpose<<<nblk((size_t)KIN * L, 256), 256, 0, c->st>>>(c->wg_tmp, L, KIN, dst);
-        return;
+        return SPH_OK;
     }
     g.X = X;
     g.ldp = ldx;
     g.dY = dY;
     g.ldq = ldy;
     g.dW = dst + (kin_half > 0 ? (size_t)kin_half * L * l.kout : 0);
-    launch_wgrad(l.kout, g, c->st);
+    if (!launch_wgrad(l.kout, g, c->st)) return fail(c, SPH_ERR_CUDA, "weight gradient: no tensor maps");
+    return SPH_OK;
 }
 
 }  // namespace
@@ -899,10 +900,10 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
     const Layer* dec = &Ls[4 + 6 * c->NL];
     __nv_bfloat16* h_last = c->XN[c->NL];
     colsum(c, c->dout, n, KOUT, KOUT, c->g + dec[1].b_off);
-    wgrad(c, dec[1], c->D1, L, c->dout, KOUT, n);
+    if ((rc = wgrad(c, dec[1], c->D1, L, c->dout, KOUT, n))) return rc;
     if ((rc = linear(c, c->dout, 0, dec[1], true, n, kEpiReluMask, c->D1, L, c->dD1, nullptr, L))) return rc;
     colsum(c, c->dD1, n, L, L, c->g + dec[0].b_off);
-    wgrad(c, dec[0], h_last, 2 * L, c->dD1, L, n);
+    if ((rc = wgrad(c, dec[0], h_last, 2 * L, c->dD1, L, n))) return rc;
     if ((rc = linear(c, c->dD1, 0, dec[0], true, n, kEpiNone, nullptr, 0, nullptr, c->dH, L))) return rc;
     cudaMemsetAsync(c->dE, 0, (size_t)E * L * sizeof(float), st);
     for (int l = c->NL - 1; l >= 0; --l) {
@@ -913,38 +914,38 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         __nv_bfloat16* y1 = c->Y1[l];
         // node update h' = h + W4 relu(W3 [h, agg] + b3) + b4
         rows_f32(c, c->dH, n, c->dHb, c->g + w[5].b_off);
-        wgrad(c, w[5], y1, L, c->dHb, L, n);
+        if ((rc = wgrad(c, w[5], y1, L, c->dHb, L, n))) return rc;
         if ((rc = linear(c, c->dHb, 0, w[5], true, n, kEpiReluMask, y1, L, c->dY1, nullptr, L))) return rc;
         colsum(c, c->dY1, n, L, L, c->g + w[4].b_off);
-        wgrad(c, w[4], xn_cur, 2 * L, c->dY1, L, n, 0);
-        wgrad(c, w[4], xn_cur + L, 2 * L, c->dY1, L, n, 1);
+        if ((rc = wgrad(c, w[4], xn_cur, 2 * L, c->dY1, L, n, 0))) return rc;
+        if ((rc = wgrad(c, w[4], xn_cur + L, 2 * L, c->dY1, L, n, 1))) return rc;
         if ((rc = linear(c, c->dY1, 0, w[4], true, n, kEpiNone, nullptr, 0, nullptr, c->dXN, 2 * L))) return rc;
         k_add_strided<<<nblk((size_t)n * L, 256), 256, 0, st>>>(n, c->dH, c->dXN, 2 * L);
         // aggregation and edge update e' = e + W2 relu(pre) + b2
         if ((rc = edge_backward(c, w[2], w[3], z1))) return rc;
-        wgrad(c, w[3], z1, L, c->dEb, L, E);
-        wgrad(c, w[2], e_in, L, c->dpre, L, E);
+        if ((rc = wgrad(c, w[3], z1, L, c->dEb, L, E))) return rc;
+        if ((rc = wgrad(c, w[2], e_in, L, c->dpre, L, E))) return rc;
         // pre = W1a h_i + W1b h_j + ...: sums over the edges of i and of j
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, c->dpre, nullptr,
                                                                            c->dPb, nullptr, L);
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, c->dpre, c->rev,
                                                                            c->dQb, nullptr, L);
-        wgrad(c, w[0], xn_cur, 2 * L, c->dPb, L, n);
-        wgrad(c, w[1], xn_cur, 2 * L, c->dQb, L, n);
+        if ((rc = wgrad(c, w[0], xn_cur, 2 * L, c->dPb, L, n))) return rc;
+        if ((rc = wgrad(c, w[1], xn_cur, 2 * L, c->dQb, L, n))) return rc;
         if ((rc = linear(c, c->dPb, 0, w[0], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
         if ((rc = linear(c, c->dQb, 0, w[1], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
     }
     // encoders
     rows_f32(c, c->dE, E, c->dEb, c->g + Ls[3].b_off);
-    wgrad(c, Ls[3], c->ee1, L, c->dEb, L, E);
+    if ((rc = wgrad(c, Ls[3], c->ee1, L, c->dEb, L, E))) return rc;
     if ((rc = linear(c, c->dEb, 0, Ls[3], true, E, kEpiReluMask, c->ee1, L, c->dEe1, nullptr, L))) return rc;
     colsum(c, c->dEe1, E, L, L, c->g + Ls[2].b_off);
-    wgrad(c, Ls[2], c->xe, KIN, c->dEe1, L, E);
+    if ((rc = wgrad(c, Ls[2], c->xe, KIN, c->dEe1, L, E))) return rc;
     rows_f32(c, c->dH, n, c->dHb, c->g + Ls[1].b_off);
-    wgrad(c, Ls[1], c->en1, L, c->dHb, L, n);
+    if ((rc = wgrad(c, Ls[1], c->en1, L, c->dHb, L, n))) return rc;
     if ((rc = linear(c, c->dHb, 0, Ls[1], true, n, kEpiReluMask, c->en1, L, c->dEn1, nullptr, L))) return rc;
     colsum(c, c->dEn1, n, L, L, c->g + Ls[0].b_off);
-    wgrad(c, Ls[0], c->xn, KIN, c->dEn1, L, n);
+    if ((rc = wgrad(c, Ls[0], c->xn, KIN, c->dEn1, L, n))) return rc;
     if (loss_host) {
         cudaMemcpyAsync(loss_host, c->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) return check(c, "sur_backward");
