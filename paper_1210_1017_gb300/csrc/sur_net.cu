@@ -68,86 +68,162 @@ __global__ void k_refresh(const float* __restrict__ w, int kin, int kout, __nv_b
 // Candidates in between take the FP64 arithmetic of the predicate as
 // written.  The edge features (bfloat16) come from the FP32 differences.
 // FP64 instructions run at 1/64 of the FP32 rate on this GPU.
+//
+// A warp takes kGraphP consecutive particles (sorted: mostly of one cell, else
+// the cells in turn) and its lanes consecutive candidates of a run of cells (the
+// x neighbours of one of the nine rows, contiguous in memory).  So a load is
+// whole lines and serves all of the warp's particles, and the hits of a ballot
+// are consecutive edges in candidate order.  (With a thread per particle every
+// load touched a line per lane, and 17k particles filled one warp per
+// scheduler.)  us per pass, count and fill, thread / this: 17k particles 94 +
+// 114 / 18 + 26, 1.39M particles in a sparser graph (23M edges) 985 + 1057 / 742
+// + 1071; one particle per warp 1341 + 1550, eight 922 + 1525 (122 registers).
+// Bound by instruction issue (3.0 per clock) at the larger size.
+constexpr int kGraphP = 4;
+
 template <int MODE>
-__global__ void k_graph(const sph::Dev d, const double* __restrict__ x, const double* __restrict__ y,
-                        const double* __restrict__ z, const float4* __restrict__ posc,
-                        const uint32_t* __restrict__ key, const uint32_t* __restrict__ off,
-                        uint32_t* __restrict__ cnt, const uint32_t* __restrict__ rowptr,
-                        uint32_t* __restrict__ col, uint32_t* __restrict__ src,
-                        __nv_bfloat16* __restrict__ xe, double inv2h, double r2, float inside,
-                        float outside) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d.n) return;
+__global__ void __launch_bounds__(256)
+    k_graph(const sph::Dev d, const double* __restrict__ x, const double* __restrict__ y,
+            const double* __restrict__ z, const float4* __restrict__ posc,
+            const uint32_t* __restrict__ key, const uint32_t* __restrict__ off,
+            uint32_t* __restrict__ cnt, const uint32_t* __restrict__ rowptr,
+            uint32_t* __restrict__ col, uint32_t* __restrict__ src,
+            __nv_bfloat16* __restrict__ xe, double inv2h, double r2, float inside, float outside) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    const uint32_t i0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * kGraphP;
+    const int lane = threadIdx.x & 31;
+    if (i0 >= d.n) return;
     const uint32_t n_in = off[d.ncells];
-    if (i >= n_in) {
-        if (MODE == 0) cnt[i] = 0;
-        return;
+    if (MODE == 0 && lane < kGraphP && i0 + lane >= n_in && i0 + lane < d.n) cnt[i0 + lane] = 0;
+    if (i0 >= n_in) return;
+    // lane p < kGraphP: particle i0 + p
+    const bool mine = lane < kGraphP && i0 + lane < n_in;
+    const uint32_t mykey = mine ? key[i0 + lane] : 0u;
+    const float4 mypos = mine ? posc[i0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t e = 0;                       // lane p: its next edge (MODE 0: edges so far)
+    if (MODE && mine) e = rowptr[i0 + lane];
+    float2 px[kGraphP / 2], py[kGraphP / 2], pz[kGraphP / 2];
+    uint32_t at[kGraphP];                 // e of every particle
+#pragma unroll
+    for (int p = 0; p < kGraphP; p += 2) {
+        px[p / 2] = make_float2(__shfl_sync(kAll, mypos.x, p), __shfl_sync(kAll, mypos.x, p + 1));
+        py[p / 2] = make_float2(__shfl_sync(kAll, mypos.y, p), __shfl_sync(kAll, mypos.y, p + 1));
+        pz[p / 2] = make_float2(__shfl_sync(kAll, mypos.z, p), __shfl_sync(kAll, mypos.z, p + 1));
+        at[p] = __shfl_sync(kAll, e, p);
+        at[p + 1] = __shfl_sync(kAll, e, p + 1);
     }
-    const uint32_t k = key[i];
-    uint32_t lo = 0, hi = d.n_inst;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (d.cell_base[mid] <= k) lo = mid;
-        else hi = mid;
-    }
-    const sph::Inst& I = d.inst[lo];
-    const uint32_t lk = k - I.cell_base;
-    const int cx = (int)(lk % (uint32_t)I.ncx);
-    const uint32_t t = lk / (uint32_t)I.ncx;
-    const int cy = (int)(t % (uint32_t)I.ncy), cz = (int)(t / (uint32_t)I.ncy);
-    const double xi = x[i], yi = y[i], zi = z[i];
-    const float4 pi = posc[i];
     const float inv2hf = (float)inv2h;
-    const int xlo = cx > 0 ? cx - 1 : 0, xhi = cx + 1 < I.ncx ? cx + 1 : I.ncx - 1;
-    uint32_t c = 0, e = MODE ? rowptr[i] : 0u;
-    for (int zz = cz - 1; zz <= cz + 1; ++zz) {
-        if (zz < 0 || zz >= I.ncz) continue;
-        const float qz = fmaf((float)(cz - zz), d.csf, pi.z);
-        for (int yy = cy - 1; yy <= cy + 1; ++yy) {
-            if (yy < 0 || yy >= I.ncy) continue;
-            const float qy = fmaf((float)(cy - yy), d.csf, pi.y);
-            const uint32_t rb = I.cell_base + (uint32_t)I.ncx * ((uint32_t)yy + (uint32_t)I.ncy * zz);
-            for (int xx = xlo; xx <= xhi; ++xx) {
-                const float qx = fmaf((float)(cx - xx), d.csf, pi.x);
-                const uint32_t s = off[rb + xx], en = off[rb + xx + 1];
-                for (uint32_t j = s; j < en; ++j) {
-                    if (j == i) continue;
-                    const float4 pj = posc[j];
-                    const float fx = qx - pj.x, fy = qy - pj.y, fz = qz - pj.z;
-                    const float d2f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+    const float2 cs2 = make_float2(d.csf, d.csf);
+    uint32_t left = __ballot_sync(kAll, mine);
+    while (left) {
+        // the particles of the first one's cell
+        const uint32_t k = __shfl_sync(kAll, mykey, __ffs(left) - 1);
+        const uint32_t grp = __ballot_sync(kAll, mykey == k) & left;
+        left &= ~grp;
+        uint32_t lo = 0, hi = d.n_inst;
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (d.cell_base[mid] <= k) lo = mid;
+            else hi = mid;
+        }
+        const sph::Inst& I = d.inst[lo];
+        const uint32_t lk = k - I.cell_base;
+        const int cx = (int)(lk % (uint32_t)I.ncx);
+        const uint32_t t = lk / (uint32_t)I.ncx;
+        const int cy = (int)(t % (uint32_t)I.ncy), cz = (int)(t / (uint32_t)I.ncy);
+        const int xlo = cx > 0 ? cx - 1 : 0, xend = cx + 1 < I.ncx ? cx + 2 : I.ncx;
+        // lane r < 9: the run of row r (y fastest), its first candidate, the
+        // first of its second and third cell, its end
+        uint32_t o[4] = {0u, 0u, 0u, 0u};
+        if (lane < 9) {
+            const int yy = cy + lane % 3 - 1, zz = cz + lane / 3 - 1;
+            if (yy >= 0 && yy < I.ncy && zz >= 0 && zz < I.ncz) {
+                const uint32_t rb = I.cell_base + (uint32_t)I.ncx * ((uint32_t)yy + (uint32_t)I.ncy * zz);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) o[q] = off[rb + (xlo + q < xend ? xlo + q : xend)];
+            }
+        }
+#pragma unroll 1
+        for (int r = 0; r < 9; ++r) {
+            const uint32_t s0 = __shfl_sync(kAll, o[0], r), s1 = __shfl_sync(kAll, o[1], r);
+            const uint32_t s2 = __shfl_sync(kAll, o[2], r), en = __shfl_sync(kAll, o[3], r);
+            const float oy = (float)(1 - r % 3), oz = (float)(1 - r / 3);
+            for (uint32_t j0 = s0; j0 < en; j0 += 32) {
+                const uint32_t j = j0 + (uint32_t)lane;
+                const bool in = j < en;
+                const float4 pj = posc[in ? j : s0];
+                const float ox = (float)(cx - xlo - (j >= s1 ? 1 : 0) - (j >= s2 ? 1 : 0));
+#pragma unroll
+                for (int h = 0; h < kGraphP / 2; ++h) {
+                    if (!((grp >> (2 * h)) & 3u)) continue;          // warp-uniform
+                    // two particles at a time, each with the roundings of one
+                    const float2 m1 = make_float2(-1.f, -1.f);
+                    const float2 fx = __ffma2_rn(make_float2(pj.x, pj.x), m1,
+                                                 __ffma2_rn(make_float2(ox, ox), cs2, px[h]));
+                    const float2 fy = __ffma2_rn(make_float2(pj.y, pj.y), m1,
+                                                 __ffma2_rn(make_float2(oy, oy), cs2, py[h]));
+                    const float2 fz = __ffma2_rn(make_float2(pj.z, pj.z), m1,
+                                                 __ffma2_rn(make_float2(oz, oz), cs2, pz[h]));
+                    const float2 d2 = __ffma2_rn(fx, fx, __ffma2_rn(fy, fy, __fmul2_rn(fz, fz)));
                     // outside, or not finite (the FP64 predicate rejects those too)
-                    if (!(d2f < outside)) continue;
-                    if (!(d2f < inside)) {
-                        const double dx = __dsub_rn(xi, x[j]);
-                        const double dy = __dsub_rn(yi, y[j]);
-                        const double dz = __dsub_rn(zi, z[j]);
-                        const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                                    __dmul_rn(dz, dz));
-                        if (!(d2 < r2)) continue;
+                    bool hits[2] = {d2.x < outside && in && j != i0 + 2 * h && ((grp >> (2 * h)) & 1u),
+                                    d2.y < outside && in && j != i0 + 2 * h + 1 && ((grp >> (2 * h + 1)) & 1u)};
+                    // (a vote: the compiler would run the FP64 test every time, predicated)
+                    if (__any_sync(kAll, (hits[0] && !(d2.x < inside)) || (hits[1] && !(d2.y < inside)))) {
+#pragma unroll
+                        for (int b = 0; b < 2; ++b) {
+                            if (!hits[b] || (b ? d2.y : d2.x) < inside) continue;
+                            const uint32_t i = i0 + 2 * h + b;
+                            const double dx = __dsub_rn(x[i], x[j]);
+                            const double dy = __dsub_rn(y[i], y[j]);
+                            const double dz = __dsub_rn(z[i], z[j]);
+                            const double q = __dadd_rn(
+                                __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+                            hits[b] = q < r2;
+                        }
                     }
-                    if (MODE) {
-                        // the edge inputs are bfloat16: the FP32 differences (within
-                        // 3.6e-7 of a cell of the FP64 ones) round to the bfloat16 of
-                        // the FP64 value except where that lies within this error of
-                        // a rounding midpoint (one bfloat16 step then)
-                        col[e] = j;
-                        src[e] = i;
-                        // one 32-byte row: (x, y, z, |r|) / 2h, then zeros
-                        const __nv_bfloat162 f01 = __floats2bfloat162_rn(fx * inv2hf, fy * inv2hf);
-                        const __nv_bfloat162 f23 =
-                            __floats2bfloat162_rn(fz * inv2hf, sqrtf(d2f) * inv2hf);
-                        uint4* f = reinterpret_cast<uint4*>(xe + (size_t)e * KIN);
-                        f[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&f01),
-                                          *reinterpret_cast<const uint32_t*>(&f23), 0u, 0u);
-                        f[1] = make_uint4(0u, 0u, 0u, 0u);
-                        ++e;
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const uint32_t i = i0 + 2 * h + b;
+                        const float d2f = b ? d2.y : d2.x;
+                        const bool hit = hits[b];
+                        if (MODE == 0) {
+                            at[2 * h + b] += hit ? 1u : 0u;          // this lane's
+                            continue;
+                        }
+                        const uint32_t m = __ballot_sync(kAll, hit);
+                        if (hit) {
+                            // the edge inputs are bfloat16: the FP32 differences (within
+                            // 3.6e-7 of a cell of the FP64 ones) round to the bfloat16 of
+                            // the FP64 value except where that lies within this error of
+                            // a rounding midpoint (one bfloat16 step then)
+                            const uint32_t to = at[2 * h + b] + (uint32_t)__popc(m & ((1u << lane) - 1u));
+                            col[to] = j;
+                            src[to] = i;
+                            // one 32-byte row: (x, y, z, |r|) / 2h, then zeros
+                            const __nv_bfloat162 f01 = __floats2bfloat162_rn((b ? fx.y : fx.x) * inv2hf,
+                                                                             (b ? fy.y : fy.x) * inv2hf);
+                            const __nv_bfloat162 f23 = __floats2bfloat162_rn((b ? fz.y : fz.x) * inv2hf,
+                                                                             sqrtf(d2f) * inv2hf);
+                            uint4* f = reinterpret_cast<uint4*>(xe + (size_t)to * KIN);
+                            f[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&f01),
+                                              *reinterpret_cast<const uint32_t*>(&f23), 0u, 0u);
+                            f[1] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        at[2 * h + b] += (uint32_t)__popc(m);
                     }
-                    ++c;
                 }
             }
         }
     }
-    if (MODE == 0) cnt[i] = c;
+    if (MODE == 0) {
+#pragma unroll
+        for (int p = 0; p < kGraphP; ++p) {
+            const uint32_t t = __reduce_add_sync(kAll, at[p]);
+            if (lane == p) e = t;
+        }
+        if (mine) cnt[i0 + lane] = e;
+    }
 }
 
 // rev[e] = index of the edge (j, i) in row j (rows are sorted ascending).
@@ -824,7 +900,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
     const bool fp32_ok = r2 >= 0.01 * (2.0 * s->p.h) * (2.0 * s->p.h);
     const float inside = fp32_ok ? (float)r2 * (1.0f - 0x1p-12f) : -1.0f;
     const float outside = fp32_ok ? (float)r2 * (1.0f + 0x1p-12f) : INFINITY;
-    k_graph<0><<<nblk(n, 128), 128, 0, st>>>(d, s->x[cur], s->y[cur], s->z[cur], s->posc, key,
+    k_graph<0><<<nblk(n, 8 * kGraphP), 256, 0, st>>>(d, s->x[cur], s->y[cur], s->z[cur], s->posc, key,
                                              s->off, c->cnt, nullptr, nullptr, nullptr, nullptr,
                                              inv2h, r2, inside, outside);
     sph::launch_scan(c->cnt, n, c->bsum, c->rowptr, st);
@@ -833,7 +909,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return check(c, "graph count");
     if (E > c->cfg.max_edges) return fail(c, SPH_ERR_CAPACITY, "more edges than max_edges");
     c->E = E;
-    k_graph<1><<<nblk(n, 128), 128, 0, st>>>(d, s->x[cur], s->y[cur], s->z[cur], s->posc, key,
+    k_graph<1><<<nblk(n, 8 * kGraphP), 256, 0, st>>>(d, s->x[cur], s->y[cur], s->z[cur], s->posc, key,
                                              s->off, nullptr, c->rowptr, c->col, c->src, c->xe,
                                              inv2h, r2, inside, outside);
     if (c->cfg.train && E) k_graph_rev<<<nblk(E, 256), 256, 0, st>>>(E, c->rowptr, c->col, c->src, c->rev);
