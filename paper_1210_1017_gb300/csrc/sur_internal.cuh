@@ -90,6 +90,26 @@ struct EdgeBwdArgs {
     uint32_t* status;
 };
 
+// Node update of a message-passing layer over n nodes, x = [h, agg] (n x 256):
+//   y = relu(x W3 + b3) (to Y when Y != null),  h' = h + y W4 + b4 (to H, row
+//   stride 256),  and when P != null the next layer's P = h' Wp, Q = h' Wq.
+// W3t (128 x 256), W4t, Wpt, Wqt (128 x 128): the weights transposed, bf16.
+struct NodeArgs {
+    const __nv_bfloat16* X;
+    const __nv_bfloat16* W3t;
+    const __nv_bfloat16* W4t;
+    const __nv_bfloat16* Wpt;
+    const __nv_bfloat16* Wqt;
+    const float* b3;
+    const float* b4;
+    uint32_t n;
+    __nv_bfloat16* Y;
+    __nv_bfloat16* H;
+    __nv_bfloat16* P;
+    __nv_bfloat16* Q;
+    uint32_t* status;
+};
+
 int num_sms();
 bool launch_linear(int K, int N, const LinearArgs& g, cudaStream_t st);
 // False when the driver has no tensor maps for the tiles (nothing launched).
@@ -97,6 +117,7 @@ bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st);
 // The edge encoder in one kernel: E (M x 16) -> Eout = relu(E W1 + b1) W2 + b2
 // (z = relu(E W1 + b1) to Z when Z != null); P, Q, src, dst unused.
 bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st);
+bool launch_node_update(const NodeArgs& g, cudaStream_t st);
 bool launch_edge_backward(const EdgeBwdArgs& g, uint32_t* nparts, cudaStream_t st);
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st);
 

@@ -1252,6 +1252,206 @@ __global__ void __launch_bounds__(512, 1)
     }
 }
 
+// The node update of a message-passing layer and the node terms of the next
+// layer's edge update in one kernel, per 128-node tile (x = [h, agg], 256 columns):
+//   y = relu(x W3 + b3),  h' = h + y W4 + b4,  P = h' W1a,  Q = h' W1b
+// x comes by TMA (128-byte swizzle) and serves MMA 1 and the residual; y and h'
+// go to TMEM as the A operands of the next products, so nothing returns from HBM
+// between the layers.  The weights (160 KB) and one x tile (64 KB) fill the
+// shared memory; the next tile's x loads under MMA 3.  512 threads: the four
+// warps of a TMEM lane quarter split the columns.  A small system has one tile
+// per SM and is bound by the chain of three products, a large one by HBM (512 B
+// in, 768 out per node; 1,792 and four launches as separate layers).
+// On one GB300, us per layer, four launches / one: 17k nodes 36 / 18, 1.39M
+// nodes 860 / 361 (4.9 TB/s).
+// TMEM columns: accumulators of MMA 1 at 0, y at 128, accumulators of MMA 2 at
+// 256, h' at 384; those of MMA 3 at 0 .. 255, over what MMA 2 has read.
+constexpr size_t kNodeSmem = (size_t)7 * kETile + 1024;   // W3 (2), W4, W1a and W1b, x (2); alignment
+
+__global__ void __launch_bounds__(512, 1)
+    k_node_update(const NodeArgs g, const __grid_constant__ CUtensorMap map_x, const bool wide) {
+    constexpr int N = 128;
+    constexpr uint32_t T = kETile, BOX = T / 2;          // a box: 64 columns of 128 rows
+    extern __shared__ unsigned char s_dyn[];
+    __shared__ __align__(16) float s_b3[128], s_b4[128];
+    __shared__ __align__(8) uint64_t s_full, s_bar[3];   // x loaded; MMAs 1 to 3
+    __shared__ uint32_t s_tmem;
+    unsigned char* s_raw = s_dyn + ((1024u - (sm_addr(s_dyn) & 1023u)) & 1023u);
+    unsigned char* sx = s_raw;                           // four boxes
+    unsigned char* sw3 = sx + 2 * T;                     // N x 256
+    unsigned char* sw4 = sw3 + 2 * T;                    // N x N
+    unsigned char* swp = sw4 + T;                        // 2 N x N: W1a, then W1b
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const bool mover = tid == 32;
+    if (w == 0) tmem_alloc(&s_tmem, 512);
+    if (tid == 0) {
+        mbar_init1(&s_full);
+        for (int k = 0; k < 3; ++k) mbar_init1(&s_bar[k]);
+    }
+    for (int c = tid; c < N * (2 * N / 8); c += 512) {
+        const int r = c % N, gk = c / N;
+        cp_async16(sw3 + kmajor_offset(r, gk * 8, 2 * N), g.W3t + (size_t)r * 2 * N + gk * 8, true);
+    }
+    cp_async_commit();
+    for (int c = tid; c < N * (N / 8); c += 512) {
+        const int r = c % N, gk = c / N;
+        cp_async16(sw4 + kmajor_offset(r, gk * 8, N), g.W4t + (size_t)r * N + gk * 8, true);
+        if (g.P) {
+            cp_async16(swp + kmajor_offset(r, gk * 8, N), g.Wpt + (size_t)r * N + gk * 8, true);
+            cp_async16(swp + kmajor_offset(N + r, gk * 8, N), g.Wqt + (size_t)r * N + gk * 8, true);
+        }
+    }
+    cp_async_commit();
+    if (tid < 128) {
+        s_b3[tid] = g.b3[tid];
+        s_b4[tid] = g.b4[tid];
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory"); // W3
+    fence_async_shared();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    const uint32_t ntiles = (g.n + 127) / 128;
+    const int wq = w & 3, part = w >> 2;                 // lane quarter, column part
+    const int r = wq * 32 + lane;                        // this thread's row of a tile
+    const uint32_t quarter = (uint32_t)(wq * 32) << 16;
+    auto load_x = [&](uint32_t t) {
+        mbar_expect(&s_full, 2 * T);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) tma_load(sx + b * BOX, &map_x, 64 * b, (int)(t * 128), &s_full);
+    };
+    auto put = [&](__nv_bfloat16* row, const uint32_t (&v)[8]) {   // 16 columns of a row
+        uint4* o = reinterpret_cast<uint4*>(row);
+        const uint4 a = make_uint4(v[0], v[1], v[2], v[3]), b = make_uint4(v[4], v[5], v[6], v[7]);
+        if (wide) {
+            stg32(o, a, b);
+        } else {
+            o[0] = a;
+            o[1] = b;
+        }
+    };
+    uint32_t tile = blockIdx.x, phase = 0;
+    bool ok = true, weights = false;
+    if (mover && tile < ntiles) load_x(tile);
+    for (; tile < ntiles; tile += gridDim.x) {
+        const uint32_t m = tile * 128 + (uint32_t)r, next = tile + gridDim.x;
+        bool got = mbar_wait(&s_full, phase);            // x, for MMA 1 and the residual
+        if (got && tid == 0) {
+            tc_fence_after();
+#pragma unroll
+            for (int s = 0; s < 2 * N / 16; ++s)
+                tc_mma(tmem, smem_desc_sw128(sm_addr(sx) + (s >> 2) * BOX + (s & 3) * 32),
+                       smem_desc(sm_addr(sw3) + s * 256, kLBO, (2 * N / 8) * 128), idesc_bf16(N),
+                       s > 0 ? 1u : 0u);
+            tc_commit(&s_bar[0]);
+        }
+        if (!weights) {                                  // the other weights, under MMA 1
+            cp_async_wait_all();
+            fence_async_shared();
+            weights = true;
+        }
+        got = got && mbar_wait(&s_bar[0], phase);
+        tc_fence_after();
+        // y = relu(acc + b3)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c0 = part * 32 + 16 * k;
+            float v[16];
+            tmem_ld16(tmem + quarter + c0, v);
+            uint32_t z[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const __nv_bfloat162 t = __floats2bfloat162_rn(fmaxf(v[2 * q] + s_b3[c0 + 2 * q], 0.f),
+                                                               fmaxf(v[2 * q + 1] + s_b3[c0 + 2 * q + 1], 0.f));
+                z[q] = *reinterpret_cast<const uint32_t*>(&t);
+            }
+            tmem_st8(tmem + quarter + 128u + (uint32_t)(c0 / 2), z);
+            if (g.Y && m < g.n) put(g.Y + (size_t)m * N + c0, z);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        ok = __syncthreads_and(got) != 0;                // y complete
+        if (!ok) break;
+        if (tid == 0) {
+            tc_fence_after();
+#pragma unroll
+            for (int s = 0; s < N / 16; ++s)
+                tc_mma_ta(tmem + 256u, tmem + 128u + s * 8,
+                          smem_desc(sm_addr(sw4) + s * 256, kLBO, (N / 8) * 128), idesc_bf16(N),
+                          s > 0 ? 1u : 0u);
+            tc_commit(&s_bar[1]);
+        }
+        got = mbar_wait(&s_bar[1], phase);
+        tc_fence_after();
+        // h' = (acc + b4) + h
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c0 = part * 32 + 16 * k;
+            float v[16], t[16];
+            tmem_ld16(tmem + quarter + 256u + c0, v);
+            const unsigned char* box = sx + (c0 >> 6) * BOX;
+            unpack8(*reinterpret_cast<const uint4*>(box + sw128_offset(r, (c0 & 63) / 8)), t);
+            unpack8(*reinterpret_cast<const uint4*>(box + sw128_offset(r, (c0 & 63) / 8 + 1)), t + 8);
+            uint32_t z[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const __nv_bfloat162 u =
+                    __floats2bfloat162_rn(v[2 * q] + s_b4[c0 + 2 * q] + t[2 * q],
+                                          v[2 * q + 1] + s_b4[c0 + 2 * q + 1] + t[2 * q + 1]);
+                z[q] = *reinterpret_cast<const uint32_t*>(&u);
+            }
+            if (g.P) tmem_st8(tmem + quarter + 384u + (uint32_t)(c0 / 2), z);
+            if (m < g.n) put(g.H + (size_t)m * (2 * N) + c0, z);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        ok = __syncthreads_and(got) != 0;                // h' complete, x free
+        if (!ok) break;
+        if (mover && next < ntiles) load_x(next);
+        if (g.P) {
+            if (tid == 0) {
+                tc_fence_after();
+#pragma unroll
+                for (int s = 0; s < N / 16; ++s)
+                    tc_mma_ta(tmem, tmem + 384u + s * 8,
+                              smem_desc(sm_addr(swp) + s * 256, kLBO, (N / 8) * 128), idesc_bf16(2 * N),
+                              s > 0 ? 1u : 0u);
+                tc_commit(&s_bar[2]);
+            }
+            got = mbar_wait(&s_bar[2], phase);
+            tc_fence_after();
+            __nv_bfloat16* out = (part < 2 ? g.P : g.Q) + (size_t)m * N + (part & 1) * 64;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float v[16];
+                tmem_ld16(tmem + quarter + (uint32_t)(part * 64 + 16 * k), v);
+                uint32_t z[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const __nv_bfloat162 u = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+                    z[q] = *reinterpret_cast<const uint32_t*>(&u);
+                }
+                if (m < g.n) put(out + 16 * k, z);
+            }
+            tc_fence_before();
+            ok = __syncthreads_and(got) != 0;            // MMA 3's columns free
+            if (!ok) break;
+        }
+        phase ^= 1u;
+    }
+    if (!ok) {
+        if (tid == 0 && g.status) atomicOr(g.status, 1u);
+        mbar_wait(&s_full, phase);                       // let MMAs and copies in flight
+        mbar_wait(&s_full, phase ^ 1u);
+        for (int k = 0; k < 3; ++k) mbar_wait(&s_bar[k], phase);   // land first
+    }
+    cp_async_wait_all();
+    tc_fence_before();
+    __syncthreads();
+    if (w == 0) tmem_dealloc(tmem, 512);
+}
+
 template <int K, int N>
 void launch_linear_t(const LinearArgs& g, int sms, cudaStream_t st) {
     static bool init = false;
@@ -1279,9 +1479,10 @@ void launch_linear_t(const LinearArgs& g, int sms, cudaStream_t st) {
     k_linear<K, N><<<grid, linear_threads<N>(), smem, st>>>(g);
 }
 
-// Tensor map of an M x 128 bf16 matrix (row stride ld) in boxes of 128 rows x 64 columns with
+// Tensor map of an M x cols bf16 matrix (row stride ld) in boxes of 128 rows x 64 columns with
 // the 128-byte swizzle.  Rows past M load as zeros and are not stored.
-bool tile_map(CUtensorMap* map, const void* base, uint32_t M, uint32_t ld = 128) {
+bool tile_map(CUtensorMap* map, const void* base, uint32_t M, uint32_t ld = 128,
+              uint32_t cols = 128) {
     using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                 const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                 const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -1298,7 +1499,7 @@ bool tile_map(CUtensorMap* map, const void* base, uint32_t M, uint32_t ld = 128)
         return reinterpret_cast<Encode>(fn);
     }();
     if (!encode) return false;
-    const cuuint64_t dims[2] = {128, M}, strides[1] = {(cuuint64_t)ld * 2};
+    const cuuint64_t dims[2] = {cols, M}, strides[1] = {(cuuint64_t)ld * 2};
     const cuuint32_t box[2] = {64, 128}, step[2] = {1, 1};
     return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
                   box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1410,6 +1611,22 @@ bool launch_edge_backward(const EdgeBwdArgs& g, uint32_t* nparts, cudaStream_t s
     if (grid > (tiles + 1) / 2) grid = (tiles + 1) / 2;
     *nparts = 2 * grid;
     k_edge_bwd<<<grid, 512, kEdgeBwdSmem, st>>>(g, map_z, map_v, map_p, all % 32u == 0u && g.ldn % 8u == 0u);
+    return true;
+}
+
+bool launch_node_update(const NodeArgs& g, cudaStream_t st) {
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_node_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNodeSmem);
+    });
+    if (g.n == 0) return true;
+    CUtensorMap map_x;
+    if (!tile_map(&map_x, g.X, g.n, 256, 256)) return false;
+    const uintptr_t all = reinterpret_cast<uintptr_t>(g.Y) | reinterpret_cast<uintptr_t>(g.H) |
+                          reinterpret_cast<uintptr_t>(g.P) | reinterpret_cast<uintptr_t>(g.Q);
+    const uint32_t tiles = (g.n + 127) / 128;
+    const uint32_t sms = (uint32_t)num_sms();
+    k_node_update<<<tiles < sms ? tiles : sms, 512, kNodeSmem, st>>>(g, map_x, all % 32u == 0u);
     return true;
 }
 

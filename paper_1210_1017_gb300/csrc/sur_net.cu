@@ -675,7 +675,7 @@ size_t carve(sur_ctx* c, void* base) {
     c->XN.assign(nx, nullptr);
     c->Ebuf.assign(ne, nullptr);
     c->Z1.assign(nz, nullptr);
-    c->Y1.assign(train ? NL : 1, nullptr);
+    c->Y1.assign(train ? NL : 0, nullptr);
     for (auto& p : c->XN) p = cv.take<__nv_bfloat16>(N * 2 * L);
     for (auto& p : c->Ebuf) p = cv.take<__nv_bfloat16>(E * L);
     for (auto& p : c->Z1) p = cv.take<__nv_bfloat16>(E * L);
@@ -753,6 +753,30 @@ int edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16
     g.Z = z;
     g.Eout = e_out;
     if (!launch_edge_layer(g, c->st)) return fail(c, SPH_ERR_CUDA, "edge layer: no tensor maps");
+    return SPH_OK;
+}
+
+// The node update of a layer (weights w[4], w[5]) from xn = [h, agg] to h' in
+// xn_next, y kept for the backward pass when y != null, and the node terms of
+// the next layer (weights next[0], next[1]) when there is one.
+int node_update(sur_ctx* c, const Layer* w, const Layer* next, const __nv_bfloat16* xn,
+                __nv_bfloat16* y, __nv_bfloat16* xn_next) {
+    NodeArgs g = {};
+    g.X = xn;
+    g.W3t = w[4].Wt;
+    g.W4t = w[5].Wt;
+    g.b3 = c->w + w[4].b_off;
+    g.b4 = c->w + w[5].b_off;
+    g.n = c->n;
+    g.Y = y;
+    g.H = xn_next;
+    if (next) {
+        g.Wpt = next[0].Wt;
+        g.Wqt = next[1].Wt;
+        g.P = c->P;
+        g.Q = c->Q;
+    }
+    if (!launch_node_update(g, c->st)) return fail(c, SPH_ERR_CUDA, "node update: no tensor maps");
     return SPH_OK;
 }
 
@@ -921,22 +945,24 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
     if ((rc = linear(c, c->xn, 0, Ls[0], false, n, kEpiRelu, nullptr, 0, c->en1, nullptr, L))) return rc;
     if ((rc = linear(c, c->en1, 0, Ls[1], false, n, kEpiNone, nullptr, 0, c->XN[0], nullptr, 2 * L))) return rc;
     if ((rc = edge_encoder(c, Ls[2], Ls[3], train ? c->ee1 : nullptr, c->Ebuf[0]))) return rc;
-    // message passing
+    // message passing (the node terms P, Q of each layer come from the node
+    // update before it, the first ones from here)
+    if (c->NL > 0) {
+        const Layer* w = &Ls[4];
+        if ((rc = linear(c, c->XN[0], 2 * L, w[0], false, n, kEpiNone, nullptr, 0, c->P, nullptr, L))) return rc;
+        if ((rc = linear(c, c->XN[0], 2 * L, w[1], false, n, kEpiNone, nullptr, 0, c->Q, nullptr, L))) return rc;
+    }
     for (int l = 0; l < c->NL; ++l) {
         __nv_bfloat16* xn_cur = c->XN[train ? l : l % 2];
         __nv_bfloat16* xn_next = c->XN[train ? l + 1 : (l + 1) % 2];
         __nv_bfloat16* e_in = c->Ebuf[train ? l : l % 2];
         __nv_bfloat16* e_out = c->Ebuf[train ? l + 1 : (l + 1) % 2];
         __nv_bfloat16* z1 = train ? c->Z1[l] : nullptr;
-        __nv_bfloat16* y1 = c->Y1[train ? l : 0];
         const Layer* w = &Ls[4 + 6 * l];
-        if ((rc = linear(c, xn_cur, 2 * L, w[0], false, n, kEpiNone, nullptr, 0, c->P, nullptr, L))) return rc;
-        if ((rc = linear(c, xn_cur, 2 * L, w[1], false, n, kEpiNone, nullptr, 0, c->Q, nullptr, L))) return rc;
         if ((rc = edge_layer(c, w[2], w[3], e_in, train ? z1 : nullptr, e_out))) return rc;
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, e_out, nullptr,
                                                                            xn_cur + L, nullptr, 2 * L);
-        if ((rc = linear(c, xn_cur, 0, w[4], false, n, kEpiRelu, nullptr, 0, y1, nullptr, L))) return rc;
-        if ((rc = linear(c, y1, 0, w[5], false, n, kEpiResidual, xn_cur, 2 * L, xn_next, nullptr, 2 * L)))
+        if ((rc = node_update(c, w, l + 1 < c->NL ? w + 6 : nullptr, xn_cur, train ? c->Y1[l] : nullptr, xn_next)))
             return rc;
     }
     __nv_bfloat16* h_last = c->XN[train ? c->NL : c->NL % 2];
