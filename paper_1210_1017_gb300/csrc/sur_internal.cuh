@@ -119,6 +119,10 @@ bool launch_edge_layer(const EdgeArgs& g, cudaStream_t st);
 bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st);
 bool launch_node_update(const NodeArgs& g, cudaStream_t st);
 bool launch_edge_backward(const EdgeBwdArgs& g, uint32_t* nparts, cudaStream_t st);
+// `batch` (1 .. kWgradBatch) gradients with N = 128 over the same rows (M, nparts,
+// partial and scale of the first).
+constexpr int kWgradBatch = 3;
+bool launch_wgrads(const WgradArgs* g, int batch, cudaStream_t st);
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st);
 
 }  // namespace sur

@@ -410,9 +410,20 @@ constexpr int kWgStages = 3, kWgAcc = 4;
 constexpr uint32_t kWgMinTiles = 2;   // tiles per block where there are enough (fewer partials)
 constexpr size_t kWgSmem = (size_t)kWgStages * 2 * 32768 + 1024;
 
+// Up to kWgradBatch gradients over the same rows, one per blockIdx.y, and their
+// outputs: a small system's rows fill the chip once for all of them, with one
+// reduction (a training step of 17k particles and 10 layers: 11.92 -> 11.54 ms
+// with the five node gradients of a layer in two launches and its four column
+// sums finished in one).
+struct WgradMaps {
+    CUtensorMap x[kWgradBatch], y[kWgradBatch];
+};
+struct WgradOuts {
+    float* dW[kWgradBatch];
+};
+
 __global__ void __launch_bounds__(128, 1)
-    k_wgrad_tma(const WgradArgs g, const __grid_constant__ CUtensorMap map_x,
-                const __grid_constant__ CUtensorMap map_y) {
+    k_wgrad_tma(const WgradArgs g, const __grid_constant__ WgradMaps maps) {
     constexpr int N = 128;
     constexpr uint32_t T = 128 * 128 * 2, BOX = T / 2;
     extern __shared__ unsigned char s_dyn[];
@@ -432,6 +443,7 @@ __global__ void __launch_bounds__(128, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    const CUtensorMap *map_x = &maps.x[blockIdx.y], *map_y = &maps.y[blockIdx.y];
     const uint32_t ntiles = (g.M + 127) / 128;
     const uint32_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     bool ok = true;
@@ -443,10 +455,10 @@ __global__ void __launch_bounds__(128, 1)
             unsigned char* x = s_raw + s * 2 * T;
             const int row = (int)((blockIdx.x + i * gridDim.x) * 128);
             mbar_expect(&s_full[s], 2 * T);
-            tma_load(x, &map_x, 0, row, &s_full[s]);
-            tma_load(x + BOX, &map_x, 64, row, &s_full[s]);
-            tma_load(x + T, &map_y, 0, row, &s_full[s]);
-            tma_load(x + T + BOX, &map_y, 64, row, &s_full[s]);
+            tma_load(x, map_x, 0, row, &s_full[s]);
+            tma_load(x + BOX, map_x, 64, row, &s_full[s]);
+            tma_load(x + T, map_y, 0, row, &s_full[s]);
+            tma_load(x + T + BOX, map_y, 64, row, &s_full[s]);
         }
     } else if (tid == 32) {                              // MMAs
         for (uint32_t i = 0; i < mine && ok; ++i) {
@@ -478,7 +490,7 @@ __global__ void __launch_bounds__(128, 1)
     }
     tc_fence_after();
     const uint32_t used = all && got ? (mine < (uint32_t)kWgAcc ? mine : (uint32_t)kWgAcc) : 0u;
-    uint4* o = reinterpret_cast<uint4*>(g.partial + ((size_t)blockIdx.x * 128 + tid) * N);
+    uint4* o = reinterpret_cast<uint4*>(g.partial + ((size_t)(blockIdx.y * gridDim.x + blockIdx.x) * 128 + tid) * N);
     const uint32_t quarter = (uint32_t)(w * 32) << 16;   // feature row tid of dW
 #pragma unroll 1
     for (int c0 = 0; c0 < N; c0 += 16) {
@@ -500,12 +512,12 @@ __global__ void __launch_bounds__(128, 1)
 
 // Adds the partials: 32 outputs per block (128 bytes of each partial), its
 // eight warps taking every eighth partial, their sums added in warp order.
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partial, int nparts,
-                                                      int count, float* __restrict__ out,
-                                                      float scale) {
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partials, int nparts,
+                                                      int count, const WgradOuts outs, float scale) {
     __shared__ float s_sum[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
+    const float* __restrict__ partial = partials + (size_t)blockIdx.y * nparts * count;
     float s = 0.f;
     if (i < count) {
 #pragma unroll 8
@@ -517,7 +529,7 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
     s = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += s_sum[k][lane];
-    out[i] = s * scale;
+    outs.dW[blockIdx.y][i] = s * scale;
 }
 
 // The network's edge encoder (its two edge layers) in one kernel, per
@@ -1520,26 +1532,38 @@ void launch_wgrad_t(const WgradArgs& g, int sms, cudaStream_t st) {
     if (grid > tiles) grid = tiles ? tiles : 1;
     k_wgrad<N><<<grid, 128, smem, st>>>(g);
     const int count = 128 * N;
-    k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
+    WgradOuts outs = {};
+    outs.dW[0] = g.dW;
+    k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, outs, g.scale);
 }
 
-bool launch_wgrad_tma(const WgradArgs& g, int sms, cudaStream_t st) {
+bool launch_wgrad_tma(const WgradArgs* gs, int batch, int sms, cudaStream_t st) {
     static std::once_flag once;
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_wgrad_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
     });
     constexpr int count = 128 * 128;
-    if (g.M == 0) return cudaMemsetAsync(g.dW, 0, count * sizeof(float), st) == cudaSuccess;
-    CUtensorMap map_x, map_y;
-    if (!tile_map(&map_x, g.X, g.M, g.ldp ? g.ldp : 128u) ||
-        !tile_map(&map_y, g.dY, g.M, g.ldq ? g.ldq : 128u))
-        return false;
+    const WgradArgs& g = gs[0];
+    WgradMaps maps;
+    WgradOuts outs = {};
+    for (int k = 0; k < batch; ++k) {
+        outs.dW[k] = gs[k].dW;
+        if (g.M == 0) {
+            if (cudaMemsetAsync(gs[k].dW, 0, count * sizeof(float), st) != cudaSuccess) return false;
+        } else if (!tile_map(&maps.x[k], gs[k].X, g.M, gs[k].ldp ? gs[k].ldp : 128u) ||
+                   !tile_map(&maps.y[k], gs[k].dY, g.M, gs[k].ldq ? gs[k].ldq : 128u)) {
+            return false;
+        }
+    }
+    if (g.M == 0) return true;
     const uint32_t tiles = (g.M + 127) / 128;
     uint32_t grid = (tiles + kWgMinTiles - 1) / kWgMinTiles;
-    if (grid > (uint32_t)sms) grid = (uint32_t)sms;
-    if (grid > g.nparts) grid = g.nparts;
-    k_wgrad_tma<<<grid, 128, kWgSmem, st>>>(g, map_x, map_y);
-    k_wgrad_reduce<<<(count + 31) / 32, 256, 0, st>>>(g.partial, (int)grid, count, g.dW, g.scale);
+    const uint32_t most = (uint32_t)sms / (uint32_t)batch, parts = g.nparts / (uint32_t)batch;
+    if (grid > most) grid = most ? most : 1;
+    if (grid > parts) grid = parts;
+    k_wgrad_tma<<<dim3(grid, batch), 128, kWgSmem, st>>>(g, maps);
+    k_wgrad_reduce<<<dim3((count + 31) / 32, batch), 256, 0, st>>>(g.partial, (int)grid, count, outs,
+                                                                   g.scale);
     return true;
 }
 
@@ -1646,8 +1670,12 @@ bool launch_edge_encoder(const EdgeArgs& g, cudaStream_t st) {
     return true;
 }
 
+bool launch_wgrads(const WgradArgs* g, int batch, cudaStream_t st) {
+    return launch_wgrad_tma(g, batch, num_sms(), st);
+}
+
 bool launch_wgrad(int N, const WgradArgs& g, cudaStream_t st) {
-    if (N == 128) return launch_wgrad_tma(g, num_sms(), st);
+    if (N == 128) return launch_wgrad_tma(&g, 1, num_sms(), st);
     if (N == 16) launch_wgrad_t<16>(g, num_sms(), st);
     else return false;
     return true;

@@ -14,6 +14,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -311,6 +312,7 @@ __global__ void k_rowsum(uint32_t n, const uint32_t* __restrict__ rowptr, const 
 // the partials in a fixed order.  (One column per thread read 2 or 4 bytes a
 // lane: 200 us for 1.27M x 128, a quarter to a half of the copy bandwidth.)
 constexpr uint32_t kColParts = 4 * 152;   // blocks: four per SM
+constexpr uint32_t kColRegion = 1024;      // partials that a region of the scratch holds
 
 template <int V>
 __device__ __forceinline__ void colsum_block(const float (&s)[V], int C, float* __restrict__ part) {
@@ -377,13 +379,19 @@ __global__ void __launch_bounds__(256) k_rows_f32(uint32_t M, const float* __res
 // out[c] = the sum of the partials: a block takes up to 32 columns, 1024 / 32
 // slices of the partials in parallel.  (One block for all columns had 76 loads
 // in a row per thread at 608 partials: 14 us.)
-__global__ void __launch_bounds__(1024) k_colsum_final(int nparts, int C,
-                                                       const float* __restrict__ part,
-                                                       float* __restrict__ out) {
+constexpr int kColBatch = 4;   // sums that one launch finishes (blockIdx.y)
+struct ColFinals {
+    const float* part[kColBatch];
+    float* out[kColBatch];
+    int nparts[kColBatch];
+};
+
+__global__ void __launch_bounds__(1024) k_colsum_final(int C, const ColFinals f) {
     __shared__ float s_sum[1024];
-    const int nc = C < 32 ? C : 32;
+    const int nc = C < 32 ? C : 32, nparts = f.nparts[blockIdx.y];
     const int c = threadIdx.x % nc, g = threadIdx.x / nc, ng = 1024 / nc;
     const int col = blockIdx.x * nc + c;
+    const float* __restrict__ part = f.part[blockIdx.y];
     float s = 0.f;
 #pragma unroll 8
     for (int b = g; b < nparts; b += ng) s += part[(size_t)b * C + col];
@@ -392,7 +400,7 @@ __global__ void __launch_bounds__(1024) k_colsum_final(int nparts, int C,
     if (threadIdx.x >= nc) return;
     float t = 0.f;
     for (int k = 0; k < ng; ++k) t += s_sum[k * nc + c];
-    out[col] = t;
+    f.out[blockIdx.y][col] = t;
 }
 
 // Loss over fluid nodes and its gradient: out (n x 16 fp32, sorted order),
@@ -686,7 +694,7 @@ size_t carve(sur_ctx* c, void* base) {
     c->out = cv.take<float>(N * KOUT);
     c->acc = cv.take<float>(N * 3);
     c->partial = cv.take<float>((size_t)kWgradParts * L * L);
-    c->colpart = cv.take<float>((size_t)1024 * 2 * L);
+    c->colpart = cv.take<float>((size_t)kColBatch * kColRegion * L);
     c->losspart = cv.take<float>(nblk(N, 256) + 1);
     c->loss = cv.take<float>(1);
     c->wg_tmp = cv.take<float>((size_t)L * L);
@@ -799,7 +807,7 @@ int edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z,
 // grad of W (kin x kout) += X^T dY over M rows (X: M x kin with stride ldx,
 // dY: M x kout with stride ldy); kin = 16 layers are computed as (dY^T X)^T.
 int wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
-           const __nv_bfloat16* dY, uint32_t ldy, uint32_t M, int kin_half = -1) {
+           const __nv_bfloat16* dY, uint32_t ldy, uint32_t M) {
     WgradArgs g = {};
     g.M = M;
     g.partial = c->partial;
@@ -821,8 +829,34 @@ int wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
     g.ldp = ldx;
     g.dY = dY;
     g.ldq = ldy;
-    g.dW = dst + (kin_half > 0 ? (size_t)kin_half * L * l.kout : 0);
+    g.dW = dst;
     if (!launch_wgrad(l.kout, g, c->st)) return fail(c, SPH_ERR_CUDA, "weight gradient: no tensor maps");
+    return SPH_OK;
+}
+
+// The same for up to kWgradBatch 128 x 128 gradients over the same rows.
+struct Wgrad {
+    const __nv_bfloat16* X;
+    uint32_t ldx;
+    const __nv_bfloat16* dY;    // row stride L
+    size_t w_off;               // of the (half) weight matrix
+};
+
+int wgrads(sur_ctx* c, uint32_t M, std::initializer_list<Wgrad> list) {
+    WgradArgs g[kWgradBatch] = {};
+    int k = 0;
+    for (const Wgrad& w : list) {
+        g[k].X = w.X;
+        g[k].ldp = w.ldx;
+        g[k].dY = w.dY;
+        g[k].ldq = L;
+        g[k].M = M;
+        g[k].partial = c->partial;
+        g[k].nparts = kWgradParts;
+        g[k].scale = 1.f;
+        g[k++].dW = c->g + w.w_off;
+    }
+    if (!launch_wgrads(g, k, c->st)) return fail(c, SPH_ERR_CUDA, "weight gradient: no tensor maps");
     return SPH_OK;
 }
 
@@ -836,27 +870,45 @@ uint32_t col_parts(uint32_t M, uint32_t rpb) {
     return b == 0 ? 1u : (b < kColParts ? b : kColParts);
 }
 
-// out[0:C] = the sums of `parts` partials of C columns (C = 16 or 128).
-void colsum_final(sur_ctx* c, uint32_t parts, int C, const float* part, float* out) {
-    k_colsum_final<<<C < 32 ? 1 : C / 32, 1024, 0, c->st>>>((int)parts, C, part, out);
+// A pending column sum: `parts` partials in region k of colpart, added up by
+// col_finals (C = 16 or 128 columns).
+struct ColSum {
+    int region;
+    uint32_t parts;
+    float* out;
+};
+
+float* col_region(sur_ctx* c, int k) { return c->colpart + (size_t)k * kColRegion * L; }
+
+void col_finals(sur_ctx* c, int C, std::initializer_list<ColSum> sums) {
+    ColFinals f = {};
+    int k = 0;
+    for (const ColSum& s : sums) {
+        if (s.parts == 0) continue;
+        f.part[k] = col_region(c, s.region);
+        f.out[k] = s.out;
+        f.nparts[k++] = (int)s.parts;
+    }
+    if (k) k_colsum_final<<<dim3(C < 32 ? 1 : C / 32, k), 1024, 0, c->st>>>(C, f);
 }
 
-// Column sums of an (M x C) bf16 matrix into out[0:C].
-void colsum(sur_ctx* c, const __nv_bfloat16* in, uint32_t M, int C, uint32_t ld, float* out) {
+// Column sums of an (M x C) bf16 matrix for out[0:C], pending in a region.
+ColSum colsum(sur_ctx* c, int region, const __nv_bfloat16* in, uint32_t M, int C, uint32_t ld, float* out) {
     const uint32_t parts = col_parts(M, 256 / (C / 8));
-    k_colsum_bf16<<<parts, 256, 0, c->st>>>(M, C, in, ld, c->colpart);
-    colsum_final(c, parts, C, c->colpart, out);
+    k_colsum_bf16<<<parts, 256, 0, c->st>>>(M, C, in, ld, col_region(c, region));
+    return {region, parts, out};
 }
 
-// bf16 copy of acc (M x 128 fp32) to out_bf, column sums to out.
-void rows_f32(sur_ctx* c, const float* acc, uint32_t M, __nv_bfloat16* out_bf, float* out) {
+// bf16 copy of acc (M x 128 fp32) to out_bf, column sums for out.
+ColSum rows_f32(sur_ctx* c, int region, const float* acc, uint32_t M, __nv_bfloat16* out_bf, float* out) {
     const uint32_t parts = col_parts(M, 8);
-    k_rows_f32<<<parts, 256, 0, c->st>>>(M, acc, out_bf, c->colpart);
-    colsum_final(c, parts, L, c->colpart, out);
+    k_rows_f32<<<parts, 256, 0, c->st>>>(M, acc, out_bf, col_region(c, region));
+    return {region, parts, out};
 }
 
-// The backward pass of edge_layer (dE, dEb, dpre and both bias gradients).
-int edge_backward(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* z) {
+// The backward pass of edge_layer (dE, dEb, dpre); the column sums of v and dpre,
+// pending in regions 2 and 3, are the gradients of b2 and b1.
+int edge_backward(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* z, uint32_t* parts) {
     EdgeBwdArgs g = {};
     g.dE = c->dE;
     g.node = c->dXN + L;
@@ -868,14 +920,9 @@ int edge_backward(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloa
     g.M = c->E;
     g.dEb = c->dEb;
     g.dpre = c->dpre;
-    g.part_v = c->colpart;
-    g.part_p = c->colpart + (size_t)1024 * L;
-    uint32_t parts = 0;
-    if (!launch_edge_backward(g, &parts, c->st)) return fail(c, SPH_ERR_CUDA, "edge layer: no tensor maps");
-    if (parts) {
-        colsum_final(c, parts, L, g.part_v, c->g + l2.b_off);
-        colsum_final(c, parts, L, g.part_p, c->g + l1.b_off);
-    }
+    g.part_v = col_region(c, 2);
+    g.part_p = col_region(c, 3);
+    if (!launch_edge_backward(g, parts, c->st)) return fail(c, SPH_ERR_CUDA, "edge layer: no tensor maps");
     return SPH_OK;
 }
 
@@ -1001,10 +1048,10 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
     // decoder
     const Layer* dec = &Ls[4 + 6 * c->NL];
     __nv_bfloat16* h_last = c->XN[c->NL];
-    colsum(c, c->dout, n, KOUT, KOUT, c->g + dec[1].b_off);
+    col_finals(c, KOUT, {colsum(c, 0, c->dout, n, KOUT, KOUT, c->g + dec[1].b_off)});
     if ((rc = wgrad(c, dec[1], c->D1, L, c->dout, KOUT, n))) return rc;
     if ((rc = linear(c, c->dout, 0, dec[1], true, n, kEpiReluMask, c->D1, L, c->dD1, nullptr, L))) return rc;
-    colsum(c, c->dD1, n, L, L, c->g + dec[0].b_off);
+    col_finals(c, L, {colsum(c, 0, c->dD1, n, L, L, c->g + dec[0].b_off)});
     if ((rc = wgrad(c, dec[0], h_last, 2 * L, c->dD1, L, n))) return rc;
     if ((rc = linear(c, c->dD1, 0, dec[0], true, n, kEpiNone, nullptr, 0, nullptr, c->dH, L))) return rc;
     cudaMemsetAsync(c->dE, 0, (size_t)E * L * sizeof(float), st);
@@ -1015,16 +1062,19 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
         __nv_bfloat16* z1 = c->Z1[l];
         __nv_bfloat16* y1 = c->Y1[l];
         // node update h' = h + W4 relu(W3 [h, agg] + b3) + b4
-        rows_f32(c, c->dH, n, c->dHb, c->g + w[5].b_off);
-        if ((rc = wgrad(c, w[5], y1, L, c->dHb, L, n))) return rc;
+        const ColSum b4 = rows_f32(c, 0, c->dH, n, c->dHb, c->g + w[5].b_off);
         if ((rc = linear(c, c->dHb, 0, w[5], true, n, kEpiReluMask, y1, L, c->dY1, nullptr, L))) return rc;
-        colsum(c, c->dY1, n, L, L, c->g + w[4].b_off);
-        if ((rc = wgrad(c, w[4], xn_cur, 2 * L, c->dY1, L, n, 0))) return rc;
-        if ((rc = wgrad(c, w[4], xn_cur + L, 2 * L, c->dY1, L, n, 1))) return rc;
+        const ColSum b3 = colsum(c, 1, c->dY1, n, L, L, c->g + w[4].b_off);
+        if ((rc = wgrads(c, n, {{y1, L, c->dHb, w[5].w_off},
+                                {xn_cur, 2 * L, c->dY1, w[4].w_off},
+                                {xn_cur + L, 2 * L, c->dY1, w[4].w_off + (size_t)L * L}})))
+            return rc;
         if ((rc = linear(c, c->dY1, 0, w[4], true, n, kEpiNone, nullptr, 0, nullptr, c->dXN, 2 * L))) return rc;
         k_add_strided<<<nblk((size_t)n * L, 256), 256, 0, st>>>(n, c->dH, c->dXN, 2 * L);
         // aggregation and edge update e' = e + W2 relu(pre) + b2
-        if ((rc = edge_backward(c, w[2], w[3], z1))) return rc;
+        uint32_t parts = 0;
+        if ((rc = edge_backward(c, w[2], w[3], z1, &parts))) return rc;
+        col_finals(c, L, {b4, b3, {2, parts, c->g + w[3].b_off}, {3, parts, c->g + w[2].b_off}});
         if ((rc = wgrad(c, w[3], z1, L, c->dEb, L, E))) return rc;
         if ((rc = wgrad(c, w[2], e_in, L, c->dpre, L, E))) return rc;
         // pre = W1a h_i + W1b h_j + ...: sums over the edges of i and of j
@@ -1032,22 +1082,23 @@ int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
                                                                            c->dPb, nullptr, L);
         k_rowsum<__nv_bfloat16><<<nblk((size_t)n * 32, 256), 256, 0, st>>>(n, c->rowptr, c->dpre, c->rev,
                                                                            c->dQb, nullptr, L);
-        if ((rc = wgrad(c, w[0], xn_cur, 2 * L, c->dPb, L, n))) return rc;
-        if ((rc = wgrad(c, w[1], xn_cur, 2 * L, c->dQb, L, n))) return rc;
+        if ((rc = wgrads(c, n, {{xn_cur, 2 * L, c->dPb, w[0].w_off}, {xn_cur, 2 * L, c->dQb, w[1].w_off}})))
+            return rc;
         if ((rc = linear(c, c->dPb, 0, w[0], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
         if ((rc = linear(c, c->dQb, 0, w[1], true, n, kEpiAccum, nullptr, 0, nullptr, c->dH, L))) return rc;
     }
     // encoders
-    rows_f32(c, c->dE, E, c->dEb, c->g + Ls[3].b_off);
+    const ColSum be2 = rows_f32(c, 0, c->dE, E, c->dEb, c->g + Ls[3].b_off);
     if ((rc = wgrad(c, Ls[3], c->ee1, L, c->dEb, L, E))) return rc;
     if ((rc = linear(c, c->dEb, 0, Ls[3], true, E, kEpiReluMask, c->ee1, L, c->dEe1, nullptr, L))) return rc;
-    colsum(c, c->dEe1, E, L, L, c->g + Ls[2].b_off);
+    const ColSum be1 = colsum(c, 1, c->dEe1, E, L, L, c->g + Ls[2].b_off);
     if ((rc = wgrad(c, Ls[2], c->xe, KIN, c->dEe1, L, E))) return rc;
-    rows_f32(c, c->dH, n, c->dHb, c->g + Ls[1].b_off);
+    const ColSum bn2 = rows_f32(c, 2, c->dH, n, c->dHb, c->g + Ls[1].b_off);
     if ((rc = wgrad(c, Ls[1], c->en1, L, c->dHb, L, n))) return rc;
     if ((rc = linear(c, c->dHb, 0, Ls[1], true, n, kEpiReluMask, c->en1, L, c->dEn1, nullptr, L))) return rc;
-    colsum(c, c->dEn1, n, L, L, c->g + Ls[0].b_off);
+    const ColSum bn1 = colsum(c, 3, c->dEn1, n, L, L, c->g + Ls[0].b_off);
     if ((rc = wgrad(c, Ls[0], c->xn, KIN, c->dEn1, L, n))) return rc;
+    col_finals(c, L, {be2, be1, bn2, bn1});
     if (loss_host) {
         cudaMemcpyAsync(loss_host, c->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) return check(c, "sur_backward");
