@@ -19,8 +19,8 @@
 // latency but cost a hundred instructions per warp and piece: 20.4 against
 // 18.8 ms at 35.4M particles.)  Both sides on one GB300, ms per launch (the
 // counter-scheduled 4 x 2 shape of sph_kernels.cu / this kernel): 35.4M
-// particles 24.0 / 18.8, 1.39M with obstacles 0.956 / 0.713, 256 dam breaks
-// (5.5M) 3.85 / 3.12, 64k with the cubic spline 0.094 / 0.073, 17k 0.0229 /
+// particles 24.0 / 18.3, 1.39M with obstacles 0.956 / 0.697, 256 dam breaks
+// (5.5M) 3.85 / 3.12, 64k with the cubic spline 0.094 / 0.071, 17k 0.0229 /
 // 0.0196.  Next to the pair phase (0.23 ms of it at 1.39M) the largest share is
 // the units' set-up, 0.20: the latency of the staging copies.
 #include <cuda_fp16.h>
@@ -163,19 +163,46 @@ struct HitCursor {
     uint32_t m, base, next_m, next_base, rp;
 };
 
-// The next hit's entry: base + STEP (bit).  The ending word has no bit: its
-// base makes the entry the pad's from then on.
-template <uint32_t STEP>
-__device__ __forceinline__ uint32_t pop_hit(HitCursor& h, uint32_t end) {
-    uint32_t e;
+// Which candidate a column is: the SPLIT parts of a group take alternate
+// candidates, column c of part p being candidate SPLIT c + p.  With TURN, in
+// turns that change from eight to eight: SPLIT c + (p ^ (c / M mod SPLIT)), M = 8 /
+// SPLIT, because with the same turn throughout a warp's 16-byte loads of its hits
+// meet half of the banks only.  Two more instructions per hit for fewer bank
+// conflicts: ms per launch without / with, 35.4M particles 18.8 / 18.3, 1.39M
+// 0.713 / 0.697; in units of 64 particles (256 dam breaks 3.12 / 3.14) it does not pay.
+template <uint32_t SPLIT, bool TURN>
+struct Turns {
+    static constexpr uint32_t M = 8 / SPLIT, S1 = SPLIT - 1;
+    // the candidate that part p takes of SPLIT consecutive ones, at candidate t
+    static __device__ __forceinline__ uint32_t turn(uint32_t t, uint32_t p) {
+        return TURN ? p ^ ((t >> 3) & S1) : p;
+    }
+    // part and column of candidate t
+    static __device__ __forceinline__ uint32_t part(uint32_t t) { return turn(t, t & S1); }
+    static __device__ __forceinline__ uint32_t column(uint32_t t) { return t / SPLIT; }
+    // columns of part p before candidate t
+    static __device__ __forceinline__ uint32_t before(uint32_t t, uint32_t p) {
+        return (t + S1 - turn(t, p)) / SPLIT;
+    }
+};
+
+// The next hit's entry: base + 16 (SPLIT bit + its turn); mp = M part (TURN).
+// The ending word has no bit (bfind gives all ones): its base makes the entry
+// the pad's from then on.
+template <uint32_t SPLIT, bool TURN>
+__device__ __forceinline__ uint32_t pop_hit(HitCursor& h, uint32_t end, uint32_t mp) {
+    using T = Turns<SPLIT, TURN>;
+    uint32_t e, b;
     asm volatile(
-        "{\n .reg .pred p;\n .reg .u32 b, t;\n setp.eq.u32 p, %1, 0;\n @p mov.u32 %1, %3;\n"
+        "{\n .reg .pred p;\n .reg .u32 t;\n setp.eq.u32 p, %1, 0;\n @p mov.u32 %1, %3;\n"
         " @p mov.u32 %2, %4;\n @p ld.shared.v2.u32 {%3, %4}, [%5];\n @p add.u32 %5, %5, 256;\n"
-        " @p min.u32 %5, %5, %6;\n bfind.u32 b, %1;\n mov.u32 t, 1;\n shl.b32 t, t, b;\n"
-        " xor.b32 %1, %1, t;\n mad.lo.u32 %0, b, %7, %2;\n}"
-        : "=r"(e), "+r"(h.m), "+r"(h.base), "+r"(h.next_m), "+r"(h.next_base), "+r"(h.rp)
-        : "r"(end), "n"(STEP)
+        " @p min.u32 %5, %5, %6;\n bfind.u32 %0, %1;\n mov.u32 t, 1;\n shl.b32 t, t, %0;\n"
+        " xor.b32 %1, %1, t;\n}"
+        : "=&r"(b), "+r"(h.m), "+r"(h.base), "+r"(h.next_m), "+r"(h.next_base), "+r"(h.rp)
+        : "r"(end)
         : "memory");
+    e = h.base + b * (16u * SPLIT);
+    if (TURN) e += ((b & (T::M * T::S1)) ^ mp) * (16u / T::M);
     return e;
 }
 
@@ -273,6 +300,8 @@ template <int W, int SPLIT, int STAGE, int WCAP, int PIECE, int MINB, bool COUNT
 __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev d,
                                                                       const InteractArgs a) {
     using SH = TcShape<W, SPLIT, STAGE, WCAP, PIECE>;
+    constexpr bool TURN = W == 4;
+    using TN = Turns<SPLIT, TURN>;
     constexpr int NW = W * SPLIT, NT = NW * 32;
     constexpr int FBCAP = SH::fb_cap;
     constexpr uint32_t kPad = (uint32_t)STAGE * 16u;       // list entry of the pad slot
@@ -484,9 +513,8 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
         ok = mbar_wait_bounded(&s_bar, phase);
         phase ^= 1u;
         // The staged candidates go through the tensor cores in pieces of
-        // PIECE.  Candidate t of a piece is row (t mod SPLIT) kPartCols + t /
-        // SPLIT of operand B, so a part's accumulator columns are contiguous
-        // and the parts take alternate candidates.
+        // PIECE.  Operand B's rows are ordered so that a part's accumulator
+        // columns are contiguous (Turns).
         const uint32_t nst = s_base[9];
         const uint32_t npc = (nst + PIECE - 1) / PIECE;
         // 32 rows of piece k: shift the candidates' y, z into the frame of
@@ -496,7 +524,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
             const uint32_t t = g * 32u + (uint32_t)lane;
             const uint32_t j = k * PIECE + t;
             unsigned char* row =
-                s_b + sur::kmajor_offset((t % SPLIT) * kPartCols + t / SPLIT, 0, 16);
+                s_b + sur::kmajor_offset(TN::part(t) * kPartCols + TN::column(t), 0, 16);
             if (j < nst) {
                 int r = 0;
 #pragma unroll
@@ -589,14 +617,13 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                 }
                 const uint32_t p0 = k * PIECE, p1 = p0 + PIECE;
                 const uint32_t tcol = lane_base + part * kPartCols;
-                const uint32_t e0 = (p0 + part) * 16u;
+                const uint32_t e0 = (p0 + (TURN ? 0u : (uint32_t)part)) * 16u;
                 while (wa < p1) {
-                    // columns [ca, cb) of this part: candidates p0 + SPLIT c + part.
+                    // columns [ca, cb) of this part.
                     // The test rejects the neighbouring columns of a load (of
                     // candidates outside the window), so loads are cut at 8.
                     const uint32_t ja = wa > p0 ? wa - p0 : 0u, jb = (wb < p1 ? wb : p1) - p0;
-                    const uint32_t ca = ((ja + SPLIT - 1 - part) / SPLIT) & ~7u;
-                    const uint32_t cb = (jb + SPLIT - 1 - part) / SPLIT;
+                    const uint32_t ca = TN::before(ja, part) & ~7u, cb = TN::before(jb, part);
                     c = ca > c ? ca : c;
                     while (c < cb) {
                         full = __any_sync(kFull, lp >= list0 + WCAP * 256u);
@@ -666,7 +693,8 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
             // halves); lanes that run out get the pad, which contributes
             // nothing and is not counted
             const uint32_t mx = __reduce_max_sync(kFull, hits);
-            const uint32_t pad_base = kPad + 16u * SPLIT;
+            const uint32_t pad_base = kPad + 16u * (TURN ? 1u + (uint32_t)part : (uint32_t)SPLIT);
+            const uint32_t mp = TN::M * (uint32_t)part;
             asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(lp), "r"(0u), "r"(pad_base)
                          : "memory");
             HitCursor hc = {0u, pad_base, 0u, pad_base, list0};
@@ -676,7 +704,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                          : "memory");
             hc.rp = list0 + 256u < lp ? list0 + 256u : lp;
             for (uint32_t t = 0; t < mx; t += 2) {
-                uint32_t e0 = pop_hit<16 * SPLIT>(hc, lp), e1 = pop_hit<16 * SPLIT>(hc, lp);
+                uint32_t e0 = pop_hit<SPLIT, TURN>(hc, lp, mp), e1 = pop_hit<SPLIT, TURN>(hc, lp, mp);
                 if (!in_bounds(e0 < s_base[9] * 16u || e0 == kPad, d.status)) e0 = kPad;
                 if (!in_bounds(e1 < s_base[9] * 16u || e1 == kPad, d.status)) e1 = kPad;
                 const float4 pa = *reinterpret_cast<const float4*>(s_raw + e0);
@@ -889,11 +917,11 @@ Variant tc_variant() {
 
 // Large systems run best in 128-particle units on two blocks per SM, small
 // ones and ensembles of small ones in 64-particle units on four (sph_autotune
-// times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.8 /
-// 24.0, 1.39M 0.713 / 0.858, 60k 0.073 / 0.076, 256 dam breaks 3.18 / 3.12, 17k
+// times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.3 /
+// 24.0, 1.39M 0.697 / 0.858, 60k 0.071 / 0.076, 256 dam breaks 3.17 / 3.12, 17k
 // 0.0212 / 0.0196).  Between the first and the third, fourth and seventh,
 // shared memory moves from staged candidates to hit words (larger h/dp has more
-// hits per particle): 1,664 / 18 take 18.8 / 0.719 ms.
+// hits per particle): 1,664 / 18 take 18.3 / 0.704 ms.
 Variant tc_variant_n(int k) {
     switch (k) {
         case 0: return tc_variant<4, 2, 1760, 16, 256, 2>();
