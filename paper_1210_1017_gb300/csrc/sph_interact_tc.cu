@@ -19,8 +19,8 @@
 // latency but cost a hundred instructions per warp and piece: 20.4 against
 // 18.8 ms at 35.4M particles.)  Both sides on one GB300, ms per launch (the
 // counter-scheduled 4 x 2 shape of sph_kernels.cu / this kernel): 35.4M
-// particles 24.0 / 18.3, 1.39M with obstacles 0.956 / 0.697, 256 dam breaks
-// (5.5M) 3.85 / 3.12, 64k with the cubic spline 0.094 / 0.071, 17k 0.0229 /
+// particles 24.0 / 18.4, 1.39M with obstacles 0.956 / 0.701, 256 dam breaks
+// (5.5M) 3.85 / 3.15, 64k with the cubic spline 0.094 / 0.072, 17k 0.0229 /
 // 0.0196.  Next to the pair phase (0.23 ms of it at 1.39M) the largest share is
 // the units' set-up, 0.20: the latency of the staging copies.
 #include <cuda_fp16.h>
@@ -467,7 +467,6 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
     const uint32_t xi = __float_as_uint(pi.x);
     const float rri = vi.w * d.inv_rho0;
     const float ci = c0 * rri * rri * rri;
-    const float ri3 = rri * rri * rri, visc_k = -d.alpha * d.h * c0;
     // MMA operand A: the warps of the first four TMEM lane quarters write
     // their particles' rows (a group shared by several quarters is repeated)
     if (w < 4) {
@@ -719,9 +718,9 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                 const float2 dy = __ffma2_rn(ff2(pa.y, pb.y), m1, dup2(pi.y));
                 const float2 dz = __ffma2_rn(ff2(pa.z, pb.z), m1, dup2(pi.z));
                 if (anyfluid)
-                    pair_terms2<KERN, true>(d, visc_k, pi, vi, ri3, dx, dy, dz, pa, va, pb, vb, acc2);
+                    pair_terms2<KERN, true>(d, c0, pi, vi, ci, dx, dy, dz, pa, va, pb, vb, acc2);
                 else
-                    pair_terms2<KERN, false>(d, visc_k, pi, vi, ri3, dx, dy, dz, pa, va, pb, vb, acc2);
+                    pair_terms2<KERN, false>(d, c0, pi, vi, ci, dx, dy, dz, pa, va, pb, vb, acc2);
             }
             acc.np += (uint32_t)acc2.npf.x + (uint32_t)acc2.npf.y;
             acc2.npf = dup2(0.f);
@@ -734,7 +733,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
             mbar_wait_bounded(&s_mbar, mphase);
             break;
         }
-        add_pairs2(d, acc2, acc);
+        add_pairs2(acc2, acc);
     } else {
         if (w == 0) make_plan(&s_plan[sb ^ 1], s_nui);
         __syncthreads();
@@ -917,11 +916,11 @@ Variant tc_variant() {
 
 // Large systems run best in 128-particle units on two blocks per SM, small
 // ones and ensembles of small ones in 64-particle units on four (sph_autotune
-// times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.3 /
-// 24.0, 1.39M 0.697 / 0.858, 60k 0.071 / 0.076, 256 dam breaks 3.17 / 3.12, 17k
+// times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.4 /
+// 24.2, 1.39M 0.701 / 0.865, 60k 0.072 / 0.077, 256 dam breaks 3.20 / 3.15, 17k
 // 0.0212 / 0.0196).  Between the first and the third, fourth and seventh,
 // shared memory moves from staged candidates to hit words (larger h/dp has more
-// hits per particle): 1,664 / 18 take 18.3 / 0.704 ms.
+// hits per particle): 1,664 / 18 take 18.4 / 0.709 ms.
 Variant tc_variant_n(int k) {
     switch (k) {
         case 0: return tc_variant<4, 2, 1760, 16, 256, 2>();

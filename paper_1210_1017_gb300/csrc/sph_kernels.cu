@@ -179,7 +179,13 @@ __global__ void __launch_bounds__(256) k_reorder(const Dev d, const ReorderArgs 
         pc.y = __double2float_rn(y - (I.y0 + (double)cy * d.cs));
         pc.z = __double2float_rn(z - (I.z0 + (double)cz * d.cs));
         pc.w = p_over_rho2(d, I.B, vr.w);
-        xu = (cx << 26) + (uint32_t)__float2int_rn(pc.x * (67108864.0f / d.csf));
+        // pc.x in units of csf 2^-26, rounded once: the factor and the product
+        // in two floats each (a plain product would round to 2^-25 of a cell and
+        // scale all positions by the rounding of the factor)
+        const float kh = 67108864.0f / d.csf, kl = fmaf(-kh, d.csf, 67108864.0f) / d.csf;
+        const float u = pc.x * kh, ui = rintf(u);
+        const float ul = fmaf(pc.x, kl, fmaf(pc.x, kh, -u));
+        xu = (cx << 26) + (uint32_t)(__float2int_rn(ui) + __float2int_rn((u - ui) + ul));
     }
     a.posc[dst] = pc;
     a.posu[dst] = make_float4(__uint_as_float(xu), pc.y, pc.z, pc.w);
@@ -408,7 +414,6 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
     }
     const float rri = vi.w * d.inv_rho0;
     const float ci = c0 * rri * rri * rri;
-    const float ri3 = rri * rri * rri, visc_k = -d.alpha * d.h * c0;
     PairAcc acc = {0.f, 0.f, 0.f, 0.f, 0.f, 0u};
     uint32_t ncand = 0;
     __syncthreads();
@@ -598,10 +603,10 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
                     const float2 dy2 = __ffma2_rn(ff2(pp[0].y, pp[1].y), m1, dup2(pi.y));
                     const float2 dz2 = __ffma2_rn(ff2(pp[0].z, pp[1].z), m1, dup2(pi.z));
                     if (anyfluid)
-                        pair_terms2<KERN, true>(d, visc_k, pi, vi, ri3, dx2, dy2, dz2, pp[0], vv[0],
+                        pair_terms2<KERN, true>(d, c0, pi, vi, ci, dx2, dy2, dz2, pp[0], vv[0],
                                                 pp[1], vv[1], acc2);
                     else
-                        pair_terms2<KERN, false>(d, visc_k, pi, vi, ri3, dx2, dy2, dz2, pp[0], vv[0],
+                        pair_terms2<KERN, false>(d, c0, pi, vi, ci, dx2, dy2, dz2, pp[0], vv[0],
                                                  pp[1], vv[1], acc2);
                 }
                 __syncwarp();   // every lane is done reading before the words are reused
@@ -682,7 +687,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
                 }
             }
             flush();
-            add_pairs2(d, acc2, acc);
+            add_pairs2(acc2, acc);
         } else {
             // candidates straight from global memory (unit too large to stage)
             uint32_t* lst = reinterpret_cast<uint32_t*>(s_raw) + w * (FBCAP * 32);

@@ -206,10 +206,8 @@ __device__ void reduce_counters_and_dt(const Dev& d, const ReduceArgs& a, int se
 }
 
 // Packed accumulators of two pair streams (the two pairs a lane evaluates
-// per step of the pair phase), one in each half of a float2.  Constant
-// factors are left out of the sums and applied once by add_pairs2: the
-// gradient factor fc (and the sign of Eq. 9, whose sums hold +sum f r_ij) and
-// the h of mu.
+// per step of the pair phase), one in each half of a float2.  The momentum
+// sums hold +sum f r_ij (negated once by add_pairs2, which is exact).
 struct PairAcc2 {
     float2 ax, ay, az, dr, npf;
     float mu;
@@ -228,15 +226,14 @@ __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 // counted, which lets lane work be padded with one.  Masks are products with
 // 0 or 1 rather than selects, keeping the integer/logic pipe free.  MOM:
 // evaluate the momentum terms (a warp-uniform choice).
-// The pair phase is bound by instruction issue and by the registers of its
-// duplicated constants, so constant factors are pulled out of the sums
-// (PairAcc2) and c_j + c_i is c0 (rr_j^3 + ri3), rr = rho / rho_0, with ri3 =
-// rr_i^3 handed in; visc_k = -alpha h c0.  (With the factors inside, the
-// 35.4M-particle launch of the counter-scheduled 4 x 2 shape took 24.3
-// against 24.0 ms, the 1.39M one 0.968 against 0.956.)
+// Same arithmetic per pair as pair_terms, factor by factor: with the constant
+// factors pulled out of the sums a launch is 0.5 to 1% faster (1.39M particles
+// 0.697 against 0.701 ms), but every term is rounded differently, and after 30
+// steps the positions are 1.2e-9 instead of 0.9e-9 from those of another order of
+// the same sums.
 template <int KERN, bool MOM>
-__device__ __forceinline__ void pair_terms2(const Dev& d, float visc_k, const float4& pi,
-                                            const float4& vi, float ri3, float2 dx, float2 dy,
+__device__ __forceinline__ void pair_terms2(const Dev& d, float c0, const float4& pi,
+                                            const float4& vi, float ci, float2 dx, float2 dy,
                                             float2 dz, const float4& pa, const float4& va,
                                             const float4& pb, const float4& vb, PairAcc2& s) {
     const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
@@ -244,20 +241,19 @@ __device__ __forceinline__ void pair_terms2(const Dev& d, float visc_k, const fl
     const float2 use = ff2(__saturatef(fmaf(d2.x, -0x1p100f, r2s)),
                            __saturatef(fmaf(d2.y, -0x1p100f, r2s)));
     s.npf = __fadd2_rn(s.npf, use);
-    const float2 r = ff2(sqrt_approx(d2.x), sqrt_approx(d2.y));
+    const float2 q = __fmul2_rn(ff2(sqrt_approx(d2.x), sqrt_approx(d2.y)), dup2(d.inv_h));
     float2 shape;
     if (KERN == 1) {
-        const float2 q = __fmul2_rn(r, dup2(d.inv_h));
         const float2 wo = __ffma2_rn(q, dup2(-1.0f), dup2(2.0f));
         const float2 outer =
             __fmul2_rn(__fmul2_rn(dup2(-0.75f), __fmul2_rn(wo, wo)), ff2(rcp_approx(q.x), rcp_approx(q.y)));
         const float2 inner = __ffma2_rn(dup2(2.25f), q, dup2(-3.0f));
         shape = ff2(q.x < 1.0f ? inner.x : outer.x, q.y < 1.0f ? inner.y : outer.y);
     } else {
-        const float2 wq = __ffma2_rn(r, dup2(-0.5f * d.inv_h), dup2(1.0f));
+        const float2 wq = __ffma2_rn(dup2(-0.5f), q, dup2(1.0f));
         shape = __fmul2_rn(__fmul2_rn(wq, wq), wq);
     }
-    const float2 F = __fmul2_rn(shape, use);
+    const float2 F = __fmul2_rn(__fmul2_rn(dup2(d.fc), shape), use);
     const float2 m1 = dup2(-1.0f);
     const float2 dvx = __ffma2_rn(ff2(va.x, vb.x), m1, dup2(vi.x));
     const float2 dvy = __ffma2_rn(ff2(va.y, vb.y), m1, dup2(vi.y));
@@ -266,30 +262,29 @@ __device__ __forceinline__ void pair_terms2(const Dev& d, float visc_k, const fl
     s.dr = __ffma2_rn(vr, F, s.dr);                                 // Eq. 7
     if (MOM) {
         const float2 de = __fadd2_rn(d2, dup2(d.eta2));
-        const float2 nu = __fmul2_rn(vr, ff2(rcp_approx(de.x), rcp_approx(de.y)));   // 1/h of Sec. 2.2's
-        const float2 rho = ff2(va.w, vb.w);
-        const float2 rr = __fmul2_rn(rho, dup2(d.inv_rho0));
-        const float2 cs = __ffma2_rn(__fmul2_rn(rr, rr), rr, dup2(ri3));
-        const float2 rs = __fadd2_rn(dup2(vi.w), rho);
-        // Pi_ij only for approaching pairs (v_ij . r_ij < 0, the sign of nu)
+        const float2 nu = __fmul2_rn(__fmul2_rn(dup2(d.h), vr), ff2(rcp_approx(de.x), rcp_approx(de.y)));
+        const float2 rrj = __fmul2_rn(ff2(va.w, vb.w), dup2(d.inv_rho0));
+        const float2 cj = __fmul2_rn(__fmul2_rn(__fmul2_rn(dup2(c0), rrj), rrj), rrj);
+        const float2 rs = __fadd2_rn(dup2(vi.w), ff2(va.w, vb.w));
         const float2 nmin = ff2(fminf(nu.x, 0.f), fminf(nu.y, 0.f));
-        const float2 visc = __fmul2_rn(__fmul2_rn(cs, nmin), ff2(rcp_approx(rs.x), rcp_approx(rs.y)));
-        const float2 f = __fmul2_rn(
-            __ffma2_rn(visc, dup2(visc_k), __fadd2_rn(dup2(pi.w), ff2(pa.w, pb.w))), F);
-        s.ax = __ffma2_rn(f, dx, s.ax);                              // Eq. 9 (factors later)
+        const float2 visc = __fmul2_rn(
+            __fmul2_rn(__fmul2_rn(dup2(-d.alpha), __fadd2_rn(dup2(ci), cj)), nmin),
+            ff2(rcp_approx(rs.x), rcp_approx(rs.y)));
+        const float2 f = __fmul2_rn(__fadd2_rn(__fadd2_rn(dup2(pi.w), ff2(pa.w, pb.w)), visc), F);
+        s.ax = __ffma2_rn(f, dx, s.ax);                              // Eq. 9 (sign later)
         s.ay = __ffma2_rn(f, dy, s.ay);
         s.az = __ffma2_rn(f, dz, s.az);
         s.mu = fmaxf(s.mu, fmaxf(fabsf(nu.x) * use.x, fabsf(nu.y) * use.y));
     }
 }
 
-// The two streams' sums, in a fixed order, with their constant factors.
-__device__ __forceinline__ void add_pairs2(const Dev& d, const PairAcc2& s, PairAcc& acc) {
-    acc.ax = fmaf(-d.fc, s.ax.x + s.ax.y, acc.ax);
-    acc.ay = fmaf(-d.fc, s.ay.x + s.ay.y, acc.ay);
-    acc.az = fmaf(-d.fc, s.az.x + s.az.y, acc.az);
-    acc.dr = fmaf(d.fc, s.dr.x + s.dr.y, acc.dr);
-    acc.mu = fmaxf(acc.mu, d.h * s.mu);
+// The two streams' sums, in a fixed order.
+__device__ __forceinline__ void add_pairs2(const PairAcc2& s, PairAcc& acc) {
+    acc.ax -= s.ax.x + s.ax.y;
+    acc.ay -= s.ay.x + s.ay.y;
+    acc.az -= s.az.x + s.az.y;
+    acc.dr += s.dr.x + s.dr.y;
+    acc.mu = fmaxf(acc.mu, s.mu);
 }
 
 }  // namespace
