@@ -794,6 +794,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
             }
         }
         flush();
+        fence_staging();   // the lists lie where the next unit's copies go
     }
 
     // parts 1 .. SPLIT-1 hand their sums to part 0, which adds them in part

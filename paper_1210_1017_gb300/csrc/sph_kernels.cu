@@ -808,6 +808,7 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact(const Dev d, 
     t_nb += fluid ? 0u : npairs;
     t_nc += owner ? ncand : 0u;
     if (DYN && pf_off) asm volatile("cp.async.wait_all;" ::: "memory");
+    fence_staging();   // the shifted candidates or the global-memory path's lists
     __syncthreads();   // the next unit overwrites the shared staging
     if (DYN) {
         ui = nui;

@@ -64,6 +64,13 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
+// This thread's plain stores to the staging area before the bulk copies that
+// another unit issues into it behind the next block barrier (the copies are of
+// the asynchronous proxy, which a barrier alone does not order after them).
+__device__ __forceinline__ void fence_staging() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
