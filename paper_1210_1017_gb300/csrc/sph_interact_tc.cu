@@ -673,8 +673,10 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
                 in_piece = false;
             }
             if (!full) {
-                // every piece read (or a wait that gave up): the next unit's
-                // plan, then its cell offsets
+                // every piece read (or a wait that gave up): the last one's
+                // accumulators before the next unit's first MMA (the barrier
+                // below), the next unit's plan, then its cell offsets
+                sur::tc_fence_before();
                 if (w == 0) {
                     asm volatile("cp.async.wait_all;" ::: "memory");
                     __syncwarp();

@@ -65,3 +65,28 @@ def test_dense_and_staged_units_in_turn():
             np.maximum(ref["sa"][fluid], 1e-300)
         assert ea.max() <= 2e-5, (v, ea.max())
     sim.close()
+
+
+@pytest.mark.parametrize("h_over_dp", [1.1, 1.7])
+def test_units_of_one_and_of_several_pieces(h_over_dp):
+    """Units of at most 256 candidates (one product) and of several: the next
+    unit's product overwrites accumulators that the last piece's readers hold."""
+    case = cases.random_block(30000, seed=13, h_over_dp=h_over_dp, jitter=0.2)
+    sim = S.Simulation.from_case(case)
+    sim.build_cells()
+    st = sim.download()
+    ref = oracle.Oracle(case.params()).interact(
+        oracle.State(st["pos"], st["vel"], st["rho"], st["ids"]))
+    fluid = st["ids"] >= case.n_bound
+    for v in range(7):
+        sim.set_variant(v)
+        first = None
+        for _ in range(4):
+            sim.interact()
+            sim.check()
+            ace = sim.read(S.SPH_ARRAY_ACE)
+            first = ace if first is None else first
+            assert np.array_equal(ace, first), v
+        ea = np.linalg.norm(first[fluid, :3] - ref["a"][fluid], axis=1) / ref["sa"][fluid]
+        assert ea.max() <= 2e-5, (v, ea.max())
+    sim.close()
