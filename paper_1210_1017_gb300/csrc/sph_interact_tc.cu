@@ -863,6 +863,8 @@ __global__ void __launch_bounds__(W * SPLIT * 32, MINB) k_interact_tc(const Dev 
     }
     sb ^= 1;
     }
+    // (a wait that gave up: the next unit's record may still be on its way)
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // the last block to finish rearms the unit counter for the next launch
     // (every block's last take precedes its finish ticket)
     __threadfence();
