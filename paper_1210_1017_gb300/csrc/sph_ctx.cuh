@@ -10,6 +10,7 @@
 
 #include "../../include/sph.h"
 #include "sph_internal.cuh"
+#include "sph_place.cuh"
 
 namespace sph {
 
@@ -129,18 +130,6 @@ struct TraceRange {
 inline void drop_pending_counts(sph_ctx* c, cudaStream_t st) {
     if (c->keys_ready) cudaMemsetAsync(c->cnt, 0, (c->ncells + 1) * sizeof(uint32_t), st);
     c->keys_ready = false;
-}
-
-// Whether p is memory of the current device, which a kernel may read or write
-// in place of a staging copy (host, managed and peer memory are staged).
-inline bool on_this_device(const void* p) {
-    cudaPointerAttributes at{};
-    int dev = -1;
-    if (!p || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
 // Record a one-line error message on the context and return the code.
