@@ -12,6 +12,7 @@ CSRC = os.path.join(ROOT, "paper_1210_1017_gb300", "csrc")
 RUNTIME = r"""
 #include "sph_place.cuh"
 #include <cstdio>
+#include <initializer_list>
 // device 0 is current; 1 MB each at 0x10000000 (its memory), 0x20000000 (of
 // device 1), 0x30000000 (managed), 0x40000000 (pinned host)
 static const uintptr_t MB = 1u << 20;
