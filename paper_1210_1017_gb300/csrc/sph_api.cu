@@ -669,20 +669,20 @@ int sph_upload(sph_ctx* c, const double* pos, const float* vel, const float* rho
     const double* spos = pos;
     const float *svel = vel, *srho = rho;
     int rc = SPH_OK;
-    if (!on_this_device(pos)) {
+    if (!on_this_device(pos, 3 * n)) {
         spos = c->stage_pos;
         rc = cuda_check(c, cudaMemcpyAsync(c->stage_pos, pos, 3 * n * sizeof(double), cudaMemcpyDefault, st), "upload pos");
         if (rc) return rc;
     }
-    if (!on_this_device(vel)) {
+    if (!on_this_device(vel, 3 * n)) {
         svel = c->stage_vr;
         cudaMemcpyAsync(c->stage_vr, vel, 3 * n * sizeof(float), cudaMemcpyDefault, st);
     }
-    if (!on_this_device(rho)) {
+    if (!on_this_device(rho, n)) {
         srho = c->stage_vr + 3 * n;
         cudaMemcpyAsync(c->stage_vr + 3 * n, rho, n * sizeof(float), cudaMemcpyDefault, st);
     }
-    const bool ids_here = on_this_device(ids);
+    const bool ids_here = on_this_device(ids, n);
     if (!ids_here)
         cudaMemcpyAsync(c->id[c->cur], ids, n * sizeof(uint32_t), cudaMemcpyDefault, st);
     cudaMemsetAsync(c->id_flag, 0, sizeof(uint32_t), st);
@@ -898,8 +898,8 @@ int sph_download(sph_ctx* c, double* pos, float* vel, float* rho, uint32_t* ids)
     cudaStream_t st = c->st;
     // arrays of this device are written in place, others from the staging
     // (cudaMemcpyDefault: any destination, unified addressing)
-    const bool hp = on_this_device(pos), hv = on_this_device(vel), hr = on_this_device(rho),
-               hi = on_this_device(ids);
+    const bool hp = on_this_device(pos, 3 * n), hv = on_this_device(vel, 3 * n),
+               hr = on_this_device(rho, n), hi = on_this_device(ids, n);
     double* dpos = hp ? pos : c->stage_pos;
     float* dv = hv ? vel : c->stage_vr;
     float* dr = hr ? rho : c->stage_vr + 3 * n;
@@ -927,7 +927,8 @@ int sph_download_by_id(sph_ctx* c, double* pos, float* vel, float* rho) {
     if (!c->ids_dense) return fail(c, SPH_ERR_STATE, "ids are not all below n");
     const size_t n = c->n;
     cudaStream_t st = c->st;
-    const bool hp = on_this_device(pos), hv = on_this_device(vel), hr = on_this_device(rho);
+    const bool hp = on_this_device(pos, 3 * n), hv = on_this_device(vel, 3 * n),
+               hr = on_this_device(rho, n);
     double* dpos = hp ? pos : c->stage_pos;
     float* dv = hv ? vel : c->stage_vr;
     float* dr = hr ? rho : c->stage_vr + 3 * n;

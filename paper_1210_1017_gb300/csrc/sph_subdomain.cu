@@ -300,8 +300,9 @@ extern "C" int sph_subdomain_select(sph_ctx* c, int mode, double xlo, double xhi
     }
     // gather straight into destinations on this device, else into the
     // transfer staging (ids into the free key buffer)
-    const bool dp = on_this_device(pos), dv = on_this_device(vel), dr = on_this_device(rho),
-               di = on_this_device(ids);
+    const size_t m3 = 3 * (size_t)m;
+    const bool dp = on_this_device(pos, m3), dv = on_this_device(vel, m3),
+               dr = on_this_device(rho, m), di = on_this_device(ids, m);
     double* spos = dp ? pos : c->stage_pos;
     float* svel = dv ? vel : c->stage_vr;
     float* srho = dr ? rho : c->stage_vr + 3 * (size_t)n;

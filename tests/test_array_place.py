@@ -2,7 +2,8 @@
 (csrc/sph_place.cuh), against a stand-in for the CUDA runtime that knows a few
 allocations: device memory of another address than the element's alignment is
 staged, as host, managed and peer memory are (a copy takes any address, a kernel's
-access of it would fault)."""
+access of it would fault), and so is an array that reaches past its allocation
+(which a copy refuses)."""
 import os
 import subprocess
 
@@ -27,6 +28,18 @@ extern "C" cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const 
               : v / 0x10000000u == 3 ? cudaMemoryTypeManaged : cudaMemoryTypeHost;
     return cudaSuccess;
 }
+static CUresult range(CUdeviceptr* b, size_t* n, CUdeviceptr p) {
+    *b = p / 0x10000000u * 0x10000000u;
+    *n = MB;
+    return p - *b < MB ? CUDA_SUCCESS : CUDA_ERROR_NOT_FOUND;
+}
+extern "C" cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned,
+                                                        unsigned long long,
+                                                        cudaDriverEntryPointQueryResult* q) {
+    *f = (void*)range;
+    *q = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
 """
 
 
@@ -42,12 +55,24 @@ def _run(tmp_path, body):
 def test_only_aligned_memory_of_this_device_is_used_in_place(tmp_path):
     got = _run(tmp_path, r"""
     for (uintptr_t base : {0x10000000u, 0x20000000u, 0x30000000u, 0x40000000u, 0x50000000u})
-        printf("%d ", sph::on_this_device((const double*)base));
-    printf("%d ", sph::on_this_device((const double*)nullptr));
+        printf("%d ", sph::on_this_device((const double*)base, 3));
+    printf("%d ", sph::on_this_device((const double*)nullptr, 3));
     for (uintptr_t o = 1; o <= 8; ++o)
-        printf("%d%d%d ", sph::on_this_device((const double*)(0x10000000u + o)),
-               sph::on_this_device((float*)(0x10000000u + o)),
-               sph::on_this_device((const uint32_t*)(0x10000000u + o)));
+        printf("%d%d%d ", sph::on_this_device((const double*)(0x10000000u + o), 3),
+               sph::on_this_device((float*)(0x10000000u + o), 3),
+               sph::on_this_device((const uint32_t*)(0x10000000u + o), 3));
     """)
     assert got[:6] == ["1", "0", "0", "0", "0", "0"]
     assert got[6:] == ["000", "000", "000", "011", "000", "000", "000", "111"]
+
+
+def test_an_array_past_its_allocation_is_not_used_in_place(tmp_path):
+    got = _run(tmp_path, r"""
+    const size_t n = MB / 8;
+    const double* p = (const double*)0x10000000u;
+    printf("%d %d %d ", sph::on_this_device(p, n), sph::on_this_device(p, n + 1),
+           sph::on_this_device(p + 1, n));
+    printf("%d %d %d", sph::on_this_device(p + 1, n - 1), sph::on_this_device(p + n - 1, 1),
+           sph::on_this_device(p, SIZE_MAX / 8));
+    """)
+    assert got == ["1", "0", "0", "1", "1", "0"]
