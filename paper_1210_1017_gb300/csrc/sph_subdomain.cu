@@ -5,9 +5,9 @@
 // particles by (label, id), and a copy of the labelled ones.
 //
 // Only the labelled particles are ordered.  While every id is below n (and
-// no two are equal), their order is that of two bit maps over the ids, one per
-// label: the labelling kernel sets a particle's bit and notes its state index
-// under its id, one pass sums the maps' bits per block and one lists the state
+// no two of a label are equal), their order is that of two bit maps over the ids,
+// one per label: the labelling kernel sets a particle's bit and notes its state
+// index under its label and id, one pass sums the maps' bits per block and one lists the state
 // indexes in (label, id) order.  Other ids are sorted: the labelling kernel
 // compacts the labelled particles (their slots come from a warp-aggregated
 // counter, so their order is arbitrary), a sort by id and a stable one by
@@ -44,7 +44,8 @@ struct SubLabelArgs {
     int mode;
     long long xlo, xhi, lo_edge, hi_edge;   // ordered images of the bounds
     uint32_t* key;            // id of each selected particle
-    uint32_t* val;            // (label << 26) | state index; maps: state index by id
+    uint32_t* val;            // (label << 26) | state index
+                              // (maps: state index by id, val label 1, key label 2)
     uint32_t* cnt;            // [0] in-domain count, [1..2] per label, [3] selected,
                               // [4] bits set
     uint32_t* bits;           // bit maps of the ids, label 1 then label 2; null: compact
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(256) k_sub_label(const SubLabelArgs a) {
             if (l != 0u) {
                 const uint32_t id = a.id[k];
                 atomicOr(a.bits + (size_t)(l - 1u) * a.words + (id >> 5), 1u << (id & 31u));
-                a.val[id] = k;
+                (l == 1u ? a.val : a.key)[id] = k;
             }
         } else {
             base = __shfl_sync(kFull, base, 0);
@@ -139,11 +140,12 @@ __global__ void __launch_bounds__(256) k_sub_sums(const uint32_t* __restrict__ b
     }
 }
 
-// State indexes of the set bits in map order: sidx[rank of the bit] =
-// by_id[id].
+// State indexes of the set bits in map order: sidx[rank of the bit] = by_id1[id]
+// in the map of label 1, by_id2[id] in that of label 2.
 __global__ void __launch_bounds__(256) k_sub_list(const uint32_t* __restrict__ bits, uint32_t m,
                                                   uint32_t words, const uint32_t* __restrict__ bsum,
-                                                  const uint32_t* __restrict__ by_id,
+                                                  const uint32_t* __restrict__ by_id1,
+                                                  const uint32_t* __restrict__ by_id2,
                                                   uint32_t* __restrict__ sidx) {
     __shared__ uint32_t s_b[8], s_w[8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(256) k_sub_list(const uint32_t* __restrict__ b
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint32_t i = i0 + j, id0 = 32u * (i < words ? i : i - words);
+        const uint32_t* by_id = i < words ? by_id1 : by_id2;
         for (uint32_t q = b.w[j]; q; q &= q - 1u) sidx[slot++] = by_id[id0 + __ffs(q) - 1];
     }
 }
@@ -259,7 +262,8 @@ extern "C" int sph_subdomain_select(sph_ctx* c, int mode, double xlo, double xhi
     la.cnt = c->sub_cnt;
     la.words = (n + 31u) / 32u;
     const uint32_t map_words = 2u * la.words, map_blocks = sub_bit_blocks(n);
-    // ids all below n: bit maps; two equal ids (fewer bits than particles): sort
+    // ids all below n: bit maps; two equal ids of one label (fewer bits than
+    // particles): sort
     bool maps = c->ids_dense && !c->ids_pending;
     uint32_t cnt[5];
     for (;;) {
@@ -288,7 +292,7 @@ extern "C" int sph_subdomain_select(sph_ctx* c, int mode, double xlo, double xhi
     uint32_t* sidx = c->sub_val[1];            // state indexes in (label, id) order
     if (maps) {
         k_sub_list<<<map_blocks, 256, 0, st>>>(c->sub_bits, map_words, la.words, c->sub_bsum,
-                                               c->sub_val[0], sidx);
+                                               c->sub_val[0], c->sub_key[0], sidx);
     } else {
         // sort A: by id (four places, in place); sort B: stable by label
         launch_radix_sort(c->sub_key[0], c->sub_val[0], c->sub_key[0], c->sub_val[0], c->sub_key[1],

@@ -1,0 +1,55 @@
+"""The sub-domain selection where an id occurs twice: once in each of the two
+labels, twice in one label, and with a particle of neither.  Every labelled
+particle comes out once, under its label, in ascending id (equal ids of one label
+in any order), with its own position, velocity and density."""
+import numpy as np
+import pytest
+
+import __graft_entry__
+from paper_1210_1017_gb300 import cases
+from paper_1210_1017_gb300 import sph as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    __graft_entry__.build()
+    yield
+
+
+@pytest.mark.parametrize("pairs", ["across", "within", "outside", "all"])
+def test_every_selected_particle_comes_out_once(pairs):
+    case = cases.random_block(9000, seed=23, jitter=0.4)
+    case.n_bound = 0
+    x = case.pos[:, 0]
+    lo, hi = float(np.quantile(x, 0.3)), float(np.quantile(x, 0.6))
+    lab = np.where(x < lo, 1, np.where(x >= hi, 2, 0))
+    one, two, none = (np.nonzero(lab == k)[0] for k in (1, 2, 0))
+    if pairs in ("across", "all"):
+        case.ids[two[:40]] = case.ids[one[:40]]
+    if pairs in ("within", "all"):
+        case.ids[one[50:60]] = case.ids[one[60:70]]
+    if pairs in ("outside", "all"):
+        case.ids[none[:20]] = case.ids[one[80:100]]
+    sim = S.Simulation.from_case(case)
+    sim.build_cells()
+    for _ in range(3):
+        got = sim.subdomain_select(S.SPH_SUBDOMAIN_MIGRATE, lo, hi)
+        assert got["counts"].tolist() == [none.size, one.size, two.size]
+        at = 0
+        for sel in (one, two):
+            part = slice(at, at + sel.size)
+            at += sel.size
+            assert np.array_equal(got["ids"][part], np.sort(case.ids[sel]))
+            rows = [np.column_stack([i, p, v, r]) for i, p, v, r in (
+                (got["ids"][part], got["pos"][part], got["vel"][part], got["rho"][part]),
+                (case.ids[sel], case.pos[sel], case.vel[sel].astype(np.float32),
+                 case.rho[sel].astype(np.float32)))]
+            a, b = (r[np.lexsort(r.T[::-1])] for r in rows)
+            assert np.array_equal(a, b)
+    sim.check()
+    sim.close()
