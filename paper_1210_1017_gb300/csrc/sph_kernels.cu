@@ -1141,6 +1141,17 @@ __global__ void __launch_bounds__(kFusedWarps * 32) k_units_fused(const Dev d,
     }
 }
 
+// The rates of sorted particle k in instance q (step size dt), 0 once the
+// instance has ended: they are no longer evaluated then, and a.ace holds what
+// was there (another run's, another particle's), which dt = 0 does not cancel
+// when it is not finite.  (done itself is being set by k_correct; a running
+// instance of infinite rates has dt = 0 as well, but not the time.)
+__device__ __forceinline__ float4 rates(const Dev& d, const IntegrateArgs& a, uint32_t k, uint32_t q,
+                                        double dt) {
+    if (dt == 0.0 && d.is.t[q] >= d.inst[q].t_end) return make_float4(0.f, 0.f, 0.f, 0.f);
+    return a.ace[k];
+}
+
 // Symplectic predictor (half step) for sorted particle k, then its new
 // label.  Boundary particles keep r and v (Sec. 2.3); excluded particles
 // (k >= in-domain count) are left untouched.  Each particle uses its
@@ -1165,8 +1176,9 @@ __global__ void __launch_bounds__(256) k_predict(const Dev d, const IntegrateArg
             const uint32_t id = a.id[k];
             const uint32_t q = find_instance(d.id_base, d.n_inst, id);
             const Inst& I = d.inst[q];
-            const float hdt = (float)(0.5 * d.is.dt[q]);
-            const float4 ac = a.ace[k];
+            const double dt = d.is.dt[q];
+            const float hdt = (float)(0.5 * dt);
+            const float4 ac = rates(d, a, k, q, dt);
             if (id >= I.id_fluid) {
                 x += (double)(hdt * vr.x);
                 y += (double)(hdt * vr.y);
@@ -1209,7 +1221,7 @@ __global__ void __launch_bounds__(256) k_correct(const Dev d, const IntegrateArg
             const float dtf = (float)dt;
             const float hdt = (float)(0.5 * dt);
             double x = a.x[k], y = a.y[k], z = a.z[k];
-            const float4 ac = a.ace[k];
+            const float4 ac = rates(d, a, k, q, dt);
             const float4 pv = a.pvr[k];
             float4 vr = a.velrhop[k];
             if (id >= I.id_fluid) {
