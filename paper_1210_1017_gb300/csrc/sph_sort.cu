@@ -234,11 +234,10 @@ __global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
     }
 }
 
-// All digit places of an input of at most one tile, by one block.
-__global__ void __launch_bounds__(kOsThreads) k_sort_tile(const uint32_t* __restrict__ kin,
-                                                          const uint32_t* __restrict__ vin,
-                                                          uint32_t* __restrict__ kout,
-                                                          uint32_t* __restrict__ vout, uint32_t n,
+// All digit places of an input of at most one tile, by one block.  The outputs
+// may be the inputs (the selection sorts in place): no __restrict__.
+__global__ void __launch_bounds__(kOsThreads) k_sort_tile(const uint32_t* kin, const uint32_t* vin,
+                                                          uint32_t* kout, uint32_t* vout, uint32_t n,
                                                           int bits_total) {
     constexpr int W = kOsThreads / 32;
     __shared__ uint32_t s_wh[W][256];

@@ -53,3 +53,24 @@ def test_every_selected_particle_comes_out_once(pairs):
             assert np.array_equal(a, b)
     sim.check()
     sim.close()
+
+
+@pytest.mark.parametrize("n", [40, 1200, 4000])
+def test_few_ids_above_n_are_sorted_in_place(n):
+    """A selection of at most one tile of pairs, by the sort (ids up to 2^32 - 1)."""
+    case = cases.random_block(n, seed=24, jitter=0.4)
+    case.n_bound = 0
+    case.ids = (np.uint32(0xffffffff) - np.random.default_rng(1).permutation(
+        4 * case.n)[:case.n].astype(np.uint32) * np.uint32(1001))
+    x = case.pos[:, 0]
+    lo, hi = float(np.quantile(x, 0.4)), float(np.quantile(x, 0.6))
+    lab = np.where(x < lo, 1, np.where(x >= hi, 2, 0))
+    sim = S.Simulation.from_case(case)
+    sim.build_cells()
+    got = sim.subdomain_select(S.SPH_SUBDOMAIN_MIGRATE, lo, hi)
+    sel = np.nonzero(lab)[0]
+    sel = sel[np.lexsort((case.ids[sel], lab[sel]))]
+    assert np.array_equal(got["ids"], case.ids[sel])
+    for key in ("pos", "vel", "rho"):
+        assert np.array_equal(got[key], getattr(case, key)[sel]), key
+    sim.close()
