@@ -545,6 +545,8 @@ int init(const sph_params* params, const sph_instance* inst, uint32_t n_inst, vo
             return SPH_ERR_CUDA;
         }
     }
+    const double cell = 2.0 * params->h;
+    c->variant = default_variant(cell * cell * cell * params->rho0 / params->mass);
     c->nparts = interact_grid(c->variant);
     c->d = make_dev(c);
     cudaStream_t st = c->st;

@@ -234,6 +234,7 @@ struct Variant {
 // The shapes whose candidate test runs on the tensor cores (sph_interact_tc.cu).
 Variant tc_variant_n(int k);
 uint32_t max_units(uint32_t n, uint32_t nrows, uint64_t ncells);   // bound on units
+int default_variant(double per_cell);        // variant at this many particles per cell
 int variant_unit(int variant);               // particles per unit of a variant
 int variant_stage(int variant);              // staged candidates of a variant
 uint32_t interact_grid(int variant);         // blocks of its persistent launch

@@ -1560,6 +1560,17 @@ int variant_unit(int v) { return g_variants[v].warps * 32; }
 int variant_stage(int v) { return g_variants[v].stage; }
 
 // Persistent grid: every resident block of the variant on this GPU.
+// Variant of a context that has not been tuned.  A unit's candidates are its
+// cells' neighbour rows, so beyond some 33 particles per cell (h/dp 1.6) shape 0
+// stages fewer particles at a time, and from 64 on none, where the half-precision
+// shape 13 with its 2,048 slots still does.  ms per launch on one GB300, 0 / 13:
+//   h/dp (per cell)   1.5 (27)     1.6 (33)     1.7 (39)     2.0 (64)     2.1 (74)
+//   20k particles     0.033/0.033  0.045/0.043  0.057/0.048  0.117/0.069  0.160/0.123
+//   200k              0.160/0.187  0.211/0.223  0.291/0.266  0.549/0.485  0.992/0.669
+//   1M                0.708/0.828  0.985/1.022  1.423/1.260  2.736/2.557  5.256/3.291
+// and above, 2.2 to 3.0, 13 takes 0.92 to 0.99 of 0's time at 200k and 1M.
+int default_variant(double per_cell) { return per_cell > 33.0 ? 13 : 0; }
+
 uint32_t interact_grid(int v) { return (uint32_t)g_variants[v].grid; }
 
 namespace {
