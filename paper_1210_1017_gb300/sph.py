@@ -560,11 +560,15 @@ def _cache_path():
 
 
 def autotune_cached(sim, reps=3):
-    """Autotune once per (GPU, size bucket, member count) and reuse the choice."""
+    """Autotune once per (GPU, size bucket, member count, particles per cell) and
+    reuse the choice.  The last in steps of 2^(1/4): a shape that is the fastest at
+    h/dp 1.3 (18 per cell) takes up to twice as long as the best one at 2.1 (74)."""
     import json
     import math
     name = sim.torch.cuda.get_device_name(sim.device)
-    key = f"{name}|{KERNEL_REV}|n2^{int(math.log2(max(sim.n, 1)))}|m{sim.n_inst}"
+    per_cell = (2.0 * sim.P.h) ** 3 * sim.P.rho0 / sim.P.mass
+    key = (f"{name}|{KERNEL_REV}|n2^{int(math.log2(max(sim.n, 1)))}|m{sim.n_inst}"
+           f"|c2^{round(4 * math.log2(per_cell)) / 4}")
     path = _cache_path()
     table = {}
     try:
@@ -666,7 +670,8 @@ class Simulation:
     def autotune(self, reps=3, cache=True):
         """Pick the fastest interaction variant for this GPU and size (needs
         built cells).  With cache=True the choice is kept in the user cache
-        directory per (GPU name, log2 particle count, member count)."""
+        directory per (GPU name, log2 particle count, member count, log2
+        particles per cell)."""
         return autotune_cached(self, reps) if cache else sph_autotune(self.ctx, reps)
 
     def set_variant(self, v):
