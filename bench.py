@@ -382,7 +382,8 @@ def run_ours(args):
             traffic = tr.get("bytes_per_launch", {}).get(args.workload)
     roofline = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak_tflops, 2),
                 "unit": "TFLOP/s", "frac": round(achieved / peak_tflops, 4), "traffic": traffic,
-                "kernel": "k_interact", "ms_per_launch": round(t_int * 1e3, 4),
+                "kernel": "k_interact_tc" if variant < 7 else "k_interact",   # (sph_interact_tc.cu)
+                "ms_per_launch": round(t_int * 1e3, 4),
                 "peak_source": ("measured: sph_fma_probe, 8 independent FMA chains per thread, "
                                 "SMs x 8 blocks x 256 threads, best of 10 launches (CUDA events)"),
                 "peak_median": round(peak_median, 2),
@@ -671,7 +672,7 @@ def subdomain_timing(sim, case, nsub, S, torch):
         ms.append(round((time.perf_counter() - t) / reps * 1e3, 3))
         sel.append(int(c[1]) + int(c[2]))
     return {"slabs": nsub, "mode": "edge", "ms_per_call": ms, "selected": sel,
-            "note": "labels of all particles, (label, id) radix sort of the selected, copy "
+            "note": "labels of all particles, (label, id) order of the selected, copy "
                     "into device buffers; wall time per synchronous call"}
 
 

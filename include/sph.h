@@ -435,8 +435,9 @@ int sph_units_selftest_timeout(sph_ctx *ctx, uint32_t polls);
 /* Block shapes of the interaction kernel ("variants": particles per work
  * unit, staged candidates per unit, neighbour-list slots per lane) and the
  * autotuner that picks one.  Results do not depend on the variant beyond
- * FP32 summation order within a particle's own sum, which is the same for
- * every variant (each particle sums its neighbours in the sorted order).
+ * FP32 rounding within a particle's own sum (the order of its terms, and x
+ * differences in fixed point for variants 0 to 6).  A context that was not
+ * tuned takes variant 0, or 13 above 33 particles per cell (h/dp 1.6).
  * sph_autotune times `reps` interaction launches of every variant on the
  * current cells (CUDA events on the context's stream), selects the fastest
  * and writes the per-variant milliseconds to ms_per_variant (NULL allowed,

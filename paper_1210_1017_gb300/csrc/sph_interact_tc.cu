@@ -223,7 +223,6 @@ struct TcShape {
                                       ? (int)(2 * stage_bytes / ((size_t)W * SPLIT * 32 * 4))
                                       : 64;
     static_assert(fb_cap >= 16, "fallback lists must fit in the staging area");
-    static_assert((size_t)(STAGE + 1) * 16 <= 65536, "list entries hold byte offsets in 16 bits");
     static_assert(PIECE % (8 * SPLIT) == 0 && PIECE % 32 == 0, "a piece's columns and rows");
 };
 
@@ -924,8 +923,12 @@ Variant tc_variant() {
 // times them all; ms per launch on one GB300, 128 / 64: 35.4M particles 18.4 /
 // 24.2, 1.39M 0.701 / 0.865, 60k 0.072 / 0.077, 256 dam breaks 3.20 / 3.15, 17k
 // 0.0212 / 0.0196).  Between the first and the third, fourth and seventh,
-// shared memory moves from staged candidates to hit words (larger h/dp has more
-// hits per particle): 1,664 / 18 take 18.4 / 0.709 ms.
+// shared memory moves from staged candidates to hit words, for larger h/dp (more
+// hits per particle); 200k particles, variants 0 / 2 / 3 / 6: h/dp 1.3 0.118 / 0.118 /
+// 0.119 / 0.126, 1.5 0.161 / 0.146 / 0.142 / 0.157, 1.7 0.291 / 0.253 / 0.218 / 0.250,
+// 1.8 0.363 / 0.371 / 0.345 / 0.318 (beyond 1.8 the shapes with 2,048 slots, 0.325 and
+// less).  Variant 5 is for a spray: 300k particles at random, one in three cells
+// 0.90 ms (variant 0 1.69, variant 1 1.12), one per cell 0.198 (0.347, 0.242).
 Variant tc_variant_n(int k) {
     switch (k) {
         case 0: return tc_variant<4, 2, 1760, 16, 256, 2>();

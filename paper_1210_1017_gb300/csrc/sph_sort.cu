@@ -7,11 +7,11 @@
 // digit, and a scatter in which each tile ranks its keys in shared memory and
 // moves them to their digit's run.  Up to kFewTiles tiles the scatter adds up
 // the counts itself (no scan launch), and an input of one tile is sorted by one
-// block in one launch, all places in shared memory.  The tiles are independent: a one-pass organisation, whose tiles
-// wait for the offsets of the tiles before them, spent most of its time and
-// half of its instructions in those waits and in __match_any_sync (one GB300:
-// 4.0M pairs with 24-bit keys 192 us, 30M with 32-bit keys 1,223 us, 1,000
-// pairs 51 us; now 113, 779 and 12.5).
+// block in one launch, all places in shared memory.  The tiles are independent:
+// a one-pass organisation, whose tiles wait for the offsets of the tiles before
+// them, spent most of its time and half of its instructions in those waits and
+// in __match_any_sync (one GB300: 4.0M pairs with 24-bit keys 197 us, 30M with
+// 32-bit keys 1,223 us, 1,000 pairs 51 us; these kernels 116, 779 and 12.5).
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -19,6 +19,11 @@ namespace sph {
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
+// Where the scan's launch costs more than every block adding up all counts: us
+// per sort of 24-bit keys without / with it, calls one after another, 32 tiles 44.7 /
+// 59.1, 64 50.7 / 57.5, 80 55.6 / 55.5, 96 57.5 / 59.7, 112 63.8 / 58.9, 160 77.8 /
+// 67.9.  (On the device alone, in a graph, the line lies lower: 32 36.0 / 38.9, 48
+// 40.4 / 38.7, 96 49.2 / 39.4.)
 constexpr uint32_t kFewTiles = 96;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {

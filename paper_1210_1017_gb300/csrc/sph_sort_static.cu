@@ -7,8 +7,8 @@
 // a latency-critical loop that must not call cudaMalloc/cudaFree at run time
 // because those calls can synchronise the whole device and stall work on
 // other streams.  Such callers still own the input and output arrays; only the
-// sort's own scratch (temporary keys/values, tile counts and digit totals) moves into a fixed array that is part of the
-// loaded library.
+// sort's own scratch (temporary keys/values, tile counts and digit totals) moves
+// into a fixed array that is part of the loaded library.
 //
 // The array below is a host-side stand-in when named from host code; the
 // device address is looked up with cudaGetSymbolAddress once per device, on

@@ -311,7 +311,7 @@ __global__ void k_rowsum(uint32_t n, const uint32_t* __restrict__ rowptr, const 
 // its threads in a fixed order and writes one partial; k_colsum_final adds
 // the partials in a fixed order.  (One column per thread read 2 or 4 bytes a
 // lane: 200 us for 1.27M x 128, a quarter to a half of the copy bandwidth.)
-constexpr uint32_t kColParts = 4 * 152;   // blocks: four per SM
+constexpr uint32_t kColParts = 4 * 152;   // blocks: four on each of the chip's SMs
 constexpr uint32_t kColRegion = 1024;      // partials that a region of the scratch holds
 
 template <int V>

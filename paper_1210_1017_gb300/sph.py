@@ -525,8 +525,8 @@ def sph_radix_sort_pairs(keys_in, vals_in, keys_out, vals_out, n, key_bits, scra
 
 
 def sph_radix_sort_status(scratch, scratch_bytes, n, stream):
-    """Raises SphError (SPH_ERR_TIMEOUT) if the last sort on this scratch
-    gave up a look-back wait."""
+    """Raises SphError (SPH_ERR_TIMEOUT) if a bounded device wait on this scratch
+    gave up since the last sort: the self-test's (the sort itself has none)."""
     _check(lib().sph_radix_sort_status(_ptr(scratch), scratch_bytes, n, stream),
            what="sph_radix_sort_status")
 
