@@ -1145,11 +1145,15 @@ __global__ void __launch_bounds__(kFusedWarps * 32) k_units_fused(const Dev d,
 // instance has ended: they are no longer evaluated then, and a.ace holds what
 // was there (another run's, another particle's), which dt = 0 does not cancel
 // when it is not finite.  (done itself is being set by k_correct; a running
-// instance of infinite rates has dt = 0 as well, but not the time.)
+// instance of infinite rates has dt = 0 as well, but not the time.)  The test of
+// dt is of its bits: one FP64 comparison per particle made both integrators 6%
+// slower (1.19 / 1.22 ms at 35.4M particles).
 __device__ __forceinline__ float4 rates(const Dev& d, const IntegrateArgs& a, uint32_t k, uint32_t q,
                                         double dt) {
-    if (dt == 0.0 && d.is.t[q] >= d.inst[q].t_end) return make_float4(0.f, 0.f, 0.f, 0.f);
-    return a.ace[k];
+    float4 ac = a.ace[k];
+    if (__double_as_longlong(dt) == 0 && d.is.t[q] >= d.inst[q].t_end)
+        ac = make_float4(0.f, 0.f, 0.f, 0.f);
+    return ac;
 }
 
 // Symplectic predictor (half step) for sorted particle k, then its new
