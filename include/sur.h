@@ -7,7 +7,9 @@
  * accumulation, forward and backward.
  *
  * Conventions as in sph.h: SPH_OK / SPH_ERR_* return codes, caller-owned
- * device memory, async on the given stream unless marked "sync".
+ * device memory, async on the given stream unless marked "sync".  The device
+ * waits of the passes on an sph_ctx are bounded; one that gave up sets
+ * SPH_STATUS_TIMEOUT in that context (sph_check).
  */
 #ifndef SUR_H
 #define SUR_H

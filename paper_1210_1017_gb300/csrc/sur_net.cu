@@ -609,6 +609,9 @@ struct sur_ctx {
     // graph
     uint32_t *cnt, *rowptr, *bsum, *col, *src, *rev;
     uint32_t n = 0, E = 0;
+    // status word of the SPH context in hand (set by every pass): where a kernel
+    // reports a bounded wait that gave up
+    uint32_t* status = nullptr;
     // activations (train: one per layer; inference: ping-pong)
     __nv_bfloat16 *xn, *xe, *en1, *ee1;
     std::vector<__nv_bfloat16*> XN, Ebuf, Z1, Y1;
@@ -725,6 +728,7 @@ int linear(sur_ctx* c, const __nv_bfloat16* A, uint32_t lda, const Layer& l, boo
            uint32_t M, int epi, const __nv_bfloat16* res, uint32_t ldr, __nv_bfloat16* out_bf,
            float* out_f, uint32_t ldo, bool with_bias = true) {
     LinearArgs g = {};
+    g.status = c->status;
     g.A = A;
     g.lda = lda;
     // forward: out = A W (+ b) uses W^T as the K-major operand; backward:
@@ -748,6 +752,7 @@ int linear(sur_ctx* c, const __nv_bfloat16* A, uint32_t lda, const Layer& l, boo
 int edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* e,
                __nv_bfloat16* z, __nv_bfloat16* e_out) {
     EdgeArgs g = {};
+    g.status = c->status;
     g.E = e;
     g.W1t = l1.Wt;
     g.W2t = l2.Wt;
@@ -770,6 +775,7 @@ int edge_layer(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16
 int node_update(sur_ctx* c, const Layer* w, const Layer* next, const __nv_bfloat16* xn,
                 __nv_bfloat16* y, __nv_bfloat16* xn_next) {
     NodeArgs g = {};
+    g.status = c->status;
     g.X = xn;
     g.W3t = w[4].Wt;
     g.W4t = w[5].Wt;
@@ -792,6 +798,7 @@ int node_update(sur_ctx* c, const Layer* w, const Layer* next, const __nv_bfloat
 // (the hidden activation kept for the backward pass when z != null).
 int edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z, __nv_bfloat16* e0) {
     EdgeArgs g = {};
+    g.status = c->status;
     g.E = c->xe;
     g.W1t = l1.Wt;
     g.W2t = l2.Wt;
@@ -809,6 +816,7 @@ int edge_encoder(sur_ctx* c, const Layer& l1, const Layer& l2, __nv_bfloat16* z,
 int wgrad(sur_ctx* c, const Layer& l, const __nv_bfloat16* X, uint32_t ldx,
            const __nv_bfloat16* dY, uint32_t ldy, uint32_t M) {
     WgradArgs g = {};
+    g.status = c->status;
     g.M = M;
     g.partial = c->partial;
     g.nparts = kWgradParts;
@@ -851,6 +859,7 @@ int wgrads(sur_ctx* c, uint32_t M, std::initializer_list<Wgrad> list) {
         g[k].dY = w.dY;
         g[k].ldq = L;
         g[k].M = M;
+        g[k].status = c->status;
         g[k].partial = c->partial;
         g[k].nparts = kWgradParts;
         g[k].scale = 1.f;
@@ -910,6 +919,7 @@ ColSum rows_f32(sur_ctx* c, int region, const float* acc, uint32_t M, __nv_bfloa
 // pending in regions 2 and 3, are the gradients of b2 and b1.
 int edge_backward(sur_ctx* c, const Layer& l1, const Layer& l2, const __nv_bfloat16* z, uint32_t* parts) {
     EdgeBwdArgs g = {};
+    g.status = c->status;
     g.dE = c->dE;
     g.node = c->dXN + L;
     g.ldn = 2 * L;
@@ -956,6 +966,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
     if (s->n > c->cfg.max_nodes) return fail(c, SPH_ERR_INVALID_ARG, "more particles than max_nodes");
     const uint32_t n = s->n;
     c->n = n;
+    c->status = s->status;
     cudaStream_t st = c->st;
     const sph::Dev& d = s->d;
     const int cur = s->cur;
@@ -1023,6 +1034,7 @@ int forward(sur_ctx* c, sph_ctx* s, const float* hist) {
 int backward(sur_ctx* c, sph_ctx* s, const float* target, float* loss_host) {
     if (!c->cfg.train) return fail(c, SPH_ERR_STATE, "context not created for training");
     if (!c->have_forward) return fail(c, SPH_ERR_STATE, "no forward pass to differentiate");
+    c->status = s->status;
     cudaStream_t st = c->st;
     const uint32_t n = c->n, E = c->E;
     const std::vector<Layer>& Ls = c->layers;
