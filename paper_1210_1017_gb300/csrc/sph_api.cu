@@ -1419,8 +1419,7 @@ int sph_radix_sort_pairs(const uint32_t* kin, const uint32_t* vin, uint32_t* kou
     uint32_t* tv = cv.take<uint32_t>(n);
     uint32_t* words = cv.take<uint32_t>(radix_sort_words(n));
     uint32_t* err = cv.take<uint32_t>(1);
-    cudaMemsetAsync(err, 0, sizeof(uint32_t), st);
-    launch_radix_sort(kin, vin, kout, vout, tk, tv, n, (int)key_bits, words, st);
+    launch_radix_sort(kin, vin, kout, vout, tk, tv, n, (int)key_bits, words, err, st);
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 

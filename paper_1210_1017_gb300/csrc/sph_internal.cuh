@@ -148,12 +148,13 @@ inline uint32_t os_tiles(uint32_t n) { return (n + kOsTile - 1) / kOsTile; }
 void launch_lookback_selftest(uint32_t* zeroed, uint32_t limit, uint32_t* err, cudaStream_t st);
 // Stable sort of n pairs by the low key_bits bits of the key (vin null: the
 // values are the input indexes).  tk, tv: n temporaries (used by more than
-// one digit place); words: radix_sort_words(n) words without initial contents.
+// one digit place); words: radix_sort_words(n) words without initial contents;
+// clear: a word that the sort sets to 0 (null: none).
 // Its kernels do not wait on one another.
 size_t radix_sort_words(uint32_t n);
 void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
                        uint32_t* tk, uint32_t* tv, uint32_t n, int key_bits, uint32_t* words,
-                       cudaStream_t st);
+                       uint32_t* clear, cudaStream_t st);
 
 // Blocks of the sub-domain selection's pass over the bit maps of n ids.
 constexpr uint32_t kBitWords = 2048;   // 32-bit words per block

@@ -12,6 +12,9 @@
 // them, spent most of its time and half of its instructions in those waits and
 // in __match_any_sync (one GB300: 4.0M pairs with 24-bit keys 197 us, 30M with
 // 32-bit keys 1,223 us, 1,000 pairs 51 us; these kernels 116, 779 and 12.5).
+// (__match_any_sync steps through the distinct digits of a warp, so that one was
+// at its best on keys with hardly any: 300k equal 32-bit keys 42.9 us on the
+// device, 38.0 here.)
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -20,11 +23,12 @@ namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
 // Where the scan's launch costs more than every block adding up all counts: us
-// per sort of 24-bit keys without / with it, calls one after another, 32 tiles 44.7 /
-// 59.1, 64 50.7 / 57.5, 80 55.6 / 55.5, 96 57.5 / 59.7, 112 63.8 / 58.9, 160 77.8 /
-// 67.9.  (On the device alone, in a graph, the line lies lower: 32 36.0 / 38.9, 48
-// 40.4 / 38.7, 96 49.2 / 39.4.)
-constexpr uint32_t kFewTiles = 96;
+// per sort of random 24-bit keys without / with it, calls one after another (bound
+// by the launches) and on the device alone (a graph):
+//   tiles           49           96           128          160
+//   calls           43.2 / 51.8  47.3 / 53.4  51.4 / 57.5  62.6 / 66.5
+//   device          31.6 / 33.6  33.8 / 33.3  38.8 / 35.6  49.4 / 44.5
+constexpr uint32_t kFewTiles = 128;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
@@ -92,13 +96,15 @@ __host__ __device__ __forceinline__ uint32_t digit_mask(int pass, int bits_total
 }
 
 // Digit counts of each tile: cnt[tile * 256 + d] for few tiles, else in the
-// scan's order, cnt[d * tiles + tile].  Two copies in shared memory (even and
+// scan's order, cnt[d * tiles + tile]; *clear (may be null) becomes 0.  Two copies in shared memory (even and
 // odd warps), four keys per load where the input is 16-byte aligned.
 __global__ void __launch_bounds__(kOsThreads) k_tile_counts(const uint32_t* __restrict__ keys,
                                                             uint32_t n, int shift, uint32_t dmask,
                                                             uint32_t tiles,
-                                                            uint32_t* __restrict__ cnt) {
+                                                            uint32_t* __restrict__ cnt,
+                                                            uint32_t* clear) {
     __shared__ uint32_t sh[2][256];
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0u;
     sh[0][threadIdx.x] = 0u;
     sh[1][threadIdx.x] = 0u;
     __syncthreads();
@@ -187,10 +193,15 @@ __global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
     // the global first slot of digit tid in this tile
     uint32_t before = 0, total = 0;
     if (tiles <= kFewTiles) {
-        for (uint32_t t = 0; t < tiles; ++t) {
-            const uint32_t c = __ldg(tab + t * 256u + tid);
-            before += t < tile ? c : 0u;
-            total += c;
+        for (uint32_t t0 = 0; t0 < tiles; t0 += 16) {   // 16 loads in flight
+            uint32_t c[16];
+#pragma unroll
+            for (uint32_t j = 0; j < 16; ++j) c[j] = t0 + j < tiles ? __ldg(tab + (t0 + j) * 256u + tid) : 0u;
+#pragma unroll
+            for (uint32_t j = 0; j < 16; ++j) {
+                before += t0 + j < tile ? c[j] : 0u;
+                total += c[j];
+            }
         }
     } else {
         before = __ldg(tab + (size_t)tid * tiles + tile);
@@ -243,7 +254,8 @@ __global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
 // may be the inputs (the selection sorts in place): no __restrict__.
 __global__ void __launch_bounds__(kOsThreads) k_sort_tile(const uint32_t* kin, const uint32_t* vin,
                                                           uint32_t* kout, uint32_t* vout, uint32_t n,
-                                                          int bits_total) {
+                                                          int bits_total, uint32_t* clear) {
+    if (clear && threadIdx.x == 0) *clear = 0u;
     constexpr int W = kOsThreads / 32;
     __shared__ uint32_t s_wh[W][256];
     __shared__ uint32_t s_w[8];
@@ -545,11 +557,11 @@ size_t radix_sort_words(uint32_t n) {
 
 void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
                        uint32_t* tk, uint32_t* tv, uint32_t n, int key_bits, uint32_t* words,
-                       cudaStream_t st) {
+                       uint32_t* clear, cudaStream_t st) {
     const uint32_t tiles = os_tiles(n);
     if (tiles == 0) return;
     if (tiles == 1) {
-        k_sort_tile<<<1, kOsThreads, 0, st>>>(kin, vin, kout, vout, n, key_bits);
+        k_sort_tile<<<1, kOsThreads, 0, st>>>(kin, vin, kout, vout, n, key_bits, clear);
         return;
     }
     uint32_t* cnt = words;
@@ -563,7 +575,8 @@ void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
         uint32_t* ok = to_out ? kout : tk;
         uint32_t* ov = to_out ? vout : tv;
         const uint32_t dm = digit_mask(p, key_bits);
-        k_tile_counts<<<tiles, kOsThreads, 0, st>>>(ck, n, 8 * p, dm, tiles, cnt);
+        k_tile_counts<<<tiles, kOsThreads, 0, st>>>(ck, n, 8 * p, dm, tiles, cnt,
+                                                      p == 0 ? clear : nullptr);
         if (tiles > kFewTiles) k_digit_scan<<<256, kOsThreads, 0, st>>>(cnt, tiles, tot);
         k_radix_scatter<<<tiles, kOsThreads, 0, st>>>(ck, cv, ok, ov, n, 8 * p, dm, tiles, cnt, tot);
         ck = ok;

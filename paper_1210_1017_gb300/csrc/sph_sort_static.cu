@@ -16,8 +16,7 @@
 // makes a CUDA runtime query and should come before any stream capture.  All
 // calls on one device share the array: calls that overlap on the GPU (two
 // streams, two threads) race on it and must be serialised by the caller.
-// Nothing here allocates: the zeroing is done with cudaMemsetAsync on the
-// fixed array.
+// Nothing here allocates; the sort's first kernel clears the array's error word.
 #include <mutex>
 
 #include "../../include/sph.h"
@@ -72,9 +71,8 @@ extern "C" int sph_radix_sort_pairs_static(const uint32_t* d_keys_in, const uint
     if (rc != SPH_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (radix_sort_words(n) > kErr - kSort) return SPH_ERR_TOO_LARGE;   // not for n <= kMaxN
-    cudaMemsetAsync(s + kErr, 0, sizeof(uint32_t), st);
     launch_radix_sort(d_keys_in, d_vals_in, d_keys_out, d_vals_out, s + kTmpKeys, s + kTmpVals, n,
-                      (int)key_bits, s + kSort, st);
+                      (int)key_bits, s + kSort, s + kErr, st);
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 

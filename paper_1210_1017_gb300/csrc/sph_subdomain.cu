@@ -296,10 +296,10 @@ extern "C" int sph_subdomain_select(sph_ctx* c, int mode, double xlo, double xhi
     } else {
         // sort A: by id (four places, in place); sort B: stable by label
         launch_radix_sort(c->sub_key[0], c->sub_val[0], c->sub_key[0], c->sub_val[0], c->sub_key[1],
-                          c->sub_val[1], m, 32, c->sub_os, st);
+                          c->sub_val[1], m, 32, c->sub_os, nullptr, st);
         k_sub_relabel<<<blocks256(m), 256, 0, st>>>(c->sub_val[0], m, c->sub_key[1], c->sub_val[1]);
         launch_radix_sort(c->sub_key[1], c->sub_val[1], c->sub_key[0], c->sub_val[0], nullptr,
-                          nullptr, m, 2, c->sub_os, st);
+                          nullptr, m, 2, c->sub_os, nullptr, st);
         sidx = c->sub_val[0];
     }
     // gather straight into destinations on this device, else into the
