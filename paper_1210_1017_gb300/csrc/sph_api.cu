@@ -235,7 +235,7 @@ size_t carve(sph_ctx* c, void* base, uint32_t n, const Table& t, int passes) {
         c->sub_val[b] = cv.take<uint32_t>(n);
     }
     c->sub_os = cv.take<uint32_t>(radix_sort_words(n));
-    c->sub_cnt = cv.take<uint32_t>(8);
+    c->sub_cnt = cv.take<uint32_t>(8);   // and the maps behind it (one memset clears both)
     c->sub_bits = cv.take<uint32_t>(2 * (((size_t)n + 31) / 32));
     c->sub_bsum = cv.take<uint32_t>(sub_bit_blocks(n));
     c->csum = cv.take<uint32_t>(t.ncells + t.nrows + 1);

@@ -64,6 +64,7 @@ struct sph_ctx {
     // and the words of their radix sorts (other ids)
     uint32_t *sub_key[2], *sub_val[2];
     uint32_t *sub_os, *sub_cnt, *sub_bits, *sub_bsum;
+    bool sub_clear = false;  // the bit maps are all 0
     double *diag_out, *diag_part;
     unsigned long long* front;   // per-member front images (sph_front)
     unsigned long long* counters;

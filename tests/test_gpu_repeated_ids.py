@@ -74,3 +74,43 @@ def test_few_ids_above_n_are_sorted_in_place(n):
     for key in ("pos", "vel", "rho"):
         assert np.array_equal(got[key], getattr(case, key)[sel]), key
     sim.close()
+
+
+def test_calls_in_turn_leave_nothing_behind():
+    """Empty, full, refused and repeated-id selections in turn on one context: each
+    as on a context of its own (the bit maps are cleared by the call that used them)."""
+    case = cases.random_block(5000, seed=25, jitter=0.4)
+    case.n_bound = 0
+    x = case.pos[:, 0]
+    lo, hi = float(np.quantile(x, 0.3)), float(np.quantile(x, 0.6))
+    one = np.nonzero(x < lo)[0]
+    ids = case.ids.copy()
+    twice = case.ids.copy()
+    twice[one[:3]] = twice[one[3:6]]
+    wide = (float(x.min()) - 1.0, float(x.max()) + 1.0)
+    sim = S.Simulation(case.params(), case.n)
+
+    def call(of, bounds):
+        alone = S.Simulation(case.params(), case.n)
+        got = []
+        for s in (sim, alone):
+            s.upload(case.pos, case.vel, case.rho, of)
+            s.build_cells()
+            got.append(s.subdomain_select(S.SPH_SUBDOMAIN_MIGRATE, *bounds))
+        alone.close()
+        assert got[0]["counts"].tolist() == got[1]["counts"].tolist()
+        assert np.array_equal(got[0]["ids"], got[1]["ids"])
+        if of is ids:
+            for key in ("pos", "vel", "rho"):
+                assert np.array_equal(got[0][key], got[1][key]), key
+        return got[0]["ids"].size
+
+    small = np.empty(1, np.uint32)
+    for of, bounds in ((ids, wide), (ids, (lo, hi)), (ids, wide), (twice, (lo, hi)), (ids, (hi, hi + 1.0)),
+                       (ids, (lo, hi)), (twice, wide), (ids, (lo, hi))):
+        m = call(of, bounds)
+        assert (m == 0) == (bounds is wide)
+        if m:
+            with pytest.raises(S.SphError, match="SPH_ERR_CAPACITY"):
+                S.sph_subdomain_select(sim.ctx, S.SPH_SUBDOMAIN_MIGRATE, *bounds, 1, None, None, None, small)
+    sim.close()
