@@ -11,7 +11,7 @@
 // a one-pass organisation, whose tiles wait for the offsets of the tiles before
 // them, spent most of its time and half of its instructions in those waits and
 // in __match_any_sync (one GB300: 4.0M pairs with 24-bit keys 197 us, 30M with
-// 32-bit keys 1,223 us, 1,000 pairs 51 us; these kernels 116, 779 and 12.5).
+// 32-bit keys 1,223 us, 1,000 pairs 51 us; these kernels 115, 761 and 10.4).
 // (__match_any_sync steps through the distinct digits of a warp, so that one was
 // at its best on keys with hardly any: 300k equal 32-bit keys 42.9 us on the
 // device, 38.0 here.)
@@ -164,10 +164,13 @@ __global__ void __launch_bounds__(kOsThreads) k_digit_scan(uint32_t* __restrict_
     if (threadIdx.x == 0) tot[blockIdx.x] = s_carry;
 }
 
-// The scatter of one digit place.  tab: the tiles' counts (few tiles) or
-// their scans per digit, tot the digits' totals.  Keys of a tile are ranked per warp (rounds of 32 in
-// input order), moved to the tile's sorted order in shared memory and written
-// from there in runs.
+// The scatter of one digit place.  tab: the tiles' counts (FEW tiles) or
+// their scans per digit, tot the digits' totals.  Keys of a tile are ranked per
+// warp (rounds of 32 in input order), moved to the tile's sorted order in shared
+// memory and written from there in runs.
+// (FEW as a run-time branch cost the other form 4%: 20M pairs, 24-bit keys, 382 us on
+// the device against 397.)
+template <bool FEW>
 __global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
     uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, uint32_t n, int shift,
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(kOsThreads, 4) k_radix_scatter(
     }
     // the global first slot of digit tid in this tile
     uint32_t before = 0, total = 0;
-    if (tiles <= kFewTiles) {
+    if (FEW) {
         for (uint32_t t0 = 0; t0 < tiles; t0 += 16) {   // 16 loads in flight
             uint32_t c[16];
 #pragma unroll
@@ -577,8 +580,14 @@ void launch_radix_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
         const uint32_t dm = digit_mask(p, key_bits);
         k_tile_counts<<<tiles, kOsThreads, 0, st>>>(ck, n, 8 * p, dm, tiles, cnt,
                                                       p == 0 ? clear : nullptr);
-        if (tiles > kFewTiles) k_digit_scan<<<256, kOsThreads, 0, st>>>(cnt, tiles, tot);
-        k_radix_scatter<<<tiles, kOsThreads, 0, st>>>(ck, cv, ok, ov, n, 8 * p, dm, tiles, cnt, tot);
+        if (tiles <= kFewTiles) {
+            k_radix_scatter<true><<<tiles, kOsThreads, 0, st>>>(ck, cv, ok, ov, n, 8 * p, dm, tiles,
+                                                                cnt, tot);
+        } else {
+            k_digit_scan<<<256, kOsThreads, 0, st>>>(cnt, tiles, tot);
+            k_radix_scatter<false><<<tiles, kOsThreads, 0, st>>>(ck, cv, ok, ov, n, 8 * p, dm, tiles,
+                                                                 cnt, tot);
+        }
         ck = ok;
         cv = ov;
     }
