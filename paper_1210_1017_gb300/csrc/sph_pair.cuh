@@ -260,7 +260,9 @@ __device__ __forceinline__ void pair_terms2(const Dev& d, float c0, const float4
         const float2 wq = __ffma2_rn(dup2(-0.5f), q, dup2(1.0f));
         shape = __fmul2_rn(__fmul2_rn(wq, wq), wq);
     }
-    const float2 F = __fmul2_rn(__fmul2_rn(dup2(d.fc), shape), use);
+    // (the mask before the shape: exact, and fc, 1e35 at h = 0.1 um, does not
+    // overflow on the shape of a pad 32 cells away)
+    const float2 F = __fmul2_rn(__fmul2_rn(dup2(d.fc), use), shape);
     const float2 m1 = dup2(-1.0f);
     const float2 dvx = __ffma2_rn(ff2(va.x, vb.x), m1, dup2(vi.x));
     const float2 dvy = __ffma2_rn(ff2(va.y, vb.y), m1, dup2(vi.y));
