@@ -562,6 +562,9 @@ int init(const sph_params* params, const sph_instance* inst, uint32_t n_inst, vo
     cudaMemsetAsync(c->i_t, 0, n_inst * sizeof(double), st);
     cudaMemsetAsync(c->i_done, 0, n_inst * sizeof(uint32_t), st);
     cudaMemsetAsync(c->i_steps, 0, n_inst * sizeof(unsigned long long), st);
+    // a predictor step before the first evaluation takes these rates: 0, whatever
+    // the workspace held
+    cudaMemsetAsync(c->ace, 0, (size_t)c->n * sizeof(float4), st);
     cudaMemsetAsync(c->i_terms, 0, 3 * (size_t)n_inst * sizeof(uint32_t), st);
     cudaMemsetAsync(c->i_last, 0, 3 * (size_t)n_inst * sizeof(float), st);
     cudaMemsetAsync(c->i_vphase, 0, n_inst * sizeof(uint32_t), st);

@@ -59,9 +59,9 @@ struct sph_ctx {
     uint32_t *done, *status;
     uint32_t* id_flag;       // set by the upload when some id >= n
     // sub-domain selection (Sec. 4.3): counters; bit maps of the selected ids
-    // per label and their block sums (dense ids; sub_val[0] and
-    // sub_key[0] then map ids to state indexes); ping-pong (key, value) arrays of the selected particles
-    // and the words of their radix sorts (other ids)
+    // per label and their block sums (dense ids; sub_val[0] and sub_key[0] then
+    // map ids to state indexes); ping-pong (key, value) arrays of the selected
+    // particles and the words of their radix sorts (other ids)
     uint32_t *sub_key[2], *sub_val[2];
     uint32_t *sub_os, *sub_cnt, *sub_bits, *sub_bsum;
     bool sub_clear = false;  // the bit maps are all 0

@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(256) k_sub_sums(const uint32_t* __restrict__ b
 
 // State indexes of the set bits in map order: sidx[rank of the bit] = by_id1[id]
 // in the map of label 1, by_id2[id] in that of label 2.  Leaves the maps clear.
-__global__ void __launch_bounds__(256) k_sub_list(uint32_t* bits, uint32_t m, uint32_t words, const uint32_t* __restrict__ bsum,
+__global__ void __launch_bounds__(256) k_sub_list(uint32_t* bits, uint32_t m, uint32_t words,
+                                                  const uint32_t* __restrict__ bsum,
                                                   const uint32_t* __restrict__ by_id1,
                                                   const uint32_t* __restrict__ by_id2,
                                                   uint32_t* __restrict__ sidx) {

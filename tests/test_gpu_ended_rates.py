@@ -45,3 +45,31 @@ def test_an_ended_member_after_a_run_that_went_non_finite():
         assert np.isfinite(st[key]).all(), key
     assert not np.array_equal(st["vel"][back][two], ens.vel[two])
     sim.close()
+
+
+def test_a_predictor_step_before_any_evaluation_takes_no_rates():
+    """In a workspace of NaNs, dt = 0 as no evaluation has set it."""
+    import torch
+    case = cases.random_block(500, seed=6, jitter=0.2)
+    P = S.make_params(case.params(), 0.0)
+    nbytes = int(S.sph_query_sizes(P, case.n).workspace_bytes)
+    ws = torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = S.sph_init(P, case.n, ws.data_ptr(), nbytes, stream.cuda_stream)
+    try:
+        S.sph_upload(ctx, np.ascontiguousarray(case.pos), np.ascontiguousarray(case.vel, np.float32),
+                     np.ascontiguousarray(case.rho, np.float32), np.ascontiguousarray(case.ids))
+        S.sph_build_cells(ctx)
+        S.sph_predict(ctx)
+        n = case.n
+        pos, vel = np.empty((n, 3)), np.empty((n, 3), np.float32)
+        rho, ids = np.empty(n, np.float32), np.empty(n, np.uint32)
+        S.sph_download(ctx, pos, vel, rho, ids)
+    finally:
+        stream.synchronize()
+        S.sph_destroy(ctx)
+    back = np.argsort(ids)
+    order = np.argsort(case.ids)
+    for got, want in ((pos, case.pos), (vel, case.vel), (rho, case.rho)):
+        assert np.array_equal(got[back], want[order])
